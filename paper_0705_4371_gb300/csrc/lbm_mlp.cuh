@@ -116,14 +116,70 @@ __device__ __forceinline__ void mlp_inputs(const MlpSmem& s, float f0, float f1,
     p23 = bf16_pack((f2 - s.mean[2]) * s.istd[2], (f3 - s.mean[3]) * s.istd[3]);
 }
 
+// Forward pass of one 16-row tile (rows r0 = g and r0 + 8 of the fragment
+// layout, g = lane / 4): a0, a1 the standardised inputs 2 tig, 2 tig + 1 of
+// the two rows (zero for tig >= 2).  yc: output 2 tig + j of row r0 in
+// register j, of row r0 + 8 in register 2 + j (lanes with tig < 2).  Every
+// lane of the warp must call it.  CAP: also store the hidden activations
+// (BF16 values, after ReLU) of the two rows at h1, h2 (rows of stride ld).
+template <bool CAP>
+__device__ __forceinline__ void mlp_tile_forward(const MlpSmem& s, unsigned a0, unsigned a1, float* yc,
+                                                 int r0 = 0, float* h1 = nullptr, float* h2 = nullptr, int ld = 0) {
+    const int lane = threadIdx.x & 31, tig = lane & 3, r1 = r0 + 8;
+    // layer 1; its n-tiles 2j, 2j+1 form k-step j of layer 2
+    unsigned A2[4][4];
+#pragma unroll
+    for (int nt = 0; nt < 8; nt++) {
+        const float bl = s.b1[8 * nt + 2 * tig], bh = s.b1[8 * nt + 2 * tig + 1];
+        float c[4] = {bl, bh, bl, bh};
+        mma_bf16(c, a0, a1, 0u, 0u, s.w1[nt][lane], 0u);
+        const unsigned u0 = bf16_pack_relu(c[0], c[1]), u1 = bf16_pack_relu(c[2], c[3]);
+        A2[nt >> 1][(nt & 1) * 2 + 0] = u0;
+        A2[nt >> 1][(nt & 1) * 2 + 1] = u1;
+        if constexpr (CAP) {
+            const int col = 8 * nt + 2 * tig;
+            h1[r0 * ld + col] = bf16_lo(u0);
+            h1[r0 * ld + col + 1] = bf16_hi(u0);
+            h1[r1 * ld + col] = bf16_lo(u1);
+            h1[r1 * ld + col + 1] = bf16_hi(u1);
+        }
+    }
+    // layers 2 and 3: each pair of layer-2 n-tiles is one layer-3 k-step
+    yc[0] = yc[2] = s.b3[2 * tig];
+    yc[1] = yc[3] = s.b3[2 * tig + 1];
+#pragma unroll
+    for (int jp = 0; jp < 4; jp++) {
+        unsigned A3[4];
+#pragma unroll
+        for (int hh = 0; hh < 2; hh++) {
+            const int nt = 2 * jp + hh;
+            const float bl = s.b2[8 * nt + 2 * tig], bh = s.b2[8 * nt + 2 * tig + 1];
+            float c[4] = {bl, bh, bl, bh};
+#pragma unroll
+            for (int j = 0; j < 4; j++) {
+                const uint2 b = s.w2[nt][j][lane];
+                mma_bf16(c, A2[j][0], A2[j][1], A2[j][2], A2[j][3], b.x, b.y);
+            }
+            const unsigned u0 = bf16_pack_relu(c[0], c[1]), u1 = bf16_pack_relu(c[2], c[3]);
+            A3[2 * hh] = u0;
+            A3[2 * hh + 1] = u1;
+            if constexpr (CAP) {
+                const int col = 8 * nt + 2 * tig;
+                h2[r0 * ld + col] = bf16_lo(u0);
+                h2[r0 * ld + col + 1] = bf16_hi(u0);
+                h2[r1 * ld + col] = bf16_lo(u1);
+                h2[r1 * ld + col + 1] = bf16_hi(u1);
+            }
+        }
+        const uint2 b = s.w3[jp][lane];
+        mma_bf16(yc, A3[0], A3[1], A3[2], A3[3], b.x, b.y);
+    }
+}
+
 // Forward pass of the network for the warp's 32 sites, lane l holding site
 // l: inputs (p01, p23) from mlp_inputs, outputs y[0..3].  Every lane of the
 // warp must call it (lanes without a site pass zeros and ignore y).
-// CAP: also store the hidden activations (BF16 values, after ReLU) of site
-// l at h1[l * ld + j], h2[l * ld + j] (training).
-template <bool CAP>
-__device__ __forceinline__ void mlp_warp_forward(const MlpSmem& s, unsigned p01, unsigned p23, float* y,
-                                                 float* h1 = nullptr, float* h2 = nullptr, int ld = 0) {
+__device__ __forceinline__ void mlp_warp_forward(const MlpSmem& s, unsigned p01, unsigned p23, float* y) {
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31, g = lane >> 2, tig = lane & 3;
 #pragma unroll
@@ -134,53 +190,8 @@ __device__ __forceinline__ void mlp_warp_forward(const MlpSmem& s, unsigned p01,
         const unsigned x1lo = __shfl_sync(FULL, p01, r1), x1hi = __shfl_sync(FULL, p23, r1);
         const unsigned a0 = tig == 0 ? x0lo : (tig == 1 ? x0hi : 0u);
         const unsigned a1 = tig == 0 ? x1lo : (tig == 1 ? x1hi : 0u);
-        // layer 1; its n-tiles 2j, 2j+1 form k-step j of layer 2
-        unsigned A2[4][4];
-#pragma unroll
-        for (int nt = 0; nt < 8; nt++) {
-            const float bl = s.b1[8 * nt + 2 * tig], bh = s.b1[8 * nt + 2 * tig + 1];
-            float c[4] = {bl, bh, bl, bh};
-            mma_bf16(c, a0, a1, 0u, 0u, s.w1[nt][lane], 0u);
-            const unsigned u0 = bf16_pack_relu(c[0], c[1]), u1 = bf16_pack_relu(c[2], c[3]);
-            A2[nt >> 1][(nt & 1) * 2 + 0] = u0;
-            A2[nt >> 1][(nt & 1) * 2 + 1] = u1;
-            if constexpr (CAP) {
-                const int col = 8 * nt + 2 * tig;
-                h1[r0 * ld + col] = bf16_lo(u0);
-                h1[r0 * ld + col + 1] = bf16_hi(u0);
-                h1[r1 * ld + col] = bf16_lo(u1);
-                h1[r1 * ld + col + 1] = bf16_hi(u1);
-            }
-        }
-        // layers 2 and 3: each pair of layer-2 n-tiles is one layer-3 k-step
-        float yc[4] = {s.b3[2 * tig], s.b3[2 * tig + 1], s.b3[2 * tig], s.b3[2 * tig + 1]};
-#pragma unroll
-        for (int jp = 0; jp < 4; jp++) {
-            unsigned A3[4];
-#pragma unroll
-            for (int hh = 0; hh < 2; hh++) {
-                const int nt = 2 * jp + hh;
-                const float bl = s.b2[8 * nt + 2 * tig], bh = s.b2[8 * nt + 2 * tig + 1];
-                float c[4] = {bl, bh, bl, bh};
-#pragma unroll
-                for (int j = 0; j < 4; j++) {
-                    const uint2 b = s.w2[nt][j][lane];
-                    mma_bf16(c, A2[j][0], A2[j][1], A2[j][2], A2[j][3], b.x, b.y);
-                }
-                const unsigned u0 = bf16_pack_relu(c[0], c[1]), u1 = bf16_pack_relu(c[2], c[3]);
-                A3[2 * hh] = u0;
-                A3[2 * hh + 1] = u1;
-                if constexpr (CAP) {
-                    const int col = 8 * nt + 2 * tig;
-                    h2[r0 * ld + col] = bf16_lo(u0);
-                    h2[r0 * ld + col + 1] = bf16_hi(u0);
-                    h2[r1 * ld + col] = bf16_lo(u1);
-                    h2[r1 * ld + col + 1] = bf16_hi(u1);
-                }
-            }
-            const uint2 b = s.w3[jp][lane];
-            mma_bf16(yc, A3[0], A3[1], A3[2], A3[3], b.x, b.y);
-        }
+        float yc[4];
+        mlp_tile_forward<false>(s, a0, a1, yc);
         // output j of tile row r sits in lane 4 (r mod 8) + j / 2, register
         // (j mod 2) (+2 for rows 8..15): bring it to lane 16 m + r
 #pragma unroll
@@ -204,7 +215,7 @@ __device__ __forceinline__ void mlp_warm_start(const MlpSmem& s, bool valid, flo
     unsigned p01 = 0u, p23 = 0u;
     if (valid) mlp_inputs(s, rho, ux, uy, th, p01, p23);
     float y[kMlpOut] = {0.0f, 0.0f, 0.0f, 0.0f};
-    mlp_warp_forward<false>(s, p01, p23, y);
+    mlp_warp_forward(s, p01, p23, y);
     a[0] = 3.0f * ux;
     a[1] = 3.0f * uy;
     a[2] = 0.0f;

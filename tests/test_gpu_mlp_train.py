@@ -1,0 +1,84 @@
+"""The training launch (every optimiser step in one cooperative kernel)
+against the gradient and Adam entry points called step by step, and the
+normalisation's sums, at the edges of the kernels' sample groups (32) and
+batches."""
+import numpy as np
+import pytest
+
+from tests._common import mlp_random_features, mlp_random_params
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def env():
+    import torch
+    from paper_0705_4371_gb300 import lbm
+    lbm.load()
+    assert torch.cuda.is_available()
+    return torch, lbm
+
+
+def _data(torch, seed, n):
+    from paper_0705_4371_gb300 import inputs
+    feat = torch.from_numpy(mlp_random_features(seed, n).astype(np.float32)).cuda()
+    dmu = torch.from_numpy((0.05 * inputs.uniform(seed + 7, (n, 4))).astype(np.float32)).cuda()
+    return feat, dmu
+
+
+@pytest.mark.parametrize("n, batch, epochs", [(1, 4, 2), (31, 31, 1), (33, 32, 2), (70, 33, 2), (300, 1000, 2),
+                                              (5000, 2048, 1), (9001, 4864, 1), (12000, 6001, 2)])
+def test_train_equals_gradient_and_adam_steps(env, n, batch, epochs):
+    # the two paths add the same FP32 products in different orders: gradients
+    # agree to about 1e-6 of their norm, so every Adam update (at most ~lr per
+    # entry) agrees to 1e-3 lr in the root mean square, all but gradients
+    # cancelled to a thousandth of their typical size following their sign
+    torch, lbm = env
+    feat, dmu = _data(torch, 500 + n, n)
+    p0 = torch.from_numpy(mlp_random_params(91).astype(np.float32)).cuda()
+    lr0, lr1 = 2e-3, 5e-4
+    a = p0.clone()
+    losses = torch.full((epochs,), -1.0, dtype=torch.float32, device="cuda")
+    lbm.mlp_train(a.data_ptr(), feat.data_ptr(), dmu.data_ptr(), n, batch, epochs, lr0, lr1, losses.data_ptr())
+    b, g = p0.clone(), torch.zeros_like(p0)
+    m, v = torch.zeros_like(p0), torch.zeros_like(p0)
+    loss = torch.zeros(1, dtype=torch.float32, device="cuda")
+    nb = -(-n // batch)
+    t, want = 0, []
+    for _ in range(epochs):
+        mean = 0.0
+        for k in range(nb):
+            i0, nn = k * batch, min(batch, n - k * batch)
+            lr = lr0 * (lr1 / lr0) ** (t / (nb * epochs - 1) if nb * epochs > 1 else 0.0)
+            t += 1
+            lbm.mlp_grad(b.data_ptr(), feat[i0:].data_ptr(), dmu[i0:].data_ptr(), nn, g.data_ptr(), loss.data_ptr())
+            lbm.mlp_adam(b.data_ptr(), g.data_ptr(), m.data_ptr(), v.data_ptr(), t, lr)
+            mean += float(loss.item()) / nb
+        want.append(mean)
+    torch.cuda.synchronize()
+    d = (a - b).double()
+    assert torch.isfinite(a).all()
+    assert float(d.square().mean().sqrt()) <= 1e-3 * lr0 * t
+    assert not d[-12:].any()                      # the normalisation entries are not trained
+    assert np.allclose(losses.cpu().numpy(), want, rtol=1e-4)
+
+
+@pytest.mark.parametrize("n", [1, 255, 257, 100_003, 400_000])
+def test_normalise_matches_fp64_sums(env, n):
+    torch, lbm = env
+    feat, dmu = _data(torch, 900 + n, n)
+    p = torch.zeros(lbm.mlp_param_count(), dtype=torch.float32, device="cuda")
+    lbm.mlp_normalise(p.data_ptr(), feat.data_ptr(), dmu.data_ptr(), n)
+    torch.cuda.synchronize()
+    f, d = feat.double(), dmu.double()
+    mean = f.mean(0)
+    var = (f * f).mean(0) - mean * mean
+    istd = torch.where(var > 0, 1 / var.clamp_min(1e-300).sqrt(), torch.ones_like(var))
+    want = torch.cat([mean, istd, (d * d).mean(0).sqrt()]).cpu().numpy()
+    got = p[-12:].cpu().numpy().astype(np.float64)
+    # FP64 sums of n terms in another order, then one FP32 rounding; the
+    # variance is a difference of two sums (about 1e3 times smaller here)
+    if n > 1:
+        assert np.allclose(got, want, rtol=1.5e-7)
+    else:
+        assert np.allclose(got[[0, 1, 2, 3, 8, 9, 10, 11]], want[[0, 1, 2, 3, 8, 9, 10, 11]], rtol=1.5e-7)
