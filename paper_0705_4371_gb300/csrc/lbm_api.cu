@@ -55,12 +55,12 @@ constexpr int kDefaultLog = 65536;
 // latency) run faster register-fed (shape 1): the 600 x 500 channel 15.7 k
 // against 13.0 k MLUPS, 1024 x 512 23.2 k against 22.2 k; from 1536 x 768
 // on shape 5 is ahead (34.3 k against 31.1 k), and FP16 storage is fastest
-// on shape 5 at every size measured.  The energy forms are bound by the Newton solve, not
-// by memory: FP64 storage's FP64 finish wants the most resident warps
-// (register-fed shape 1); the float-float finish of FP32 / FP16 storage and
-// the network's warm start run best in the staged shape 4 (measured at
-// 2048 x 1024: Newton start 0.22 ms per step against 0.44 on shape 0 and 0.24
-// on shape 5; warm start 0.35 against 0.54 and 0.35).
+// on shape 5 at every size measured.  The energy forms: FP64 storage's FP64
+// solve wants the most resident warps (register-fed shape 1); the
+// float-float solve of FP32 / FP16 storage and the network's warm start run
+// best in the staged shape 4 (measured at 2048 x 1024: Newton start 89 us
+// per step against 235 on shape 0 and 93 on shape 5; warm start 211 against
+// 263 and 233).
 int default_tile_shape(int lattice, int eq, int precision, long long sites) {
     if (lattice != LB_D2Q9) return 0;
     if (eq < LB_EQ_ENTROPIC_ENERGY) {

@@ -38,39 +38,19 @@ __device__ __forceinline__ void equilibrium(const Params& P, T drho, T rho, T ux
 // moments (drho, j, 2E); Newton from the start point a0 (the network's
 // warm start in the learned form) or, when a0 is null, from the polynomial
 // start point (3 u_x, 3 u_y, 0) (the multipliers of the first-order
-// expansion about rest).
+// expansion about rest).  The momentum multipliers are eliminated in closed
+// form, so only the energy multiplier's start enters the iteration.
 template <typename T, int EQ>
-__device__ __forceinline__ void equilibrium_energy(const Params& P, T rho, T jx, T jy, T e2, T* gs,
-                                                   NewtonCount& nc, const float* a0 = nullptr) {
+__device__ __forceinline__ void equilibrium_energy(T rho, T jx, T jy, T e2, T* gs, NewtonCount& nc,
+                                                   const float* a0 = nullptr) {
+    const float mu3 = a0 ? a0[2] : 0.0f;
     if constexpr (sizeof(T) == 4) {
         // FP32 / FP16 storage: the float-float finish (no FP64 work)
-        float a[3];
-        if (a0) {
-            a[0] = a0[0];
-            a[1] = a0[1];
-            a[2] = a0[2];
-        } else {
-            const float ir = __frcp_rn(rho);
-            a[0] = 3.0f * (jx * ir);
-            a[1] = 3.0f * (jy * ir);
-            a[2] = 0.0f;
-        }
-        energy_solve_ff(rho, jx, jy, e2, Par<T>::rho0(P), a, gs, nc);
+        energy_solve_ff(rho, jx, jy, e2, mu3, gs, nc);
     } else {
-        // FP64 storage: FP64 finish to 4e-15 (the FP64 parity bound)
-        const double r = (double)rho, ir = recip64(r);
-        const double ux = (double)jx * ir, uy = (double)jy * ir;
-        float a[3] = {3.0f * (float)ux, 3.0f * (float)uy, 0.0f};
-        if (a0) {
-            a[0] = a0[0];
-            a[1] = a0[1];
-            a[2] = a0[2];
-        }
-        double fs[9];
-        energy_solve(r, ux, uy, (double)e2 * ir, a, fs, nc, 4e-15);
-        const double rho0 = P.rho0;
-#pragma unroll
-        for (int i = 0; i < 9; i++) gs[i] = (T)(fs[i] - D2Q9::w(i) * rho0);
+        // FP64 storage (rho0 = 0): FP64 finish to 4e-15 (the FP64 parity bound)
+        const double ir = recip64(rho);
+        energy_solve(rho, jx * ir, jy * ir, e2 * ir, mu3, gs, nc, 4e-15f);
     }
 }
 
@@ -126,7 +106,7 @@ __device__ __forceinline__ void site_equilibrium(const Params& P, const T* g, T*
     velocity<T>(jx, jy, rho, ux, uy);
     if constexpr (EQ >= EQ_ENERGY) {
         const T e2 = energy_moment<L, T>(g, Par<T>::rho0(P));
-        equilibrium_energy<T, EQ>(P, rho, jx, jy, e2, gs, nc, a0);
+        equilibrium_energy<T, EQ>(rho, jx, jy, e2, gs, nc, a0);
     } else {
         (void)nc;
         (void)a0;
@@ -166,10 +146,9 @@ __device__ __noinline__ double delta_s_fp64(PopArr<L::Q, T> g, double rho0) {
         double e2 = L::sum_w_c2 * rho0;
 #pragma unroll
         for (int i = 0; i < L::Q; i++) e2 += (double)(L::cx(i) * L::cx(i) + L::cy(i) * L::cy(i)) * gd[i];
-        float a[3] = {3.0f * (float)ux, 3.0f * (float)uy, 0.0f};
         double fs[9];
         NewtonCount nc = {0, 0, 0, 0};
-        energy_solve(rho, ux, uy, e2 / rho, a, fs, nc, 4e-15);
+        energy_solve(rho, ux, uy, e2 / rho, 0.0f, fs, nc, 4e-15f);
 #pragma unroll
         for (int i = 0; i < L::Q; i++) gs[i] = fs[i] - L::w(i) * rho0;
     } else if constexpr (EQ == EQ_POLY) {
@@ -1839,7 +1818,7 @@ __global__ void k_init_eq(const __grid_constant__ Params P, const double* rho, c
             if (e2) {
                 const T r = T(rho[sid]), u = T(ux[sid]);
                 NewtonCount nc = {0, 0, 0, 0};
-                equilibrium_energy<T, EQ>(P, r, r * u, r * T(v), T(e2[sid]), gs, nc);
+                equilibrium_energy<T, EQ>(r, r * u, r * T(v), T(e2[sid]), gs, nc);
 #pragma unroll
                 for (int i = 0; i < L::Q; i++) gs[i] = store_round<L, S>(i, gs[i]);
                 done = true;

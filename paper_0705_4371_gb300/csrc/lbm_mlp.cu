@@ -78,18 +78,15 @@ __global__ void __launch_bounds__(256) k_energy_dataset(const double* __restrict
     NewtonCount nc = {0, 0, 0, 0};
     if (i < n) {
         const double r = rho[i], u = ux[i], v = uy[i];
-        double fi[9];
-        feq_entropic<D2Q9, double>(r, u, v, 0.0, fi);
-        double e2iso = 0.0;
-#pragma unroll
-        for (int j = 0; j < 9; j++) e2iso += (double)(D2Q9::cx(j) * D2Q9::cx(j) + D2Q9::cy(j) * D2Q9::cy(j)) * fi[j];
-        const double e2 = escale[i] * e2iso;
-        float a[3] = {3.0f * (float)u, 3.0f * (float)v, 0.0f};
-        double fs[9], a64[3];
-        energy_solve(r, u, v, e2 / r, a, fs, nc, 4e-15, a64);
-        const double m[4] = {log(fs[0] / D2Q9::w(0)), a64[0], a64[1], a64[2]};
+        // second moment of the isothermal product form (Sec. 4.2) per axis:
+        // (2 sqrt(1 + 3 u^2) - 1) / 3
+        const double sx = sqrt(fma(3.0 * u, u, 1.0)), sy = sqrt(fma(3.0 * v, v, 1.0));
+        const double th = escale[i] * (2.0 / 3.0) * (sx + sy - 1.0);
+        double fs[9], mu3[3];
+        energy_solve(r, u, v, th, 0.0f, fs, nc, 4e-15f, mu3);
+        const double m[4] = {log(fs[0] / D2Q9::w(0)), mu3[0], mu3[1], mu3[2]};
         const double m0[4] = {log(r) - 1.5 * (u * u + v * v), 3.0 * u, 3.0 * v, 0.0};
-        const double f[4] = {r, u, v, e2 / r - u * u - v * v};
+        const double f[4] = {r, u, v, th - u * u - v * v};
 #pragma unroll
         for (int j = 0; j < 4; j++) {
             feat[i * 4 + j] = (float)f[j];

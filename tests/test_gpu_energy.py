@@ -143,3 +143,45 @@ def test_energy_tile_shapes_give_identical_results(lbm, prec):
         assert np.array_equal(states[0][0], states[shape][0]), shape
         assert np.array_equal(states[0][1], states[shape][1]), shape
     assert states[0][1].sum() > 0
+
+
+@pytest.mark.parametrize("umax, lo, hi", [(0.02, 0.99, 1.01), (0.2, 0.9, 1.1), (0.35, 0.8, 1.3), (0.0, 0.7, 1.5)])
+def test_energy_solve_over_its_range(lbm, umax, lo, hi):
+    # the scalar form of the solve (one energy multiplier, then a cubic in the
+    # difference of the axes' second moments) against the oracle's Newton on
+    # all multipliers: equal axes (D = 0), rest, fast and hot or cold sites
+    w = energy_cylinder(nx=40, ny=24, L=4)
+    cfg = oracle_cfg(w)
+    shape = (w.ny, w.nx)
+    rho = inputs.uniform(31, shape, 0.5, 2.0)
+    ux, uy = inputs.uniform(32, shape, -umax, umax), inputs.uniform(33, shape, -umax, umax)
+    ux[::3] = uy[::3]
+    ux[1::6] = -uy[1::6]
+    iso = (2 * np.sqrt(1 + 3 * ux * ux) + 2 * np.sqrt(1 + 3 * uy * uy) - 2) / 3
+    e2 = rho * iso * inputs.uniform(34, shape, lo, hi)
+    fo = ora.init_field(cfg, rho, ux, uy, e2)
+    for prec, tol in (("f64", 1e-12), ("f32dev", 2e-6)):
+        g = lbm.Lattice.from_workload(w, precision=lbm.PRECISIONS[prec])
+        g.init_equilibrium(rho, ux, uy, e2)
+        assert rel_err(g.get_state(), fo) < tol, prec
+        g.step(1)                       # the same solve inside the collision
+        g.sync()
+        assert g.newton_stats()[3] == 0
+        g.close()
+
+
+def test_energy_solve_reports_moments_without_a_solution(lbm):
+    # 2E below |rho u| has no positive f*: the sticky Newton error
+    w = energy_cylinder(nx=40, ny=24, L=4)
+    cfg = oracle_cfg(w)
+    f = ora.init_field(cfg, *inputs.cylinder_fields(w, noise=1e-3))
+    f[:, 6, 10] = 0.0
+    f[1, 6, 10], f[3, 6, 10] = 1.3, -0.3
+    f[0, 6, 10] = 0.4
+    g = lbm.Lattice.from_workload(w, precision=lbm.LB_F32_DEV)
+    g.set_state(f)
+    with pytest.raises(lbm.LBError) as e:
+        g.step(1)
+        g.sync()
+    assert e.value.code in (lbm.LB_ERR_NEWTON, lbm.LB_ERR_NONFINITE)
+    g.close()
