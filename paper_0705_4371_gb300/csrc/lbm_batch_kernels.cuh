@@ -149,13 +149,11 @@ __global__ void __launch_bounds__(32 * R, 16 / R) k_collide_batch(const __grid_c
         const int tiles_x = (P.nx + TX - 1) / TX;
         const int ty = lt / tiles_x, tx = lt - ty * tiles_x;
         const long long t = __ldcg(P.step);
-        bool nonfinite = false;
-        NewtonCount nc = {0, 0, 0, 0};
-        const S* box = stages + (size_t)st * (LY::STAGE_BYTES / sizeof(S));
-        GlobalCandSink sink;
-        if (lt <= -2) edge_item<S, EQ, R>(P, -2 - lt, t, sink, mslot, nonfinite, nc);
-        else tma_tile<S, EQ, R, kTmaTX, true>(P, box, tx * TX, ty * R, t, sink, mslot, nonfinite, nc, P);
-        if (nonfinite) atomicOr(P.err, ERR_NONFINITE);
+        S* box = stages + (size_t)st * (LY::STAGE_BYTES / sizeof(S));
+        TileState<GlobalCandSink> state{{}, {0, 0, 0, 0}, false};
+        if (lt <= -2) state = edge_item<S, EQ, R>(P, -2 - lt, t, state, mslot);
+        else tma_tile<S, EQ, R, kTmaTX>(P, box, tx * TX, ty * R, t, state, mslot, P);
+        if (state.nonfinite) atomicOr(P.err, ERR_NONFINITE);
     }
     __syncthreads();
     if (sh.abort && threadIdx.x == 0) {

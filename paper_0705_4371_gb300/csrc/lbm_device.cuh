@@ -492,7 +492,8 @@ __device__ __forceinline__ unsigned long long ds_key(double d) {
 // Free flight with boundary rules (Sec. 3 map Theta_tau; Sec. 4.2).
 // Pre-collision deviation populations at fluid site (x, y) from the
 // post-collision field src.  Rules where x - v_i leaves the fluid:
-//   x side: PERIODIC wraps, INLET = f*(rho_in, u_in), OUTLET = f*(rho, u of
+//   x side: PERIODIC wraps, INLET = f*(rho_in, u_in) (computed once in FP64 by
+//           the host, Params::gin), OUTLET = f*(rho, u of
 //           column nx-2 in the same row), BB = own opposite population;
 //   y side: PERIODIC wraps, FREESLIP = population (v_x, -v_y) of (x - v_x, y),
 //           BB = own opposite population;
@@ -552,81 +553,69 @@ __device__ __forceinline__ void outlet_equilibrium(const Params& P, const T* v, 
     feq_rho_u<L, T>(P.eq, rho, jx / rho, jy / rho, rho0, g);
 }
 
-// Inlet rule of Sec. 4.2: the quasiequilibrium of the free stream, computed
-// once in FP64 by the host (Params::gin).
-template <typename L, typename T>
-__device__ __forceinline__ void inlet_equilibrium(const Params& P, T* g) {
-#pragma unroll
-    for (int i = 0; i < L::Q; i++) g[i] = (T)P.gin[i];
-}
-
+// Sites whose nine sources lie in the fluid (almost all) load them at once.
+// The others resolve every population to one load (plane, column, row) by
+// selects and load them together too: the rules cost their instructions, not
+// a chain of dependent branches and loads.
 template <typename L, typename S>
 __device__ void gather_site(const Params& P, int x, int y, typename Store<S>::T* g) {
     using T = typename Store<S>::T;
     const long long s0 = (long long)y * P.nxp + x;
-    if (P.prestream) {
+    const bool inside = x >= 1 && x <= P.nx - 2 && (L::Q == 3 || (y >= 1 && y <= P.ny - 2));
+    const bool near = P.ow > 0 && x >= P.ox0 - 1 && x <= P.ox0 + P.ow && y >= P.oy0 - 1 && y <= P.oy0 + P.oh;
+    if (P.prestream || (inside && !near)) {
+        const long long shift = P.prestream ? 0 : 1;
 #pragma unroll
-        for (int i = 0; i < L::Q; i++) g[i] = Store<S>::load(P.src, i * P.plane + s0);
+        for (int i = 0; i < L::Q; i++)
+            g[i] = Store<S>::load(P.src, i * P.plane + s0 - shift * (L::cy(i) * (long long)P.nxp + L::cx(i)));
         return;
     }
-    bool have_in = false, have_out = false;
-    unsigned wall_mask = 0u;
-    T gin[L::Q], gout[L::Q];
+    unsigned wall_mask = 0u, in_mask = 0u, out_mask = 0u;
 #pragma unroll
     for (int i = 0; i < L::Q; i++) {
         const int cx = L::cx(i), cy = L::cy(i);
+        // source (sx, sy) of plane i; done: the rule is settled
         int sx = x - cx, sy = y - cy;
-        if (sx < 0 || sx >= P.nx) {
+        bool own = false, mirror = false, done = false;   // own opposite population; population (v_x, -v_y)
+        if (cx != 0 && (sx < 0 || sx >= P.nx)) {
             const int kind = sx < 0 ? P.bc[0] : P.bc[1];
-            if (kind == BC_PERIODIC) {
-                sx = sx < 0 ? sx + P.nx : sx - P.nx;
-            } else if (kind == BC_INLET) {
-                if (!have_in) {
-                    inlet_equilibrium<L, T>(P, gin);
-                    have_in = true;
-                }
-                g[i] = gin[i];
-                continue;
-            } else if (kind == BC_OUTLET) {
-                if (!have_out) {
-                    const long long sp = (long long)y * P.nxp + (P.nx - 2);
-                    T v[L::Q];
-#pragma unroll
-                    for (int j = 0; j < L::Q; j++) v[j] = Store<S>::load(P.src, j * P.plane + sp);
-                    outlet_equilibrium<L, T>(P, v, gout);
-#pragma unroll
-                    for (int j = 0; j < L::Q; j++) gout[j] = store_round<L, S>(j, gout[j]);
-                    have_out = true;
-                }
-                g[i] = gout[i];
-                continue;
-            } else if (kind == BC_OUTLET_COPY) {
-                // zero-gradient outflow: the column beyond the side is a copy
-                // of the side column; the y and obstacle rules then apply
-                sx = x;
-            } else {
-                g[i] = Store<S>::load(P.src, L::opp(i) * P.plane + s0);
-                continue;
-            }
+            if (kind == BC_INLET) in_mask |= 1u << i;
+            if (kind == BC_OUTLET) out_mask |= 1u << i;
+            own = kind != BC_PERIODIC && kind != BC_OUTLET_COPY;   // (inlet, outlet: replaced below)
+            done = own;
+            // zero-gradient outflow: the column beyond the side is a copy
+            // of the side column; the y and obstacle rules then apply
+            sx = kind == BC_PERIODIC ? (sx < 0 ? sx + P.nx : sx - P.nx) : x;
         }
-        if (sy < 0 || sy >= P.ny) {
+        if (cy != 0 && !done && (sy < 0 || sy >= P.ny)) {
             const int kind = sy < 0 ? P.bc[2] : P.bc[3];
-            if (kind == BC_PERIODIC) {
-                sy = sy < 0 ? sy + P.ny : sy - P.ny;
-            } else if (kind == BC_FREESLIP) {
-                g[i] = Store<S>::load(P.src, L::mir_y(i) * P.plane + (long long)y * P.nxp + sx);
-                continue;
-            } else {
-                g[i] = Store<S>::load(P.src, L::opp(i) * P.plane + s0);
-                continue;
-            }
+            done = kind != BC_PERIODIC;
+            mirror = kind == BC_FREESLIP;
+            own = done && !mirror;
+            sy = kind == BC_PERIODIC ? (sy < 0 ? sy + P.ny : sy - P.ny) : y;
         }
-        if (is_solid(P, sx, sy)) {
-            g[i] = Store<S>::load(P.src, L::opp(i) * P.plane + s0);
+        if (i > 0 && !done && is_solid(P, sx, sy)) {
+            own = true;
             if (P.wall == WALL_DIFFUSE) wall_mask |= 1u << i;
-            continue;
         }
-        g[i] = Store<S>::load(P.src, i * P.plane + (long long)sy * P.nxp + sx);
+        const int plane = own ? L::opp(i) : (mirror ? L::mir_y(i) : i);
+        const long long at = own ? s0 : (long long)sy * P.nxp + sx;
+        g[i] = Store<S>::load(P.src, plane * P.plane + at);
+    }
+    if (out_mask) {
+        T v[L::Q], gout[L::Q];
+        const long long sp = (long long)y * P.nxp + (P.nx - 2);
+#pragma unroll
+        for (int j = 0; j < L::Q; j++) v[j] = Store<S>::load(P.src, j * P.plane + sp);
+        outlet_equilibrium<L, T>(P, v, gout);
+#pragma unroll
+        for (int i = 0; i < L::Q; i++)
+            if ((out_mask >> i) & 1u) g[i] = store_round<L, S>(i, gout[i]);
+    }
+    if (in_mask) {
+#pragma unroll
+        for (int i = 0; i < L::Q; i++)
+            if ((in_mask >> i) & 1u) g[i] = (T)P.gin[i];
     }
     if (wall_mask) diffuse_wall<L, T>(wall_mask, g);
 }

@@ -565,6 +565,8 @@ __device__ __forceinline__ void block_room(const Params& P, BlockCandT<CAP>& bc,
 // What the block contributes to the global select: its k best (all threads).
 template <int CAP>
 __device__ __forceinline__ void block_finish(const Params& P, BlockCandT<CAP>& bc, TopkScratch& sc) {
+    __syncthreads();
+    if (bc.n == 0) return;   // uniform: almost every block
     if (P.k > 0) block_cut(bc, sc, P.k);
     block_flush(P, bc);
 }
@@ -583,10 +585,43 @@ __device__ __forceinline__ void block_finish(const Params& P, BlockCandT<CAP>& b
 // ---------------------------------------------------------------------------
 struct SelectShared {
     TopkScratch sc;
-    int nsel;
     unsigned cnt;
 };
 
+// The Ehrenfests' step at one site, whose post-collision populations g are
+// at hand: the collision conserves every moment f* depends on, so this is f*
+// of the pre-collision state.
+template <typename L, typename S, int EQ>
+__device__ __forceinline__ void ehrenfest_site(const Params& P, long long o, const typename Store<S>::T* g) {
+    using T = typename Store<S>::T;
+    T gs[L::Q], rho, ux, uy;
+    site_equilibrium<L, T, EQ>(P, g, gs, rho, ux, uy);
+    if constexpr (Store<S>::kProject) {
+        // f' = f* = f - (f - f*), with the conserved moments of
+        // f - f* freed of rounding as in the collision
+        T d[L::Q];
+#pragma unroll
+        for (int i = 0; i < L::Q; i++) d[i] = g[i] - gs[i];
+        conserve_neq<L, EQ>(d);
+#pragma unroll
+        for (int i = 0; i < L::Q; i++) gs[i] = g[i] - d[i];
+    }
+#pragma unroll
+    for (int i = 0; i < L::Q; i++) Store<S>::store(P.dst, i * P.plane + o, store_round<L, S>(i, gs[i]));
+}
+
+constexpr int kRankMax = 256;   // candidates ranked by counting, one per thread
+
+// What bounds this: one block runs it while the rest of the GPU is done, a
+// chain of dependent loads.  Up to kRankMax candidates (and no more than the
+// block has threads) go one per thread: a candidate's rank is the number of
+// candidates before it in the selection's total order, counted in shared
+// memory, its site's populations are fetched meanwhile, and the threads of
+// rank below k perform the Ehrenfests' step at once -- one load after
+// another: count, candidate, populations.  The radix select that larger sets
+// take costs several block barriers and passes and puts its result in global
+// memory first: from the ticket to the last store 6 us against 4 us on the
+// 4096 x 2048 cylinder.
 template <typename L, typename S, int EQ>
 __device__ __noinline__ void select_and_fix(const Params& P, SelectShared& ss,
                                             unsigned long long* stage_key, unsigned* stage_idx,
@@ -600,24 +635,54 @@ __device__ __noinline__ void select_and_fix(const Params& P, SelectShared& ss,
         r = t - P.replay_t0;
         replay = r >= 0 && r < P.replay_n;
     }
-    int mine = -1;   // the site this thread selected itself, when it did (j = tid)
-    if (replay) {
-        const int c = P.replay_cnt[r];
-        const long long off = P.replay_off[r];
-        for (int j = tid; j < c; j += nt) P.sel_idx[j] = P.replay_idx[off + j];
-        if (tid == 0) ss.nsel = c;
-    } else if (P.k <= 0) {
-        if (tid == 0) ss.nsel = 0;
+    const int n = P.k > 0 && !replay ? (int)__ldcg(P.cand_count) : 0;
+    int m;   // sites selected
+    if (!replay && n <= min(min(nt, kRankMax), stage_cap)) {
+        unsigned long long key = 0ull;
+        unsigned id = 0u;
+        T g[L::Q];
+        long long o = 0;
+        if (tid < n) {
+            id = __ldcg(P.cand_idx + tid);
+            key = __ldcg(P.cand_key + tid);
+            stage_key[tid] = key;
+            stage_idx[tid] = id;
+            if (mode == 0) {
+                o = (long long)(id / (unsigned)P.nx) * P.nxp + id % (unsigned)P.nx;
+#pragma unroll
+                for (int i = 0; i < L::Q; i++) g[i] = Store<S>::load(P.dst, i * P.plane + o);
+            }
+        }
+        __syncthreads();
+        if (tid < n) {
+            int rank = tid;
+            if (n > P.k) {
+                rank = 0;
+#pragma unroll 8
+                for (int e = 0; e < n; e++) {
+                    const unsigned long long ke = stage_key[e];
+                    rank += ke > key || (ke == key && stage_idx[e] < id);
+                }
+            }
+            if (rank < P.k) {
+                P.sel_idx[rank] = (int)id;
+                if (P.sel_key) P.sel_key[rank] = key;
+                if (mode == 0) ehrenfest_site<L, S, EQ>(P, o, g);
+            }
+        }
+        m = min(n, P.k);
     } else {
-        const int n = (int)__ldcg(P.cand_count);
-        if (n <= P.k) {
+        if (replay) {
+            const int c = P.replay_cnt[r];
+            const long long off = P.replay_off[r];
+            for (int j = tid; j < c; j += nt) P.sel_idx[j] = P.replay_idx[off + j];
+            m = c;
+        } else if (n <= P.k) {
             for (int j = tid; j < n; j += nt) {
-                const int id = (int)__ldcg(P.cand_idx + j);
-                P.sel_idx[j] = id;
-                if (j == tid) mine = id;
+                P.sel_idx[j] = (int)__ldcg(P.cand_idx + j);
                 if (P.sel_key) P.sel_key[j] = __ldcg(P.cand_key + j);
             }
-            if (tid == 0) ss.nsel = n;
+            m = n;
         } else {
             const bool staged = n <= stage_cap;
             if (staged) {
@@ -643,45 +708,27 @@ __device__ __noinline__ void select_and_fix(const Params& P, SelectShared& ss,
                     }
                 }
             }
-            if (tid == 0) ss.nsel = P.k;
+            m = P.k;
         }
-    }
-    __syncthreads();
-    const int m = ss.nsel;
-    if (mode == 0) {
-        const long long nsites = (long long)P.nx * P.ny;
-        for (int j = tid; j < m; j += nt) {
-            const int site = j == tid && mine >= 0 ? mine : P.sel_idx[j];
-            if (site < 0 || site >= nsites) { atomicOr(P.err, ERR_REPLAY); continue; }
-            const int x = site % P.nx, y = site / P.nx;
-            if (is_solid(P, x, y)) { atomicOr(P.err, ERR_REPLAY); continue; }
-            const long long o = (long long)y * P.nxp + x;
-            // f* of the site from its post-collision populations: the
-            // collision conserves every moment f* depends on, so this is f*
-            // of the pre-collision state, read at the site itself (nine
-            // independent loads, no boundary rules: the block that runs this
-            // is alone on the device by then, and its code path stays short)
-            T g[L::Q], gs[L::Q], rho, ux, uy;
+        __syncthreads();
+        if (mode == 0) {
+            const long long nsites = (long long)P.nx * P.ny;
+            for (int j = tid; j < m; j += nt) {
+                const int site = P.sel_idx[j];
+                if (site < 0 || site >= nsites) { atomicOr(P.err, ERR_REPLAY); continue; }
+                const int x = site % P.nx, y = site / P.nx;
+                if (is_solid(P, x, y)) { atomicOr(P.err, ERR_REPLAY); continue; }
+                const long long o = (long long)y * P.nxp + x;
+                T g[L::Q];
 #pragma unroll
-            for (int i = 0; i < L::Q; i++) g[i] = Store<S>::load(P.dst, i * P.plane + o);
-            site_equilibrium<L, T, EQ>(P, g, gs, rho, ux, uy);
-            if constexpr (Store<S>::kProject) {
-                // f' = f* = f - (f - f*), with the conserved moments of
-                // f - f* freed of rounding as in the collision
-                T d[L::Q];
-#pragma unroll
-                for (int i = 0; i < L::Q; i++) d[i] = g[i] - gs[i];
-                conserve_neq<L, EQ>(d);
-#pragma unroll
-                for (int i = 0; i < L::Q; i++) gs[i] = g[i] - d[i];
+                for (int i = 0; i < L::Q; i++) g[i] = Store<S>::load(P.dst, i * P.plane + o);
+                ehrenfest_site<L, S, EQ>(P, o, g);
             }
-#pragma unroll
-            for (int i = 0; i < L::Q; i++)
-                Store<S>::store(P.dst, i * P.plane + o, store_round<L, S>(i, gs[i]));
         }
+        __syncthreads();
     }
-    __syncthreads();
     if (tid == 0) {
+        // (every thread has read the count: the barriers above)
         *P.sel_count = m;
         *P.cand_count = 0;
         if (mode == 0) {
@@ -1248,6 +1295,15 @@ struct GlobalCandSink {
     }
 };
 
+// What a warp carries from tile to tile; passed to and returned from the
+// out-of-line paths by value, so that it stays in registers.
+template <typename Sink>
+struct TileState {
+    Sink sink;
+    NewtonCount nc;
+    bool nonfinite;
+};
+
 // Pre-collision deviations of site (x, y) of a staged tile: the same rules
 // as gather_site (free flight, Sec. 4.2 boundaries).  Plane j's window holds
 // source rows y0 - v_jy .. y0 - v_jy + R - 1 (box[j][row][col] with
@@ -1272,9 +1328,9 @@ __device__ __forceinline__ void gather_site_smem(const Params& P, const S* box, 
         for (int i = 0; i < L::Q; i++) g[i] = at(i, x, y);
         return;
     }
-    bool have_in = false, have_out = false;
+    bool have_out = false;
     unsigned wall_mask = 0u;
-    T gin[L::Q], gout[L::Q];
+    T gout[L::Q];
 #pragma unroll
     for (int i = 0; i < L::Q; i++) {
         const int cx = L::cx(i), cy = L::cy(i);
@@ -1285,11 +1341,7 @@ __device__ __forceinline__ void gather_site_smem(const Params& P, const S* box, 
             if (kind == BC_OUTLET_COPY) {
                 sx = x;   // the column beyond the side is a copy of the side column
             } else if (kind == BC_INLET) {
-                if (!have_in) {
-                    inlet_equilibrium<L, T>(P, gin);
-                    have_in = true;
-                }
-                g[i] = gin[i];
+                g[i] = (T)P.gin[i];
             } else if (kind == BC_OUTLET) {
                 if (!have_out) {
                     T v[L::Q];
@@ -1321,13 +1373,13 @@ __device__ __forceinline__ void gather_site_smem(const Params& P, const S* box, 
     if (wall_mask) diffuse_wall<L, T>(wall_mask, g);
 }
 
-// The sites of a staged tile that touches a boundary, the obstacle or the
-// probe site, one by one with the boundary rules (kept out of line so that
-// the interior path is allocated registers on its own).
-template <typename S, int EQ, int R, int TX, bool SPLIT, typename Sink>
-__device__ __noinline__ void tma_tile_general(const Params& P, const S* box, int x0, int y0, long long t,
-                                              Sink& sink, MlpSlot<EQ>& mslot,
-                                              bool& nonfinite, NewtonCount& nc, bool clean) {
+// The sites of a staged row next to a diffuse wall in FP16 storage, one by
+// one with the boundary rules: the wall's populations are FP32 values that a
+// staged FP16 row cannot hold (patch_row serves every other case).  Out of
+// line, so that the interior path is allocated registers on its own.
+template <typename S, int EQ, int R, int TX, typename Sink>
+__device__ __noinline__ TileState<Sink> tma_tile_general(const Params& P, const S* box, int x0, int y0, long long t,
+                                                         TileState<Sink> state, MlpSlot<EQ>& mslot) {
     using L = D2Q9;
     using T = typename Store<S>::T;
     using LY = TmaLayout<S, R, TX>;
@@ -1343,19 +1395,16 @@ __device__ __noinline__ void tma_tile_general(const Params& P, const S* box, int
         T ds = T(-1);
         // the learned form enters with every lane (its warm start is a
         // warp-wide evaluation); lanes outside the grid then carry no site
-        // SPLIT: the columns x = 0 and x = nx - 1 are updated apart (edge_item)
-        const bool mine = x < P.nx && y < P.ny && !(SPLIT && (x == 0 || x == P.nx - 1));
+        // the columns x = 0 and x = nx - 1 are updated apart (edge_item)
+        const bool mine = x < P.nx && y < P.ny && !(x == 0 || x == P.nx - 1);
         if (EQ == EQ_ENERGY_MLP || mine) {
             const bool inside = mine;
             const int c = x - x0;
             const int o = y * nxp + x;
-            bool shift = clean;
-            if (!shift) {
-                const bool near_obstacle = P.ow > 0 && x >= P.ox0 - 1 && x <= P.ox0 + P.ow &&
-                                           y >= P.oy0 - 1 && y <= P.oy0 + P.oh;
-                shift = !P.prestream && x >= 1 && x <= P.nx - 2 && y >= 1 && y <= P.ny - 2 &&
-                        !near_obstacle;
-            }
+            const bool near_obstacle = P.ow > 0 && x >= P.ox0 - 1 && x <= P.ox0 + P.ow &&
+                                       y >= P.oy0 - 1 && y <= P.oy0 + P.oh;
+            const bool shift = !P.prestream && x >= 1 && x <= P.nx - 2 && y >= 1 && y <= P.ny - 2 &&
+                               !near_obstacle;
             T g[L::Q];
             bool fluid = inside;
             if (!inside) {
@@ -1378,11 +1427,12 @@ __device__ __noinline__ void tma_tile_general(const Params& P, const S* box, int
                 __syncwarp();
                 mlp_site_start<T>(P, mslot.s, fluid, g, a0);
                 if (fluid)
-                    update_site<L, T, EQ, Store<S>::kProject, true, true>(P, g, x, y, t, nonfinite, nc, a0, &ds);
+                    update_site<L, T, EQ, Store<S>::kProject, true, true>(P, g, x, y, t, state.nonfinite, state.nc,
+                                                                          a0, &ds);
             } else {
                 if (fluid)
-                    update_site<L, T, EQ, Store<S>::kProject, true, true>(P, g, x, y, t, nonfinite, nc, nullptr,
-                                                                          &ds);
+                    update_site<L, T, EQ, Store<S>::kProject, true, true>(P, g, x, y, t, state.nonfinite, state.nc,
+                                                                          nullptr, &ds);
             }
             if (inside) {
 #pragma unroll
@@ -1390,8 +1440,9 @@ __device__ __noinline__ void tma_tile_general(const Params& P, const S* box, int
                     Store<S>::store(dst + i * plane + o, 0, fluid ? store_round<L, S>(i, g[i]) : g[i]);
             }
         }
-        sink.put(P, ds, (unsigned)(y * P.nx + x));
+        state.sink.put(P, ds, (unsigned)(y * P.nx + x));
     }
+    return state;
 }
 
 
@@ -1401,8 +1452,8 @@ __device__ __noinline__ void tma_tile_general(const Params& P, const S* box, int
 // then x = nx - 1, one site per lane, gathered from the source field with
 // the boundary rules (gather_site).  Every lane of the block calls.
 template <typename S, int EQ, int R, typename Sink>
-__device__ __noinline__ void edge_item(const Params& P, int item, long long t, Sink& sink, MlpSlot<EQ>& mslot,
-                                       bool& nonfinite, NewtonCount& nc) {
+__device__ __noinline__ TileState<Sink> edge_item(const Params& P, int item, long long t, TileState<Sink> state,
+                                                  MlpSlot<EQ>& mslot) {
     using L = D2Q9;
     using T = typename Store<S>::T;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1423,10 +1474,12 @@ __device__ __noinline__ void edge_item(const Params& P, int item, long long t, S
     if constexpr (EQ == EQ_ENERGY_MLP) {
         float a0[3];
         mlp_site_start<T>(P, mslot.s, fluid, g, a0);
-        if (fluid) update_site<L, T, EQ, Store<S>::kProject, true, true>(P, g, x, y, t, nonfinite, nc, a0, &ds);
+        if (fluid)
+            update_site<L, T, EQ, Store<S>::kProject, true, true>(P, g, x, y, t, state.nonfinite, state.nc, a0, &ds);
     } else {
         if (fluid)
-            update_site<L, T, EQ, Store<S>::kProject, true, true>(P, g, x, y, t, nonfinite, nc, nullptr, &ds);
+            update_site<L, T, EQ, Store<S>::kProject, true, true>(P, g, x, y, t, state.nonfinite, state.nc, nullptr,
+                                                                  &ds);
     }
     if (inside) {
         S* dst = static_cast<S*>(P.dst);
@@ -1435,7 +1488,8 @@ __device__ __noinline__ void edge_item(const Params& P, int item, long long t, S
         for (int i = 0; i < L::Q; i++)
             Store<S>::store(dst, i * P.plane + o, fluid ? store_round<L, S>(i, g[i]) : g[i]);
     }
-    sink.put(P, ds, (unsigned)(y * P.nx + x));
+    state.sink.put(P, ds, (unsigned)(y * P.nx + x));
+    return state;
 }
 
 // Exact dS of the pending sites of a clean staged row (warp w: row y; lane
@@ -1444,8 +1498,8 @@ __device__ __noinline__ void edge_item(const Params& P, int item, long long t, S
 // computed it; the sites go to the sink (which keeps the candidates).  Every
 // lane of the warp calls.
 template <typename S, int EQ, int R, int TX, typename Sink>
-__device__ __noinline__ void resolve_staged_row(const Params& P, const S* box, int x0, int y, unsigned pmask,
-                                                Sink& sink) {
+__device__ __noinline__ Sink resolve_staged_row(const Params& P, const S* box, int x0, int y, unsigned pmask,
+                                                Sink sink) {
     using L = D2Q9;
     using T = typename Store<S>::T;
     using LY = TmaLayout<S, R, TX>;
@@ -1464,21 +1518,135 @@ __device__ __noinline__ void resolve_staged_row(const Params& P, const S* box, i
         }
         sink.put(P, ds, (unsigned)(y * P.nx + x0 + c));
     }
+    return sink;
 }
 
-// One staged tile: rows y0 .. y0 + R - 1 and columns x0 .. x0 + 127 of the
+// Boundary rules of a staged row, written into the staged planes: where the
+// source of population i at a fluid site x of row y lies outside the grid in
+// y or inside the obstacle, the staged slot it would be read from -- plane
+// i, column x - v_ix of the warp's own row of that plane's window, which no
+// other site reads -- takes the population the rule gives (gather_site; the
+// columns x = 0 and x = nx - 1 go apart, edge_item).  The row then takes the
+// interior path as it stands.  prestream (the first step after a state
+// upload): every slot takes its own site's population.  The window rows
+// outside the grid and the obstacle's sites hold zeros before.  Warp w: row
+// y; every lane calls.
+// Every load of a rule is issued before its first use, and whole rows at
+// once at the y sides, so a patched row costs about one memory latency more
+// than a plain one; evaluated site by site with the rules (the former path for
+// every tile that touched a wall, the obstacle, a ragged edge or the probe) a
+// row took about 10 us: at 2048 x 1024 the last block ended 12 - 28 us after
+// the median one.
+template <typename S, int R, int TX>
+__device__ __noinline__ void patch_row(const Params& P, S* box, int x0, int y) {
+    using L = D2Q9;
+    using T = typename Store<S>::T;
+    using LY = TmaLayout<S, R, TX>;
+    constexpr int C = TX / 32;   // sites per lane
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    S* sb = box + warp * LY::W + LY::H;
+    const S* __restrict__ src = static_cast<const S*>(P.src);
+    const long long row = (long long)y * P.nxp;
+    if (P.prestream) {
+#pragma unroll 1
+        for (int c = lane; c < TX; c += 32) {
+            const int x = x0 + c;
+            if (x < 1 || x > P.nx - 2) continue;
+            S v[L::Q];
+#pragma unroll
+            for (int i = 0; i < L::Q; i++) v[i] = src[i * P.plane + row + x];
+#pragma unroll
+            for (int i = 0; i < L::Q; i++) sb[i * LY::PLANE + c - L::cx(i)] = v[i];
+        }
+    } else if (y == 0 || y == P.ny - 1) {
+        // the three populations that come from beyond the side: v_y = e
+        const int e = y == 0 ? 1 : -1;
+        const int kind = P.bc[y == 0 ? 2 : 3];
+        const long long far = (long long)(P.ny - 1 - y) * P.nxp;   // periodic: the opposite row
+        S v[3][C];
+#pragma unroll
+        for (int p = 0; p < 3; p++) {
+            const int cx = p == 0 ? 0 : (p == 1 ? 1 : -1);
+            const int i = e > 0 ? (p == 0 ? 2 : (p == 1 ? 5 : 6)) : (p == 0 ? 4 : (p == 1 ? 8 : 7));
+            const int mir = e > 0 ? (p == 0 ? 4 : (p == 1 ? 8 : 7)) : (p == 0 ? 2 : (p == 1 ? 5 : 6));
+            const int opp = e > 0 ? (p == 0 ? 4 : (p == 1 ? 7 : 8)) : (p == 0 ? 2 : (p == 1 ? 6 : 5));
+            const bool bb = kind != BC_PERIODIC && kind != BC_FREESLIP;
+            const S* q = src + (kind == BC_PERIODIC ? i : (bb ? opp : mir)) * P.plane +
+                         (kind == BC_PERIODIC ? far : row) + x0 - (bb ? 0 : cx);
+#pragma unroll
+            for (int s = 0; s < C; s++) {
+                const int c = lane + 32 * s, x = x0 + c;
+                if (x >= 1 && x <= P.nx - 2) v[p][s] = q[c];
+            }
+        }
+#pragma unroll
+        for (int p = 0; p < 3; p++) {
+            const int cx = p == 0 ? 0 : (p == 1 ? 1 : -1);
+            const int i = e > 0 ? (p == 0 ? 2 : (p == 1 ? 5 : 6)) : (p == 0 ? 4 : (p == 1 ? 8 : 7));
+#pragma unroll
+            for (int s = 0; s < C; s++) {
+                const int c = lane + 32 * s, x = x0 + c;
+                if (x >= 1 && x <= P.nx - 2) sb[i * LY::PLANE + c - cx] = v[p][s];
+            }
+        }
+    }
+    if (!P.prestream && P.ow > 0 && y >= P.oy0 - 1 && y <= P.oy0 + P.oh) {
+#pragma unroll 1
+        for (int c = lane; c < TX; c += 32) {
+            const int x = x0 + c;
+            const bool mine = x >= 1 && x <= P.nx - 2 && x >= P.ox0 - 1 && x <= P.ox0 + P.ow && !is_solid(P, x, y);
+            if (!__any_sync(0xffffffffu, mine)) continue;
+            if (mine) {
+                T g[L::Q];
+                unsigned links = 0u;
+#pragma unroll
+                for (int i = 0; i < L::Q; i++) {
+                    g[i] = Store<S>::load(src, L::opp(i) * P.plane + row + x);
+                    if (i > 0 && is_solid(P, x - L::cx(i), y - L::cy(i))) links |= 1u << i;
+                }
+                if (P.wall == WALL_DIFFUSE && links) diffuse_wall<L, T>(links, g);
+#pragma unroll
+                for (int i = 1; i < L::Q; i++)
+                    if ((links >> i) & 1u) Store<S>::store(sb + i * LY::PLANE + c - L::cx(i), 0, g[i]);
+            }
+        }
+    }
+    // the stage is refilled by the async proxy after the block's next barrier
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncwarp();
+}
+
+// u_x of the probe site of a staged row (the values the update read), logged
+// for step t.  One lane calls.
+template <typename S, int EQ, int R, int TX>
+__device__ __noinline__ void log_probe(const Params& P, const S* box, int x0, long long t) {
+    using L = D2Q9;
+    using T = typename Store<S>::T;
+    using LY = TmaLayout<S, R, TX>;
+    const S* sb = box + (threadIdx.x >> 5) * LY::W + LY::H + (P.probe_x - x0);
+    T g[L::Q], drho, rho, jx, jy, ux, uy;
+#pragma unroll
+    for (int i = 0; i < L::Q; i++) g[i] = Store<S>::load(sb + i * LY::PLANE - L::cx(i), 0);
+    moments<L, T>(g, Par<T>::rho0(P), drho, rho, jx, jy);
+    velocity<T>(jx, jy, rho, ux, uy);
+    P.probe_ring[t % P.ring_cap] = (double)ux;
+}
+
+// One staged tile: rows y0 .. y0 + R - 1 and columns x0 .. x0 + TX - 1 of the
 // run P, from box (the tile's staged source planes); warp w computes row
-// y0 + w, lane l the sites x0 + l + 32 s.  The updated sites go to sink.
-// Pc: the parameters for the out-of-line rule-by-rule path (the same values
-// as P, held where that path reads them fast).
-// SPLIT: the columns x = 0 and x = nx - 1 are not updated here (edge_item
-// updates them); a tile then takes the interior path whenever it spans TX
-// columns of the grid and its rows and columns stay away from the y sides
-// and the obstacle.
-template <typename S, int EQ, int R, int TX = kTmaTX, bool SPLIT = false, typename Sink>
-__device__ __forceinline__ void tma_tile(const Params& P, const S* box, int x0, int y0, long long t, Sink& sink,
-                                         MlpSlot<EQ>& mslot, bool& nonfinite, NewtonCount& nc,
-                                         const Params& Pc) {
+// y0 + w, lane l the site pairs x0 + 2 l + 64 s.  The updated sites go to sink.
+// Pc: the parameters for the out-of-line paths (the same values as P, held
+// where those paths read them fast).  state: what the warp carries on.
+// Every row takes one path, the shifted shared-memory reads, after patch_row
+// has put the boundary rules' populations into the rows that need any.  The
+// sites that are not the tile's to update (the columns x = 0 and x = nx - 1,
+// which edge_item updates, columns past the grid, the obstacle's sites) are
+// updated from the rest state at unit density, whatever the staged planes
+// hold, and are neither stored nor pending; solid sites hold zeros in both
+// buffers from the start.
+template <typename S, int EQ, int R, int TX = kTmaTX, typename Sink>
+__device__ __forceinline__ void tma_tile(const Params& P, S* box, int x0, int y0, long long t,
+                                         TileState<Sink>& state, MlpSlot<EQ>& mslot, const Params& Pc) {
     using L = D2Q9;
     using T = typename Store<S>::T;
     using LY = TmaLayout<S, R, TX>;
@@ -1486,87 +1654,98 @@ __device__ __forceinline__ void tma_tile(const Params& P, const S* box, int x0, 
     S* __restrict__ dst = static_cast<S*>(P.dst);
     const int nxp = P.nxp, plane = (int)P.plane;
     const int y = y0 + warp;
-    const bool xin = SPLIT ? x0 + TX <= P.nx : x0 >= 1 && x0 + TX <= P.nx - 1;
-    const bool clean = !P.prestream && xin && y0 >= 1 && y0 + R <= P.ny - 1 &&
-                       (P.ow == 0 || x0 + TX + 1 <= P.ox0 || x0 - 1 >= P.ox0 + P.ow ||
-                        y0 + R + 1 <= P.oy0 || y0 - 1 >= P.oy0 + P.oh);
+    // one test clears almost every tile of the rows' own tests below
+    const bool plain = !P.prestream && y0 >= 1 && y0 + R <= P.ny - 1 &&
+                       (P.ow == 0 || x0 + TX < P.ox0 || x0 > P.ox0 + P.ow || y0 + R < P.oy0 || y0 > P.oy0 + P.oh);
+    bool solid_row = false;
+    if (!plain) {
+        if (y >= P.ny) return;
+        const bool near_obstacle = P.ow > 0 && y >= P.oy0 - 1 && y <= P.oy0 + P.oh && x0 + TX >= P.ox0 &&
+                                   x0 <= P.ox0 + P.ow;
+        if constexpr (sizeof(S) == 2) {
+            if (near_obstacle && P.wall == WALL_DIFFUSE && !P.prestream) {
+                state = tma_tile_general<S, EQ, R, TX>(Pc, box, x0, y0, t, state, mslot);
+                return;
+            }
+        }
+        if (P.prestream || y == 0 || y == P.ny - 1 || near_obstacle) patch_row<S, R, TX>(Pc, box, x0, y);
+        solid_row = near_obstacle && y >= P.oy0 && y < P.oy0 + P.oh;
+    }
     const S* sb = box + warp * LY::W + LY::H;
-    // Interior tile without the probe site (almost every tile): every site is
-    // fluid and away from every boundary rule, so the sites take the shifted
-    // shared-memory reads with no per-site checks (the branch is uniform).
-    const bool probe_here = P.probe_ring && P.probe_y >= y0 && P.probe_y < y0 + R &&
-                            P.probe_x >= x0 && P.probe_x < x0 + TX;
-    if (clean && !probe_here) {
-        const int row = y * nxp + x0;
-        unsigned pmask = 0u;   // pending sites of the lane (bit 2 s + h: column 2 l + 64 s + h)
-        const bool edge_tile = SPLIT && (x0 == 0 || x0 + TX >= P.nx - 1);
-        // two adjacent sites per lane, columns c and c + 1 (c = 2 l + 64 s):
-        // planes at rest and every store move both with one access, and the
-        // two updates are independent work for the scheduler
+    const int row = y * nxp + x0;
+    unsigned pmask = 0u;   // pending sites of the lane (bit 2 s + h: column 2 l + 64 s + h)
+    const bool masked = x0 == 0 || x0 + TX >= P.nx || solid_row;   // uniform: some sites are not the row's
+    // two adjacent sites per lane, columns c and c + 1 (c = 2 l + 64 s):
+    // planes at rest and every store move both with one access, and the
+    // two updates are independent work for the scheduler
 #pragma unroll 1
-        for (int s = 0; s < TX / 64; s++) {
-            const int c = 2 * lane + 64 * s;
-            T ga[L::Q], gb[L::Q];
+    for (int s = 0; s < TX / 64; s++) {
+        const int c = 2 * lane + 64 * s;
+        T ga[L::Q], gb[L::Q];
+#pragma unroll
+        for (int i = 0; i < L::Q; i++) {
+            const S* q = sb + i * LY::PLANE + c;
+            if (L::cx(i) == 0) {
+                PairIO<S>::load(q, ga[i], gb[i]);
+            } else {
+                ga[i] = Store<S>::load(q - L::cx(i), 0);
+                gb[i] = Store<S>::load(q + 1 - L::cx(i), 0);
+            }
+        }
+        bool ea = false, eb = false;   // not the row's sites
+        if (masked) {
+            const int x = x0 + c;
+            ea = x == 0 || x >= P.nx - 1 || (solid_row && x >= P.ox0 && x < P.ox0 + P.ow);
+            eb = x + 1 >= P.nx - 1 || (solid_row && x + 1 >= P.ox0 && x + 1 < P.ox0 + P.ow);
+            const T r1 = T(1) - Par<T>::rho0(P);
 #pragma unroll
             for (int i = 0; i < L::Q; i++) {
-                const S* q = sb + i * LY::PLANE + c;
-                if (L::cx(i) == 0) {
-                    PairIO<S>::load(q, ga[i], gb[i]);
-                } else {
-                    ga[i] = Store<S>::load(q - L::cx(i), 0);
-                    gb[i] = Store<S>::load(q + 1 - L::cx(i), 0);
-                }
+                ga[i] = ea ? T(L::w(i)) * r1 : ga[i];
+                gb[i] = eb ? T(L::w(i)) * r1 : gb[i];
             }
-            // SPLIT: a site of column 0 or nx - 1 (lane 0 or 31 of an edge
-            // tile) is left to edge_item; it is updated here from the rest
-            // state at unit density (whatever the staged halo holds) and is
-            // neither stored nor pending
-            bool ea = false, eb = false;
-            if constexpr (SPLIT) {
-                if (edge_tile) {   // uniform: only the tiles at either end of the rows
-                    ea = x0 + c == 0 || x0 + c == P.nx - 1;
-                    eb = x0 + c + 1 == P.nx - 1;
-                    const T r1 = T(1) - Par<T>::rho0(P);
-#pragma unroll
-                    for (int i = 0; i < L::Q; i++) {
-                        ga[i] = ea ? T(L::w(i)) * r1 : ga[i];
-                        gb[i] = eb ? T(L::w(i)) * r1 : gb[i];
-                    }
-                }
-            }
-            bool pa, pb;
-            if constexpr (EQ == EQ_ENERGY_MLP) {
-                float a0[3];
-                mlp_site_start<T>(P, mslot.s, true, ga, a0);
-                pa = update_site<L, T, EQ, Store<S>::kProject, false>(P, ga, x0 + c, y, t, nonfinite, nc, a0);
-                mlp_site_start<T>(P, mslot.s, true, gb, a0);
-                pb = update_site<L, T, EQ, Store<S>::kProject, false>(P, gb, x0 + c + 1, y, t, nonfinite, nc, a0);
-            } else {
-                pa = update_site<L, T, EQ, Store<S>::kProject, false>(P, ga, x0 + c, y, t, nonfinite, nc);
-                pb = update_site<L, T, EQ, Store<S>::kProject, false>(P, gb, x0 + c + 1, y, t, nonfinite, nc);
-            }
-            if (!(ea | eb)) {
-#pragma unroll
-                for (int i = 0; i < L::Q; i++)
-                    PairIO<S>::store(dst + i * plane + row + c, store_round<L, S>(i, ga[i]),
-                                     store_round<L, S>(i, gb[i]));
-            } else {
-#pragma unroll
-                for (int i = 0; i < L::Q; i++) {
-                    if (!ea) Store<S>::store(dst + i * plane + row + c, 0, store_round<L, S>(i, ga[i]));
-                    if (!eb) Store<S>::store(dst + i * plane + row + c + 1, 0, store_round<L, S>(i, gb[i]));
-                }
-            }
-            pa = pa && !ea;
-            pb = pb && !eb;
-            pmask |= ((pa ? 1u : 0u) | (pb ? 2u : 0u)) << (2 * s);
         }
-        // the row's pending sites, from the staged planes (valid until the
-        // next tile's barrier), out of line: the update keeps its registers
-        if (__any_sync(0xffffffffu, pmask != 0u)) resolve_staged_row<S, EQ, R, TX>(Pc, box, x0, y, pmask, sink);
-        return;
+        bool pa, pb;
+        // (the sites that are not the row's do not count as solved)
+        NewtonCount na = state.nc;
+        if constexpr (EQ == EQ_ENERGY_MLP) {
+            float a0[3];
+            mlp_site_start<T>(P, mslot.s, true, ga, a0);
+            pa = update_site<L, T, EQ, Store<S>::kProject, false>(P, ga, x0 + c, y, t, state.nonfinite, na, a0);
+            if (!ea) state.nc = na;
+            na = state.nc;
+            mlp_site_start<T>(P, mslot.s, true, gb, a0);
+            pb = update_site<L, T, EQ, Store<S>::kProject, false>(P, gb, x0 + c + 1, y, t, state.nonfinite, na, a0);
+            if (!eb) state.nc = na;
+        } else {
+            pa = update_site<L, T, EQ, Store<S>::kProject, false>(P, ga, x0 + c, y, t, state.nonfinite, na);
+            if (EQ >= EQ_ENERGY && !ea) state.nc = na;
+            na = state.nc;
+            pb = update_site<L, T, EQ, Store<S>::kProject, false>(P, gb, x0 + c + 1, y, t, state.nonfinite, na);
+            if (EQ >= EQ_ENERGY && !eb) state.nc = na;
+        }
+        if (!(ea | eb)) {
+#pragma unroll
+            for (int i = 0; i < L::Q; i++)
+                PairIO<S>::store(dst + i * plane + row + c, store_round<L, S>(i, ga[i]),
+                                 store_round<L, S>(i, gb[i]));
+        } else {
+#pragma unroll
+            for (int i = 0; i < L::Q; i++) {
+                if (!ea) Store<S>::store(dst + i * plane + row + c, 0, store_round<L, S>(i, ga[i]));
+                if (!eb) Store<S>::store(dst + i * plane + row + c + 1, 0, store_round<L, S>(i, gb[i]));
+            }
+        }
+        pa = pa && !ea;
+        pb = pb && !eb;
+        pmask |= ((pa ? 1u : 0u) | (pb ? 2u : 0u)) << (2 * s);
     }
-    tma_tile_general<S, EQ, R, TX, SPLIT>(Pc, box, x0, y0, t, sink, mslot, nonfinite, nc, clean);
+    // the row's pending sites, from the staged planes (valid until the
+    // next tile's barrier), out of line: the update keeps its registers
+    if (__any_sync(0xffffffffu, pmask != 0u))
+        state.sink = resolve_staged_row<S, EQ, R, TX>(Pc, box, x0, y, pmask, state.sink);
+    if (P.probe_ring && y == P.probe_y && lane == 0 && P.probe_x >= x0 && P.probe_x < x0 + TX &&
+        P.probe_x >= 1 && P.probe_x <= P.nx - 2 && !is_solid(P, P.probe_x, y))
+        log_probe<S, EQ, R, TX>(Pc, box, x0, t);
 }
 // Resident blocks per SM the staged kernel is compiled for: two in general
 // (128 registers per thread with 8-row tiles, 170 with 6-row tiles); three
@@ -1600,18 +1779,6 @@ __global__ void __launch_bounds__(32 * R, tma_min_blocks<S, R, TX>())
         sh.abort = 0;
         sh.bc.n = 0;
     }
-    // Launched as a programmatic dependent of the previous kernel in the
-    // stream: the block may start while that kernel finishes, and the code
-    // above reads only the launch's parameters and writes only shared
-    // memory.  Every thread waits here until the previous kernel has
-    // completed and its writes are visible, then lets the next kernel of the
-    // stream start its blocks as this one's leave the SMs (they wait here in
-    // turn).
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    mslot.fill(P);
-    __syncthreads();
-    const long long t = *P.step;
     const int tiles_x = (P.nx + TX - 1) / TX;
     const int tiles = tiles_x * ((P.ny + R - 1) / R);
     // the x = 0 and x = nx - 1 columns go first, as edge items of 32 R sites
@@ -1638,6 +1805,23 @@ __global__ void __launch_bounds__(32 * R, tma_min_blocks<S, R, TX>())
         next_tile = c < 0 ? -2 - next_claim : c;
         if (P.tile_order && c >= 0 && c < tiles) next_tile = __ldg(P.tile_order + c);
     };
+    if (threadIdx.x == 0) {
+        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<unsigned long long>(&tm)) : "memory");
+        claim();
+    }
+    // Launched as a programmatic dependent of the previous kernel in the
+    // stream: the block may start while that kernel finishes, and the code
+    // above reads only the launch's parameters and the claim order (which no
+    // kernel writes) and writes only shared memory.  Every thread waits here
+    // until the previous kernel has completed and its writes are visible, then
+    // lets the next kernel of the stream start its blocks as this one's leave
+    // the SMs (they wait here in turn).
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    mslot.fill(P);
+    __syncthreads();
+    const long long t = *P.step;
+
     auto fill = [&](int st) {
         unsigned long long* bar = &full[st];
         if (next_claim >= claims || next_tile < 0) {
@@ -1656,14 +1840,8 @@ __global__ void __launch_bounds__(32 * R, tma_min_blocks<S, R, TX>())
         for (int i = 0; i < L::Q; i++)
             tma_load_3d(base + i * LY::PLANE, &tm, tx * TX - LY::H, ty * R - L::cy(i), i, bar);
     };
-    if (threadIdx.x == 0) {
-        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<unsigned long long>(&tm))
-                     : "memory");
-        claim();
+    if (threadIdx.x == 0)
         for (int st = 0; st < STAGES - 1; st++) fill(st);
-    }
-    bool nonfinite = false;
-    NewtonCount nc = {0, 0, 0, 0};
     // The sites the dS bound does not clear are resolved as they are
     // updated; the candidates go to the block's buffer, which the block cuts
     // to its k best between tiles.  A cut happens once some warp appended
@@ -1672,7 +1850,7 @@ __global__ void __launch_bounds__(32 * R, tma_min_blocks<S, R, TX>())
     // and one tile adds at most TX * R.
     const int kept = P.k > 0 && P.k < kRoom ? P.k : 0;
     const unsigned share = (unsigned)((kRoom - kept) / R);
-    CandSink<kCap> sink{&sh.bc, 0u};
+    TileState<CandSink<kCap>> state{{&sh.bc, 0u}, {0, 0, 0, 0}, false};
     int jj = 0;
     for (;; jj++) {
         const int st = jj % STAGES;
@@ -1683,14 +1861,14 @@ __global__ void __launch_bounds__(32 * R, tma_min_blocks<S, R, TX>())
         // so that the barriers stay matched
         const bool ok = mbar_wait(&full[st], parity);
         if (!ok) sh.abort = 1;
-        if (__syncthreads_or(!ok || sink.count > share)) {
+        if (__syncthreads_or(!ok || state.sink.count > share)) {
             if (sh.abort) {
                 if (threadIdx.x == 0) atomicOr(P.err, ERR_TIMEOUT);
                 break;
             }
             if (P.k < kRoom) block_cut(sh.bc, sh.ss.sc, P.k);
             else block_flush(sh.p, sh.bc);
-            sink.count = 0;
+            state.sink.count = 0;
         }
         const int tile = sh.tile[st];
         if (tile == -1) break;
@@ -1702,12 +1880,12 @@ __global__ void __launch_bounds__(32 * R, tma_min_blocks<S, R, TX>())
             fill((jj + STAGES - 1) % STAGES);
         }
         if (tile <= -2) {
-            edge_item<S, EQ, R>(sh.p, -2 - tile, t, sink, mslot, nonfinite, nc);
+            state = edge_item<S, EQ, R>(sh.p, -2 - tile, t, state, mslot);
             continue;
         }
         const int ty = tile / tiles_x, tx = tile - ty * tiles_x;
-        const S* box = stages + (size_t)st * (LY::STAGE_BYTES / sizeof(S));
-        tma_tile<S, EQ, R, TX, true>(P, box, tx * TX, ty * R, t, sink, mslot, nonfinite, nc, sh.p);
+        S* box = stages + (size_t)st * (LY::STAGE_BYTES / sizeof(S));
+        tma_tile<S, EQ, R, TX>(P, box, tx * TX, ty * R, t, state, mslot, sh.p);
     }
     __syncthreads();
     if (sh.abort && threadIdx.x == 0) {
@@ -1717,9 +1895,8 @@ __global__ void __launch_bounds__(32 * R, tma_min_blocks<S, R, TX>())
             mbar_wait(&full[j2 % STAGES], (unsigned)((j2 / STAGES) & 1));
         }
     }
-    if (nonfinite) atomicOr(P.err, ERR_NONFINITE);
-    if constexpr (EQ >= EQ_ENERGY) flush_newton(P, nc);
-    __syncthreads();
+    if (state.nonfinite) atomicOr(P.err, ERR_NONFINITE);
+    if constexpr (EQ >= EQ_ENERGY) flush_newton(P, state.nc);
     // the staged tiles are no longer needed: their memory holds the last
     // block's candidate staging
     const int scap = (int)min((size_t)kStage, (size_t)STAGES * LY::STAGE_BYTES / 12);
