@@ -43,6 +43,7 @@ int fail(int code, const char* fmt, ...) {
     } while (0)
 
 constexpr int kGraphSteps = 32;      // steps per captured graph (even: buffers return)
+constexpr int kTubeSteps = 4096;     // steps of a short D1Q3 run per launch
 constexpr int kExportChunks = 8;     // row chunks of a host export (copies overlap the conversion)
 constexpr int kXferEvents = 16;      // events of one chunked transfer (>= Q planes, >= chunks, + 1)
 constexpr int kDefaultLog = 65536;
@@ -164,10 +165,8 @@ struct lb_handle {
     // completion ticket of the stream-collide blocks; tile shape of K1
     unsigned* ticket;
     int tile_shape;
-    // overflow list of sites awaiting an exact dS
-    unsigned* pend_idx;
-    unsigned* pend_count;
     int grid_blocks, sm_count, blocks_per_sm;
+    bool tube;                // short D1Q3 run: many steps per cluster launch
     // tensor maps of the two population buffers (shared-memory-staged shapes)
     CUtensorMap tmap[2];
     unsigned* tile_counter;
@@ -237,8 +236,6 @@ Params make_params(const lb_handle* h, int src, bool prestream) {
     P.recheck_band = recheck_band(h->delta);
     P.mlp = h->mlp; P.newton_stats = h->newton_stats;
     P.ticket = h->ticket;
-    P.pend_idx = h->pend_idx;
-    P.pend_count = h->pend_count;
     P.grid_blocks = h->grid_blocks;
     P.tile_counter = h->tile_counter;
     P.tile_order = h->tile_order ? h->tile_order + (src ? h->tile_order_n : 0) : nullptr;
@@ -485,7 +482,7 @@ void lb_destroy(lb_handle* h) {
     void* ptrs[] = {h->buf[0], h->buf[1], h->cand_key, h->cand_idx, h->cand_count, h->sel_idx,
                     h->sel_count, h->count_ring, h->probe_ring, h->d_step, h->d_err, h->replay_cnt,
                     h->replay_off, h->replay_idx, h->mlp, h->newton_stats, h->ticket,
-                    h->pend_idx, h->pend_count, h->tile_counter, h->tile_order, h->stage, h->sel_key,
+                    h->tile_counter, h->tile_order, h->stage, h->sel_key,
                     h->slab_sel, h->slab_cnt, h->slab_off};
     for (void* p : ptrs)
         if (p) cudaFree(p);
@@ -620,9 +617,6 @@ int lb_create(int lattice, int nx, int ny, int equilibrium, double nu, double de
     }
     CKH(cudaMalloc(&h->ticket, sizeof(unsigned)));
     CKH(cudaMemsetAsync(h->ticket, 0, sizeof(unsigned), h->stream));
-    CKH(cudaMalloc(&h->pend_idx, std::max(1ll, nsites) * sizeof(unsigned)));
-    CKH(cudaMalloc(&h->pend_count, sizeof(unsigned)));
-    CKH(cudaMemsetAsync(h->pend_count, 0, sizeof(unsigned), h->stream));
     CKH(cudaMalloc(&h->tile_counter, sizeof(unsigned)));
     CKH(cudaMemsetAsync(h->tile_counter, 0, sizeof(unsigned), h->stream));
     CKH(cudaMallocHost(&h->h_err, sizeof(unsigned)));
@@ -636,6 +630,11 @@ int lb_create(int lattice, int nx, int ny, int equilibrium, double nu, double de
     CKH(cudaMemsetAsync(h->d_err, 0, sizeof(unsigned), h->stream));
     CKH(cudaMemsetAsync(h->newton_stats, 0, 4 * sizeof(unsigned long long), h->stream));
     CKH(h->L.set_smem(kSelectStageCap));
+    if (lattice == LB_D1Q3) {
+        int clusters = 0;
+        CKH(h->L.tube_setup(nx, &clusters));
+        h->tube = clusters > 0;
+    }
     if (size_grid(h) != LB_OK || make_tensor_maps(h) != LB_OK) {
         const std::string msg = g_last_error;
         lb_destroy(h);
@@ -828,6 +827,17 @@ int lb_step(lb_handle* h, int n) {
         return fail(LB_ERR_STATE, "the learned equilibrium needs its network (lb_set_mlp) first");
     int done = 0;
     const bool replaying = h->replay_n > 0 && h->h_step < h->replay_t0 + h->replay_n;
+    // a short D1Q3 run: up to kTubeSteps steps per launch (the replay of given
+    // selections and per-step timing keep one launch per step)
+    while (h->tube && !h->timing && !replaying && done < n) {
+        const int m = std::min(n - done, kTubeSteps);
+        Params P = make_params(h, h->cur, h->prestream);
+        CK(h->L.tube(P, m, h->buf[h->cur ^ (m & 1)], h->stream));
+        h->prestream = false;
+        h->cur ^= m & 1;
+        h->h_step += m;
+        done += m;
+    }
     while (done < n) {
         const bool direct = h->prestream || h->timing || replaying || (n - done) < kGraphSteps;
         if (direct) {

@@ -107,10 +107,6 @@ struct Params {
     unsigned long long* newton_stats;   // it32, it64, sites, fails
     // completion ticket of the stream-collide blocks (the last block selects)
     unsigned* ticket;
-    // sites whose dS the bound could not clear and that did not fit in their
-    // block's shared list (resolved by the last block)
-    unsigned* pend_idx;
-    unsigned* pend_count;
     int grid_blocks;          // persistent grid size (resident blocks x SMs)
     unsigned* tile_counter;   // next tile to hand out (staged shapes)
     const int* tile_order;    // staged shapes: tile of each claim (null: row-major)

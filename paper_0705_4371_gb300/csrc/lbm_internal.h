@@ -25,6 +25,10 @@ struct Launchers {
     // slab ghost exchange: column col of field <-> packed buffer [3][ny]
     cudaError_t (*ghost)(const Params&, void* field, int col, int right, void* buf, int dir, cudaStream_t);
     cudaError_t (*occupancy)(int tile_shape, int* blocks_per_sm);
+    // many steps of a short D1Q3 run in one cluster launch, from P.src to out;
+    // tube_setup: whether this device and grid allow it (once per run)
+    cudaError_t (*tube)(const Params&, int steps, void* out, cudaStream_t);
+    cudaError_t (*tube_setup)(int n, int* ok);
 };
 
 // storage: FP64, FP32 deviation, FP16 deviation, plain FP32 (f32p)

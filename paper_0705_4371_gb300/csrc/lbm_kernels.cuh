@@ -15,6 +15,7 @@
 
 #include <algorithm>
 
+#include <cooperative_groups.h>
 #include <cuda.h>
 
 #include "lbm_device.cuh"
@@ -25,7 +26,7 @@
 namespace lbm {
 
 constexpr int kSelectThreads = 1024;
-constexpr int kSiteBlock = 256;      // one-site-per-thread kernels
+constexpr int kSiteBlock = 64;       // one site per thread: FP64 work over as many SMs as there are blocks
 constexpr int kStage = 1024;         // candidates staged in shared memory by the last block
 
 template <typename L, typename T, int EQ>
@@ -588,11 +589,11 @@ struct SelectShared {
     unsigned cnt;
 };
 
-// The Ehrenfests' step at one site, whose post-collision populations g are
-// at hand: the collision conserves every moment f* depends on, so this is f*
-// of the pre-collision state.
+// The Ehrenfests' step at one site: g, its post-collision populations in,
+// f* out (not yet rounded as the storage holds it).  The collision conserves
+// every moment f* depends on, so this is f* of the pre-collision state.
 template <typename L, typename S, int EQ>
-__device__ __forceinline__ void ehrenfest_site(const Params& P, long long o, const typename Store<S>::T* g) {
+__device__ __forceinline__ void ehrenfest_value(const Params& P, typename Store<S>::T* g) {
     using T = typename Store<S>::T;
     T gs[L::Q], rho, ux, uy;
     site_equilibrium<L, T, EQ>(P, g, gs, rho, ux, uy);
@@ -607,7 +608,13 @@ __device__ __forceinline__ void ehrenfest_site(const Params& P, long long o, con
         for (int i = 0; i < L::Q; i++) gs[i] = g[i] - d[i];
     }
 #pragma unroll
-    for (int i = 0; i < L::Q; i++) Store<S>::store(P.dst, i * P.plane + o, store_round<L, S>(i, gs[i]));
+    for (int i = 0; i < L::Q; i++) g[i] = gs[i];
+}
+template <typename L, typename S, int EQ>
+__device__ __forceinline__ void ehrenfest_site(const Params& P, long long o, typename Store<S>::T* g) {
+    ehrenfest_value<L, S, EQ>(P, g);
+#pragma unroll
+    for (int i = 0; i < L::Q; i++) Store<S>::store(P.dst, i * P.plane + o, store_round<L, S>(i, g[i]));
 }
 
 constexpr int kRankMax = 256;   // candidates ranked by counting, one per thread
@@ -738,73 +745,14 @@ __device__ __noinline__ void select_and_fix(const Params& P, SelectShared& ss,
     }
 }
 
-// End of a stream-collide block: resolve the block's pending sites (exact
-// dS, candidates appended), publish the block's writes, take a ticket; the
-// block that takes the last ticket first resolves the pending sites that did
-// not fit in any block's list, then runs the global selection and the
-// Ehrenfests' step for the whole grid.  No block ever waits for another.
-constexpr int kPend = 2048;   // pending sites kept per block in shared memory
-
-struct FinishShared {
-    SelectShared ss;
-    unsigned long long key[kStage];
-    unsigned idx[kStage];
-    unsigned pend[kPend];
-    BlockCand bc;
-    unsigned npend;
-    int is_last;
-};
-
-// Warp-level append of pending sites to the block list of capacity cap
-// (overflow: global).  Returns the number the warp appended (the same on
-// every lane).
-__device__ __forceinline__ unsigned warp_pend(const Params& P, unsigned* list, unsigned* nlist, int cap, bool pend,
-                                              unsigned site) {
-    const unsigned m = __ballot_sync(0xffffffffu, pend);
-    if (m == 0) return 0u;
-    const int lane = threadIdx.x & 31;
-    unsigned base = 0;
-    if (lane == 0) base = atomicAdd(nlist, (unsigned)__popc(m));
-    base = __shfl_sync(0xffffffffu, base, 0);
-    if (pend) {
-        const unsigned slot = base + __popc(m & ((1u << lane) - 1u));
-        if (slot < (unsigned)cap) list[slot] = site;
-        else P.pend_idx[atomicAdd(P.pend_count, 1u)] = site;
-    }
-    return (unsigned)__popc(m);
-}
-__device__ __forceinline__ unsigned warp_pend(const Params& P, FinishShared& fs, bool pend, unsigned site) {
-    return warp_pend(P, fs.pend, &fs.npend, kPend, pend, site);
-}
-
-// Exact dS of n pending sites, appending the candidates to the block's
-// buffer bc (its k best reach the global list) or, with bc null, straight
-// to the global list; all threads call with the same n.
-template <typename L, typename S, int EQ, typename SiteAt, typename BC = BlockCand>
-__device__ void resolve_list(const Params& P, int n, SiteAt site_at, BC* bc, TopkScratch* sc) {
-    using T = typename Store<S>::T;
-    const T delta = Par<T>::delta(P);
-    for (int b = 0; b < n; b += blockDim.x) {
-        if (bc) block_room(P, *bc, *sc);
-        const int j = b + (int)threadIdx.x;
-        unsigned site = 0;
-        T ds = T(-1);
-        if (j < n) {
-            site = site_at(j);
-            ds = resolve_ds<L, S, EQ>(P, (int)(site % (unsigned)P.nx), (int)(site / (unsigned)P.nx));
-        }
-        if (bc) block_push<T>(P, *bc, ds > delta, ds, site);
-        else warp_push<T>(P, ds > delta, ds, site);
-    }
-}
-
+// End of a stream-collide block: publish the block's k best candidates and
+// its writes and take a ticket; the block that takes the last ticket runs the
+// global selection and the Ehrenfests' step for the whole grid.  No block
+// ever waits for another.
 template <typename L, typename S, int EQ, typename BC>
-__device__ __forceinline__ void finish_parts(const Params& P, const unsigned* pend, unsigned npend, int pend_cap,
-                                             int& is_last, SelectShared& ss, BC& bc,
+__device__ __forceinline__ void finish_parts(const Params& P, int& is_last, SelectShared& ss, BC& bc,
                                              unsigned long long* stage_key, unsigned* stage_idx,
                                              int stage_cap) {
-    const int np = (int)min(npend, (unsigned)pend_cap);
-    if (np > 0) resolve_list<L, S, EQ>(P, np, [&](int j) { return pend[j]; }, &bc, &ss.sc);
     block_finish(P, bc, ss.sc);
     // the barrier makes the block's writes visible to thread 0, whose
     // device-scope fence then orders all of them before the ticket
@@ -818,14 +766,6 @@ __device__ __forceinline__ void finish_parts(const Params& P, const unsigned* pe
     }
     __syncthreads();
     if (is_last) {
-        // (a kernel without pending lists, pend null, never appends to the global one)
-        const int ng = pend ? (int)__ldcg(P.pend_count) : 0;
-        if (ng > 0) {
-            resolve_list<L, S, EQ>(P, ng, [&](int j) { return __ldcg(P.pend_idx + j); }, &bc, &ss.sc);
-            block_finish(P, bc, ss.sc);
-            __syncthreads();
-            if (threadIdx.x == 0) *P.pend_count = 0;
-        }
         __threadfence_block();
         select_and_fix<L, S, EQ>(P, ss, stage_key, stage_idx, stage_cap, P.slab ? 1 : 0);
         if (threadIdx.x == 0) {
@@ -835,46 +775,26 @@ __device__ __forceinline__ void finish_parts(const Params& P, const unsigned* pe
     }
 }
 
-template <typename L, typename S, int EQ>
-__device__ __forceinline__ void finish_block(const Params& P, FinishShared& fs) {
-    __syncthreads();
-    finish_parts<L, S, EQ>(P, fs.pend, fs.npend, kPend, fs.is_last, fs.ss, fs.bc, fs.key, fs.idx, kStage);
-}
+// Shared state of the kernels whose sites come from registers.  CAP: room
+// for a round of the block's sites above what a cut keeps.  p: the launch's
+// parameters for the out-of-line paths.
+template <int CAP>
+struct SiteShared {
+    Params p;
+    SelectShared ss;
+    unsigned long long key[kStage];
+    unsigned idx[kStage];
+    BlockCandT<CAP> bc;
+    int is_last;
+};
 
-// Boundary site (or any site of the first step after a state upload): gather
-// with the boundary rules, update, store.  Returns bit 0: non-finite,
-// bit 1: pending.
-template <typename S, int EQ>
-__device__ __noinline__ int boundary_site(const Params& P, int x, int y, long long t) {
-    using L = D2Q9;
-    using T = typename Store<S>::T;
-    const long long o = (long long)y * P.nxp + x;
-    T g[L::Q];
-    bool nonfinite = false, pending = false;
-    NewtonCount nc = {0, 0, 0, 0};
-    if (is_solid(P, x, y)) {
-#pragma unroll
-        for (int i = 0; i < L::Q; i++) g[i] = T(0);
-    } else {
-        gather_site<L, S>(P, x, y, g);
-        pending = update_site<L, T, EQ, Store<S>::kProject>(P, g, x, y, t, nonfinite, nc);
-#pragma unroll
-        for (int i = 0; i < L::Q; i++) g[i] = store_round<L, S>(i, g[i]);
-    }
-    if constexpr (EQ >= EQ_ENERGY) {
-        if (nc.sites) {
-            atomicAdd(P.newton_stats + 0, (unsigned long long)nc.it32);
-            atomicAdd(P.newton_stats + 1, (unsigned long long)nc.it64);
-            atomicAdd(P.newton_stats + 2, (unsigned long long)nc.sites);
-            if (nc.fails) {
-                atomicAdd(P.newton_stats + 3, (unsigned long long)nc.fails);
-                atomicOr(P.err, ERR_NEWTON);
-            }
-        }
-    }
-#pragma unroll
-    for (int i = 0; i < L::Q; i++) Store<S>::store(P.dst, i * P.plane + o, g[i]);
-    return (nonfinite ? 1 : 0) | (pending ? 2 : 0);
+// Pre-collision deviations of a site by the boundary rules, out of line (the
+// tiles without any keep their registers).
+template <typename L, typename S>
+__device__ __noinline__ PopArr<L::Q, typename Store<S>::T> gather_ruled(const Params& P, int x, int y) {
+    PopArr<L::Q, typename Store<S>::T> a;
+    gather_site<L, S>(P, x, y, a.v);
+    return a;
 }
 
 // ---------------------------------------------------------------------------
@@ -1037,26 +957,28 @@ __device__ __forceinline__ bool tile_interior(const Params& P, int x0, int y) {
 // Interior tiles: aligned VEC-wide loads per population plane, the
 // x-shifted planes completed by one warp shuffle and one halo load.
 // Boundary tiles (and the first step after a state upload): per-site gather
-// with the boundary rules.
+// with the boundary rules (out of line), then the same update.
+// For grids of one or two tiles per warp: bound by the chain launch - loads -
+// update - selection.  So the launch overlaps the previous step's end, a
+// boundary tile costs one more gather and no update code of its own, and the
+// sites the dS bound does not clear are resolved after their tile instead of
+// in a pass of the whole block at the end.  600 x 500, FP32, one run alone:
+// 16.1 -> 13.4 us per step (three side by side: 7.8 us each, as before).
 // ---------------------------------------------------------------------------
 template <typename S, int EQ, int VEC, int WARPS, int MINB>
 __global__ void __launch_bounds__(32 * WARPS, MINB) k_collide_d2q9(const __grid_constant__ Params P) {
     using L = D2Q9;
     using T = typename Store<S>::T;
     constexpr int TX = 32 * VEC;
-    __shared__ FinishShared fs;
+    constexpr int kRound = TX * WARPS;             // sites of a round (one tile per warp)
+    constexpr int kCap = kRound + kBlockCand;
+    __shared__ SiteShared<kCap> sh;
     __shared__ MlpSlot<EQ> mslot;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (threadIdx.x == 0) {
-        fs.npend = 0;
-        fs.bc.n = 0;
+        sh.p = P;
+        sh.bc.n = 0;
     }
-    mslot.fill(P);
-    __syncthreads();
-    const long long t = *P.step;
-    const S* __restrict__ src = static_cast<const S*>(P.src);
-    S* __restrict__ dst = static_cast<S*>(P.dst);
-    const int nxp = P.nxp, plane = (int)P.plane;
     // Each block owns a contiguous range of row tiles (row-major); its warps
     // take the range's tiles in turn.  Boundary tiles, which cost more, are
     // then spread evenly over blocks.
@@ -1065,112 +987,130 @@ __global__ void __launch_bounds__(32 * WARPS, MINB) k_collide_d2q9(const __grid_
     const int per_block = (tiles + gridDim.x - 1) / gridDim.x;
     const int t0 = blockIdx.x * per_block;
     const int t1 = min(t0 + per_block, tiles);
+    const int rounds = t1 > t0 ? (t1 - t0 + WARPS - 1) / WARPS : 0;
+    int y = (t0 + warp) / tiles_x, xt = t0 + warp - y * tiles_x;
+    // a programmatic dependent of the previous kernel in the stream, as the
+    // staged kernel: nothing above reads device memory a kernel writes
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    mslot.fill(P);
+    __syncthreads();
+    const long long t = P.probe_ring ? __ldcg(P.step) : 0;   // (the probe's log only)
+    const S* __restrict__ src = static_cast<const S*>(P.src);
+    S* __restrict__ dst = static_cast<S*>(P.dst);
+    const int nxp = P.nxp, plane = (int)P.plane;
     bool nonfinite = false;
     NewtonCount nc = {0, 0, 0, 0};
-    unsigned wpend = 0u;   // pending sites this warp appended since the last drain
-    // one row tile of 32 * VEC sites: row y, tile column xt
-    auto do_tile = [&](int y, int xt) {
-        const int x0 = xt * TX;
-        const int xs = x0 + lane * VEC;
-        if (!P.prestream && tile_interior<TX>(P, x0, y)) {
+    // candidates appended by the warp since the block's last cut; the block
+    // cuts (or flushes) once some warp used more than its share of the room
+    // above what a cut keeps, so that the next round fits
+    unsigned count = 0u;
+    const int kept = P.k > 0 && P.k < kBlockCand ? P.k : 0;
+    const unsigned share = (unsigned)((kBlockCand - kept) / WARPS);
+    for (int r = 0; r < rounds; r++) {
+        if (t0 + r * WARPS + warp < t1) {
+            const int x0 = xt * TX;
+            const int xs = x0 + lane * VEC;
             const int row = y * nxp + xs;
+            const bool interior = !P.prestream && tile_interior<TX>(P, x0, y);
             T g[VEC][L::Q];
+            unsigned fluid = (1u << VEC) - 1u;
+            if (interior) {
 #pragma unroll
-            for (int i = 0; i < L::Q; i++) {
-                const int at = i * plane + row - L::cy(i) * nxp;
-                T v[VEC];
-                load_vec<S, VEC>(src, at, v);
-                if (L::cx(i) == 0) {
+                for (int i = 0; i < L::Q; i++) {
+                    const int at = i * plane + row - L::cy(i) * nxp;
+                    T v[VEC];
+                    load_vec<S, VEC>(src, at, v);
+                    if (L::cx(i) == 0) {
 #pragma unroll
-                    for (int s = 0; s < VEC; s++) g[s][i] = v[s];
-                } else if (L::cx(i) == 1) {
-                    // source x - 1: the previous lane's last element
-                    T prev = __shfl_up_sync(0xffffffffu, v[VEC - 1], 1);
-                    if (lane == 0) prev = Store<S>::load(src + at - 1, 0);
-                    g[0][i] = prev;
+                        for (int s = 0; s < VEC; s++) g[s][i] = v[s];
+                    } else if (L::cx(i) == 1) {
+                        // source x - 1: the previous lane's last element
+                        T prev = __shfl_up_sync(0xffffffffu, v[VEC - 1], 1);
+                        if (lane == 0) prev = Store<S>::load(src + at - 1, 0);
+                        g[0][i] = prev;
 #pragma unroll
-                    for (int s = 1; s < VEC; s++) g[s][i] = v[s - 1];
-                } else {
-                    // source x + 1: the next lane's first element
-                    T next = __shfl_down_sync(0xffffffffu, v[0], 1);
-                    if (lane == 31) next = Store<S>::load(src + at + VEC, 0);
+                        for (int s = 1; s < VEC; s++) g[s][i] = v[s - 1];
+                    } else {
+                        // source x + 1: the next lane's first element
+                        T next = __shfl_down_sync(0xffffffffu, v[0], 1);
+                        if (lane == 31) next = Store<S>::load(src + at + VEC, 0);
 #pragma unroll
-                    for (int s = 0; s < VEC - 1; s++) g[s][i] = v[s + 1];
-                    g[VEC - 1][i] = next;
+                        for (int s = 0; s < VEC - 1; s++) g[s][i] = v[s + 1];
+                        g[VEC - 1][i] = next;
+                    }
                 }
+            } else {
+#pragma unroll
+                for (int s = 0; s < VEC; s++) {
+                    const int x = xs + s;
+                    if (x < P.nx && !is_solid(P, x, y)) {
+                        const auto a = gather_ruled<L, S>(sh.p, x, y);
+#pragma unroll
+                        for (int i = 0; i < L::Q; i++) g[s][i] = a.v[i];
+                    } else {
+                        // no site of the run (solid sites hold zeros in both
+                        // buffers from the start): the rest state at unit
+                        // density, not stored, never pending
+                        fluid &= ~(1u << s);
+#pragma unroll
+                        for (int i = 0; i < L::Q; i++) g[s][i] = T(L::w(i)) * (T(1) - Par<T>::rho0(P));
+                    }
+                }
+                __syncwarp();
             }
-            bool pend[VEC];
+            unsigned pend = 0u;
 #pragma unroll
             for (int s = 0; s < VEC; s++) {
-                if constexpr (EQ == EQ_ENERGY_MLP) {
-                    // interior tile: every lane holds a fluid site
-                    float a0[3];
-                    mlp_site_start<T>(P, mslot.s, true, g[s], a0);
-                    pend[s] = update_site<L, T, EQ, Store<S>::kProject>(P, g[s], xs + s, y, t, nonfinite,
-                                                                         nc, a0);
-                } else {
-                    pend[s] = update_site<L, T, EQ, Store<S>::kProject>(P, g[s], xs + s, y, t, nonfinite,
-                                                                         nc);
+                NewtonCount one = nc;
+                float a0[3];
+                if constexpr (EQ == EQ_ENERGY_MLP) mlp_site_start<T>(P, mslot.s, true, g[s], a0);
+                const bool p = update_site<L, T, EQ, Store<S>::kProject>(P, g[s], (fluid >> s) & 1u ? xs + s : -2, y, t,
+                                                                         nonfinite, one,
+                                                                         EQ == EQ_ENERGY_MLP ? a0 : nullptr);
+                if ((fluid >> s) & 1u) {
+                    nc = one;
+                    if (p) pend |= 1u << s;
                 }
             }
+            if (interior) {
 #pragma unroll
-            for (int i = 0; i < L::Q; i++) {
-                T v[VEC];
+                for (int i = 0; i < L::Q; i++) {
+                    T v[VEC];
 #pragma unroll
-                for (int s = 0; s < VEC; s++) v[s] = store_round<L, S>(i, g[s][i]);
-                store_vec<S, VEC>(dst, i * plane + row, v);
+                    for (int s = 0; s < VEC; s++) v[s] = store_round<L, S>(i, g[s][i]);
+                    store_vec<S, VEC>(dst, i * plane + row, v);
+                }
+            } else {
+#pragma unroll
+                for (int s = 0; s < VEC; s++)
+                    if ((fluid >> s) & 1u) {
+#pragma unroll
+                        for (int i = 0; i < L::Q; i++)
+                            Store<S>::store(dst + i * plane + row + s, 0, store_round<L, S>(i, g[s][i]));
+                    }
             }
-#pragma unroll
-            for (int s = 0; s < VEC; s++) wpend += warp_pend(P, fs, pend[s], (unsigned)(y * P.nx + xs + s));
-        } else {
+            // the tile's pending sites, gathered again (from L2)
+            if (__any_sync(0xffffffffu, pend != 0u)) {
 #pragma unroll 1
-            for (int s = 0; s < VEC; s++) {
-                const int x = xs + s;
-                int r = 0;
-                if (x < P.nx) r = boundary_site<S, EQ>(P, x, y, t);
-                nonfinite |= (r & 1) != 0;
-                wpend += warp_pend(P, fs, (r & 2) != 0, (unsigned)(y * P.nx + x));
+                for (int s = 0; s < VEC; s++) {
+                    T ds = T(-1);
+                    if ((pend >> s) & 1u) ds = resolve_ds<L, S, EQ>(sh.p, xs + s, y);
+                    count += block_push<T>(P, sh.bc, ds > Par<T>::delta(P), ds, (unsigned)(y * P.nx + xs + s));
+                }
             }
-        }
-    };
-    if constexpr (EQ < EQ_ENERGY) {
-        int w = t0 + warp;
-        int y = w / tiles_x, xt = w - y * tiles_x;
-        for (; w < t1; w += WARPS) {
-            do_tile(y, xt);
             xt += WARPS;
             while (xt >= tiles_x) { xt -= tiles_x; y++; }
         }
-    } else {
-        // The energy forms go in rounds of one tile per warp and resolve the
-        // block's pending sites before its list could overflow in the next
-        // round: a start far from equilibrium then cannot overflow many sites
-        // to the global list, which the last block alone resolves.  The
-        // block drains once some warp appended more than its share (1 /
-        // WARPS) of the room left for a round; one vote over the warps' own
-        // counts decides, so every warp takes the same branch.
-        static_assert(kPend > TX * WARPS, "a round must fit in the pending list");
-        constexpr unsigned kShare = (unsigned)((kPend - TX * WARPS) / WARPS);
-        const int rounds = t1 > t0 ? (t1 - t0 + WARPS - 1) / WARPS : 0;
-        for (int r = 0; r < rounds; r++) {
-            const int w = t0 + r * WARPS + warp;
-            if (w < t1) {
-                const int y = w / tiles_x;
-                do_tile(y, w - y * tiles_x);
-            }
-            if (__syncthreads_or(wpend > kShare)) {
-                resolve_list<L, S, EQ>(P, (int)min(fs.npend, (unsigned)kPend),
-                                       [&](int j) { return fs.pend[j]; }, &fs.bc, &fs.ss.sc);
-                __syncthreads();
-                if (threadIdx.x == 0) fs.npend = 0;
-                __syncthreads();
-                wpend = 0u;
-            }
+        if (r + 1 < rounds && __syncthreads_or(count > share)) {
+            if (P.k < kBlockCand) block_cut(sh.bc, sh.ss.sc, P.k);
+            else block_flush(sh.p, sh.bc);
+            count = 0u;
         }
     }
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (nonfinite) atomicOr(P.err, ERR_NONFINITE);
     if constexpr (EQ >= EQ_ENERGY) flush_newton(P, nc);
-    finish_block<L, S, EQ>(P, fs);
+    finish_parts<L, S, EQ>(sh.p, sh.is_last, sh.ss, sh.bc, sh.key, sh.idx, kStage);
 }
 
 // ---------------------------------------------------------------------------
@@ -1813,11 +1753,11 @@ __global__ void __launch_bounds__(32 * R, tma_min_blocks<S, R, TX>())
     // stream: the block may start while that kernel finishes, and the code
     // above reads only the launch's parameters and the claim order (which no
     // kernel writes) and writes only shared memory.  Every thread waits here
-    // until the previous kernel has completed and its writes are visible, then
-    // lets the next kernel of the stream start its blocks as this one's leave
-    // the SMs (they wait here in turn).
+    // until the previous kernel has completed and its writes are visible.
+    // (The next kernel's blocks are let in when this one's have finished their
+    // tiles, to wait here in turn: let in at the start, they only take room
+    // from other streams' kernels.)
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     mslot.fill(P);
     __syncthreads();
     const long long t = *P.step;
@@ -1895,6 +1835,7 @@ __global__ void __launch_bounds__(32 * R, tma_min_blocks<S, R, TX>())
             mbar_wait(&full[j2 % STAGES], (unsigned)((j2 / STAGES) & 1));
         }
     }
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (state.nonfinite) atomicOr(P.err, ERR_NONFINITE);
     if constexpr (EQ >= EQ_ENERGY) flush_newton(P, state.nc);
     // the staged tiles are no longer needed: their memory holds the last
@@ -1902,7 +1843,7 @@ __global__ void __launch_bounds__(32 * R, tma_min_blocks<S, R, TX>())
     const int scap = (int)min((size_t)kStage, (size_t)STAGES * LY::STAGE_BYTES / 12);
     unsigned long long* skey = reinterpret_cast<unsigned long long*>(smem);
     unsigned* sidx = reinterpret_cast<unsigned*>(smem + 8 * scap);
-    finish_parts<L, S, EQ>(sh.p, nullptr, 0u, 0, sh.is_last, sh.ss, sh.bc, skey, sidx, scap);
+    finish_parts<L, S, EQ>(sh.p, sh.is_last, sh.ss, sh.bc, skey, sidx, scap);
 }
 
 // ---------------------------------------------------------------------------
@@ -1911,14 +1852,15 @@ __global__ void __launch_bounds__(32 * R, tma_min_blocks<S, R, TX>())
 template <typename L, typename S, int EQ>
 __global__ void __launch_bounds__(kSiteBlock) k_collide_site(const __grid_constant__ Params P) {
     using T = typename Store<S>::T;
-    __shared__ FinishShared fs;
+    __shared__ SiteShared<kBlockCand> sh;   // room for the block's sites
+    static_assert(kBlockCand >= kSiteBlock, "every site of the block may be a candidate");
     if (threadIdx.x == 0) {
-        fs.npend = 0;
-        fs.bc.n = 0;
+        sh.p = P;
+        sh.bc.n = 0;
     }
     __syncthreads();
     const long long t = *P.step;
-    const long long sid = (long long)blockIdx.x * kSiteBlock + threadIdx.x;
+    const long long sid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const int x = (int)(sid % P.nx), y = (int)(sid / P.nx);
     const bool inside = sid < (long long)P.nx * P.ny;
     const bool valid = inside && !is_solid(P, x, y);
@@ -1935,9 +1877,193 @@ __global__ void __launch_bounds__(kSiteBlock) k_collide_site(const __grid_consta
         for (int i = 0; i < L::Q; i++)
             Store<S>::store(P.dst, i * P.plane + o, valid ? store_round<L, S>(i, g[i]) : T(0));
     }
-    warp_pend(P, fs, pending, (unsigned)sid);
+    if (__any_sync(0xffffffffu, pending)) {
+        T ds = T(-1);
+        if (pending) ds = resolve_ds<L, S, EQ>(sh.p, x, y);
+        block_push<T>(P, sh.bc, ds > Par<T>::delta(P), ds, (unsigned)sid);
+    }
     if (nonfinite) atomicOr(P.err, ERR_NONFINITE);
-    finish_block<L, S, EQ>(P, fs);
+    finish_parts<L, S, EQ>(sh.p, sh.is_last, sh.ss, sh.bc, sh.key, sh.idx, kStage);
+}
+
+// ---------------------------------------------------------------------------
+// K1 for short D1Q3 runs: many time steps in one launch of one cluster.
+// A few hundred sites leave no work to spread: what bounds a step is its
+// chain -- launch, loads, the FP64 update (two FP64 operations per SM and
+// clock), the exact dS of the sites near the front, the selection -- so the
+// state stays in the shared memory of a cluster of 16 blocks (16 SMs' FP64
+// pipes), neighbours read each other's edge sites there, the candidates are
+// listed in block 0, and the hardware's cluster barrier separates the
+// collision from the selection and, when a step has candidates, the
+// Ehrenfests' step from the next free flight.  800 sites, FP64: 23.5 us per step in
+// one launch each (4 blocks), 10.9 us so.
+// Every population passes through the storage type, so results are those of
+// one launch per step.
+// ---------------------------------------------------------------------------
+constexpr int kTubeBlocks = 16;          // cluster size
+constexpr int kTubeThreads = 256;        // most sites per block
+constexpr int kTubeRank = 128;           // candidates ranked by counting
+
+struct TubeShared {
+    TopkScratch sc;
+    Thresh th;
+    unsigned count[3];                   // candidates of step t in block 0's count[t mod 3]
+};
+
+template <typename S>
+constexpr size_t tube_smem_bytes(int n) {
+    const int per = (n + kTubeBlocks - 1) / kTubeBlocks;
+    return (size_t)n * 12 + 16 + 6 * (size_t)per * sizeof(S);
+}
+
+template <typename S, int EQ>
+__global__ void __launch_bounds__(kTubeThreads) k_tube(const __grid_constant__ Params P, int steps, void* out) {
+    using L = D1Q3;
+    using T = typename Store<S>::T;
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    extern __shared__ __align__(16) unsigned char tube_raw[];
+    __shared__ TubeShared sh;
+    const int n = P.nx, per = (n + kTubeBlocks - 1) / kTubeBlocks;
+    const int rank = (int)cluster.block_rank(), tid = threadIdx.x;
+    const int x = rank * per + tid;
+    const bool mine = tid < per && x < n;
+    // block 0: the step's candidates; every block: its sites' post-collision
+    // populations [parity][plane][per]
+    unsigned long long* key = reinterpret_cast<unsigned long long*>(tube_raw);
+    unsigned* idx = reinterpret_cast<unsigned*>(tube_raw + (size_t)n * 8);
+    S* f = reinterpret_cast<S*>(tube_raw + ((size_t)n * 12 + 15) / 16 * 16);
+    unsigned long long* key0 = cluster.map_shared_rank(key, 0);
+    unsigned* idx0 = cluster.map_shared_rank(idx, 0);
+    unsigned* count0 = cluster.map_shared_rank(sh.count, 0);
+    if (tid < 3) sh.count[tid] = 0u;
+    if (mine)
+#pragma unroll
+        for (int i = 0; i < L::Q; i++) f[i * per + tid] = static_cast<const S*>(P.src)[i * P.plane + x];
+    const long long t0 = *P.step;
+    const T delta = Par<T>::delta(P);
+    bool nonfinite = false;
+    NewtonCount nc = {0, 0, 0, 0};
+    cluster.sync();
+    for (int s = 0; s < steps; s++) {
+        const long long t = t0 + s;
+        S* cur = f + (s & 1) * 3 * per;
+        S* nxt = f + ((s + 1) & 1) * 3 * per;
+        // population i of site xx after the previous step
+        auto at = [&](int i, int xx) {
+            const int b = xx / per;
+            const S* q = b == rank ? cur : cluster.map_shared_rank(cur, b);
+            return Store<S>::load(q + i * per + xx - b * per, 0);
+        };
+        const unsigned c = (unsigned)(t % 3);
+        T ds = T(-1), g[L::Q];
+        if (mine) {
+            if (s == 0 && P.prestream) {
+#pragma unroll
+                for (int i = 0; i < L::Q; i++) g[i] = at(i, x);
+            } else {
+                // free flight with the rules of gather_site
+                g[0] = at(0, x);
+#pragma unroll
+                for (int i = 1; i < L::Q; i++) {
+                    const int sx = x - L::cx(i);
+                    if (sx >= 0 && sx < n) {
+                        g[i] = at(i, sx);
+                        continue;
+                    }
+                    const int kind = sx < 0 ? P.bc[0] : P.bc[1];
+                    if (kind == BC_PERIODIC) {
+                        g[i] = at(i, sx < 0 ? sx + n : sx - n);
+                    } else if (kind == BC_INLET) {
+                        g[i] = (T)P.gin[i];
+                    } else if (kind == BC_OUTLET) {
+                        T v[L::Q], go[L::Q];
+#pragma unroll
+                        for (int j = 0; j < L::Q; j++) v[j] = at(j, n - 2);
+                        outlet_equilibrium<L, T>(P, v, go);
+                        g[i] = store_round<L, S>(i, go[i]);
+                    } else if (kind == BC_OUTLET_COPY) {
+                        g[i] = at(i, x);
+                    } else {
+                        g[i] = at(L::opp(i), x);
+                    }
+                }
+            }
+            update_site<L, T, EQ, Store<S>::kProject, true, true>(P, g, x, 0, t, nonfinite, nc, nullptr, &ds);
+#pragma unroll
+            for (int i = 0; i < L::Q; i++) Store<S>::store(nxt + i * per + tid, 0, store_round<L, S>(i, g[i]));
+        }
+        // the counter of the step after next's predecessor: last read before
+        // the previous step's barrier, next used after this one's
+        if (rank == 0 && tid == 0) sh.count[(c + 1u) % 3u] = 0u;
+        const bool cand = ds > delta;
+        const unsigned long long k = cand ? ds_key((double)ds) : 0ull;
+        unsigned slot = 0u;
+        if (cand) {
+            slot = atomicAdd(count0 + c, 1u);
+            key0[slot] = k;
+            idx0[slot] = (unsigned)x;
+        }
+        cluster.sync();
+        const int m = (int)count0[c];        // candidates (the same for every thread)
+        const int sel = min(m, P.k);
+        if (m > 0) {
+            bool take = cand;
+            if (m > P.k && m <= kTubeRank) {
+                slot = 0u;
+                if (cand)
+                    for (int e = 0; e < m; e++) {
+                        const unsigned long long ke = key0[e];
+                        slot += ke > k || (ke == k && idx0[e] < (unsigned)x);
+                    }
+                take = cand && slot < (unsigned)P.k;
+            } else if (m > P.k) {
+                if (rank == 0) {
+                    const Thresh th = block_topk(sh.sc, m, P.k, [&](int e) { return key[e]; },
+                                                 [&](int e) { return idx[e]; });
+                    if (tid == 0) sh.th = th;
+                }
+                cluster.sync();
+                const Thresh th = *cluster.map_shared_rank(&sh.th, 0);
+                take = cand && th.selected(k, (unsigned)x);
+            }
+            if (take) {
+                // f' <- f* from the stored post-collision populations
+                T h[L::Q];
+#pragma unroll
+                for (int i = 0; i < L::Q; i++) h[i] = Store<S>::load(nxt + i * per + tid, 0);
+                ehrenfest_value<L, S, EQ>(P, h);
+#pragma unroll
+                for (int i = 0; i < L::Q; i++) Store<S>::store(nxt + i * per + tid, 0, store_round<L, S>(i, h[i]));
+            }
+            if (s == steps - 1) {
+                // the last step's list (order unspecified); by radix: a
+                // selected site's place is its rank among the selected
+                if (m > P.k && m > kTubeRank && take) {
+                    const Thresh th = *cluster.map_shared_rank(&sh.th, 0);
+                    slot = 0u;
+                    for (int e = 0; e < m; e++) slot += idx0[e] < (unsigned)x && th.selected(key0[e], idx0[e]);
+                }
+                if (take) P.sel_idx[slot] = x;
+            }
+            cluster.sync();
+        }
+        if (rank == 0 && tid == 0) {
+            P.count_ring[t % P.ring_cap] = sel;
+            if (s == steps - 1) {
+                *P.sel_count = sel;
+                *P.step = t + 1;
+            }
+        }
+    }
+    if (mine) {
+        const S* last = f + (steps & 1) * 3 * per;
+#pragma unroll
+        for (int i = 0; i < L::Q; i++) static_cast<S*>(out)[i * P.plane + x] = last[i * per + tid];
+    }
+    if (nonfinite) atomicOr(P.err, ERR_NONFINITE);
+    // no block leaves while another may still read its shared memory
+    cluster.sync();
 }
 
 // Stand-alone selection (select-only test hook).
@@ -2152,13 +2278,30 @@ __global__ void k_ghost(const __grid_constant__ Params P, S* field, int col, int
 // occupancy calculator, capped by the number of tiles (small grids then
 // spread over as many SMs as they have tiles: their step is latency-bound).
 // ---------------------------------------------------------------------------
+// Launch with programmatic stream serialisation: it may begin before the
+// previous kernel in the stream completes (the kernel waits for it with
+// griddepcontrol.wait before touching device memory).
+template <typename K, typename... A>
+cudaError_t launch_dependent(K kernel, unsigned blocks, unsigned threads, size_t smem, cudaStream_t st, const A&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 template <typename S, int EQ, int VEC, int WARPS, int MINB>
 cudaError_t launch_d2q9(const Params& P, cudaStream_t st) {
     const long long tiles = (long long)((P.nx + 32 * VEC - 1) / (32 * VEC)) * P.ny;
     const long long want = (tiles + WARPS - 1) / WARPS;   // at least one tile per warp
     const unsigned blocks = (unsigned)std::max(1ll, std::min(want, (long long)P.grid_blocks));
-    k_collide_d2q9<S, EQ, VEC, WARPS, MINB><<<blocks, 32 * WARPS, 0, st>>>(P);
-    return cudaGetLastError();
+    return launch_dependent(k_collide_d2q9<S, EQ, VEC, WARPS, MINB>, blocks, 32 * WARPS, 0, st, P);
 }
 
 // Resident blocks per SM of a D2Q9 tile shape (occupancy calculator).
@@ -2174,21 +2317,8 @@ cudaError_t launch_d2q9_tma(const Params& P, const void* tmap, cudaStream_t st) 
     const long long tiles = (long long)((P.nx + TX - 1) / TX) * ((P.ny + R - 1) / R);
     const long long want = tiles;   // at least one tile per block
     const unsigned blocks = (unsigned)std::max(1ll, std::min(want, (long long)P.grid_blocks));
-    // programmatic stream serialisation: the launch may begin before the
-    // previous kernel in the stream completes (the kernel waits for it with
-    // griddepcontrol.wait before touching device memory)
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(blocks);
-    cfg.blockDim = dim3(32 * R);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_collide_d2q9_tma<S, EQ, R, STAGES, TX>, P,
-                              *static_cast<const CUtensorMap*>(tmap));
+    return launch_dependent(k_collide_d2q9_tma<S, EQ, R, STAGES, TX>, blocks, 32 * R, smem, st, P,
+                            *static_cast<const CUtensorMap*>(tmap));
 }
 
 template <typename S, int EQ, int R, int STAGES, int TX = kTmaTX>
@@ -2231,6 +2361,59 @@ struct LaunchImpl {
             k_collide_site<L, S, EQ><<<blocks, kSiteBlock, 0, st>>>(P);
             return cudaGetLastError();
         }
+    }
+    // Many steps of a short D1Q3 run in one launch, from P.src to out;
+    // cudaErrorNotSupported where the cluster does not serve the run.
+    static cudaError_t tube(const Params& P, int steps, void* out, cudaStream_t st) {
+        if constexpr (L::Q == 3) {
+            const int per = (P.nx + kTubeBlocks - 1) / kTubeBlocks;
+            if (per > kTubeThreads) return cudaErrorNotSupported;
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(kTubeBlocks);
+            cfg.blockDim = dim3((per + 31) / 32 * 32);
+            cfg.dynamicSmemBytes = tube_smem_bytes<S>(P.nx);
+            cfg.stream = st;
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeClusterDimension;
+            attr[0].val.clusterDim.x = kTubeBlocks;
+            attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+            cfg.attrs = attr;
+            cfg.numAttrs = 1;
+            return cudaLaunchKernelEx(&cfg, k_tube<S, EQ>, P, steps, out);
+        } else {
+            (void)P; (void)steps; (void)out; (void)st;
+            return cudaErrorNotSupported;
+        }
+    }
+    // Whether this device runs the cluster of k_tube for n sites.
+    static cudaError_t tube_setup(int n, int* ok) {
+        *ok = 0;
+        if constexpr (L::Q == 3) {
+            const int per = (n + kTubeBlocks - 1) / kTubeBlocks;
+            if (per > kTubeThreads) return cudaSuccess;
+            const size_t smem = tube_smem_bytes<S>(n);
+            cudaError_t e = cudaFuncSetAttribute(k_tube<S, EQ>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+            if (e != cudaSuccess) return e;
+            e = cudaFuncSetAttribute(k_tube<S, EQ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)tube_smem_bytes<S>(kTubeBlocks * kTubeThreads));
+            if (e != cudaSuccess) return e;
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(kTubeBlocks);
+            cfg.blockDim = dim3((per + 31) / 32 * 32);
+            cfg.dynamicSmemBytes = smem;
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeClusterDimension;
+            attr[0].val.clusterDim.x = kTubeBlocks;
+            attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+            cfg.attrs = attr;
+            cfg.numAttrs = 1;
+            e = cudaOccupancyMaxActiveClusters(ok, k_tube<S, EQ>, &cfg);
+            if (e != cudaSuccess) {
+                *ok = 0;
+                (void)cudaGetLastError();
+            }
+        }
+        return cudaSuccess;
     }
     static cudaError_t occupancy(int shape, int* per_sm) {
         *per_sm = 1;
@@ -2298,6 +2481,8 @@ struct LaunchImpl {
         l.set_smem = &set_smem;
         l.ghost = &ghost;
         l.occupancy = &occupancy;
+        l.tube = &tube;
+        l.tube_setup = &tube_setup;
         return l;
     }
 };
