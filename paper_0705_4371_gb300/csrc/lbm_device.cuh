@@ -240,11 +240,23 @@ template <> struct Par<double> {
 // every FP32 / FP16 form.
 // ---------------------------------------------------------------------------
 
-// FP64 value of population i whose stored deviation is g.
+// FP32 to FP64 by integer operations (the conversion instruction runs on the
+// FP64 pipe, two per SM and clock); subnormal, infinite and NaN values take
+// the instruction.
+__device__ __forceinline__ double widen(float x) {
+    const unsigned b = __float_as_uint(x), m = b & 0x7fffffffu;
+    if (m - 0x00800000u >= 0x7f000000u && m != 0u) return (double)x;
+    const unsigned hi = m ? (m >> 3) + (896u << 20) : 0u;
+    return __hiloint2double((int)(hi | (b & 0x80000000u)), (int)(b << 29));
+}
+
+// FP64 value of population i whose stored deviation is g (FP64 storage holds
+// f itself, the deviation forms have rho0 = 1).
 template <typename L, typename S>
-__device__ __forceinline__ double pop_f64(const Params& P, int i, typename Store<S>::T g) {
-    if constexpr (Store<S>::kPlain) return (double)g + (double)(float)L::w(i);
-    else return (double)g + L::w(i) * P.rho0;
+__device__ __forceinline__ double pop_f64(int i, typename Store<S>::T g) {
+    if constexpr (sizeof(typename Store<S>::T) == 8) return g;
+    else if constexpr (Store<S>::kPlain) return widen(g) + (double)(float)L::w(i);
+    else return widen(g) + L::w(i);
 }
 
 // Deviation of a population whose value f was computed in FP64 (initial and
@@ -320,35 +332,108 @@ __device__ __forceinline__ void conserve_neq(float* d) {
     }
 }
 
+// 1 / x: FP32 from the hardware approximation refined by one Newton-Raphson
+// step r + r (1 - x r) (the relative error e of the seed becomes ~e^2, below
+// one ulp); FP64 from the hardware's approximation r0 (special function
+// unit, not the FP64 pipe), with e = 1 - x r0: r0 (1 + e + e^2), whose error
+// e^3 is below 2^-57 -- three FP64 operations instead of a division's ten.
+template <typename T> __host__ __device__ __forceinline__ T recip(T x);
+template <> __host__ __device__ __forceinline__ float recip<float>(float x) {
+#ifdef __CUDA_ARCH__
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return fmaf(r, fmaf(-x, r, 1.0f), r);
+#else
+    return 1.0f / x;
+#endif
+}
+template <> __host__ __device__ __forceinline__ double recip<double>(double x) {
+#ifdef __CUDA_ARCH__
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    const double e = fma(-x, r, 1.0);
+    return fma(r, fma(e, e, e), r);
+#else
+    return 1.0 / x;
+#endif
+}
+
+// sqrt(x), x > 0: FP32 correctly rounded; FP64 from the hardware's
+// approximation r of 1 / sqrt(x): s = x r, with e = 1 - s r:
+// s + s e (1/2 + 3/8 e), whose error ~ 5/16 e^3 is below 2^-57 -- five FP64
+// operations.
 template <typename T> __host__ __device__ __forceinline__ T dsqrt(T x);
 template <> __host__ __device__ __forceinline__ float dsqrt<float>(float x) { return sqrtf(x); }
-template <> __host__ __device__ __forceinline__ double dsqrt<double>(double x) { return sqrt(x); }
+template <> __host__ __device__ __forceinline__ double dsqrt<double>(double x) {
+#ifdef __CUDA_ARCH__
+    double r;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    const double s = x * r, e = fma(-s, r, 1.0);
+    return fma(s * e, fma(0.375, e, 0.5), s);
+#else
+    return sqrt(x);
+#endif
+}
 
-// Entropic for mass and momentum.  D1Q3: closed form of Sec. 4.1 with the
-// left/right labels read so that the momentum is +rho u (rest
-// (2 rho/3)(2 - s), left (rho/6)(2s - 3u - 1), right (rho/6)(3u - 1 + 2s),
-// s = sqrt(1 + 3u^2)).  D2Q9: product formula of Sec. 4.2.
-template <typename L, typename T>
-__host__ __device__ __forceinline__ void feq_entropic(T rho, T ux, T uy, T rho0, T* gs) {
+// Entropic for mass and momentum, by axis.  Sec. 4.1's closed form (with the
+// left/right labels read so that the momentum is +rho u) is rho times
+//   rest (2/3)(2 - s), moving (1/6)(2 s - 1 +- 3 u), s = sqrt(1 + 3 u^2),
+// and the product formula of Sec. 4.2 is the product of two such axes: its
+// factors are (2 - s) ((2 u + s) / (1 - u))^{+-1} = 2 s - 1 +- 3 u, as
+// (2 - s)(2 + s) = 3 (1 - u^2).  With sigma = s - 1 = 3 u^2 / (1 + s) an axis's
+// factors are 1 + A, A = -sigma (rest), 2 sigma +- 3 u, so
+//   f*_i - W_i rho0 = W_i (drho + rho (A + B + A B)),  drho = rho - rho0,
+// without the cancellation of f*_i - W_i rho0 and without divisions (the
+// printed form takes six; in FP32 an update took 290 instructions with it).
+template <typename T>
+__host__ __device__ __forceinline__ void entropic_axis(T u, T* A) {
+    const T u3 = T(3) * u;
+    const T q = u3 * u;
+    const T s = dsqrt<T>(T(1) + q);
+    T sigma;
+    if constexpr (sizeof(T) == 8) sigma = s - T(1);
+    else sigma = q * recip<T>(T(1) + s);
+    A[0] = -sigma;
+    const T two = sigma + sigma;
+    A[1] = two + u3;
+    A[2] = two - u3;
+}
+// ZERO0: the caller's rho0 is zero (FP64 storage; drho = rho).
+template <typename L, typename T, bool ZERO0 = false>
+__host__ __device__ __forceinline__ void feq_entropic(T drho, T rho, T ux, T uy, T* gs) {
+    if constexpr (L::Q == 3 && sizeof(T) == 8) {
+        // the printed form on rho / 6, correctly rounded (quotient, residual,
+        // correction): a rounded weight's error would be the same at every
+        // site and step, a drift of the mass (5e-14 after 500 steps)
+        const T c = T(1.0 / 6.0), q = rho * c, r6 = dfma<T>(dfma<T>(T(-6), q, rho), c, q);
+        const T s = dsqrt<T>(dfma<T>(T(3) * ux, ux, T(1)));
+        const T a = dfma<T>(T(2), s, T(-1)), u3 = T(3) * ux;
+        gs[0] = T(4) * r6 * (T(2) - s);
+        gs[1] = r6 * (a - u3);
+        gs[2] = r6 * (a + u3);
+        if constexpr (!ZERO0)
+            for (int i = 0; i < 3; i++) gs[i] -= T(L::w(i)) * (rho - drho);
+        return;
+    }
+    T A[3];
+    entropic_axis<T>(ux, A);
     if constexpr (L::Q == 3) {
-        const T s = dsqrt<T>(T(1) + T(3) * ux * ux);
-        gs[0] = T(2) * rho / T(3) * (T(2) - s) - T(L::w(0)) * rho0;
-        gs[1] = rho / T(6) * (T(2) * s - T(3) * ux - T(1)) - T(L::w(1)) * rho0;
-        gs[2] = rho / T(6) * (T(3) * ux - T(1) + T(2) * s) - T(L::w(2)) * rho0;
+        // populations rest, left, right
+        gs[0] = T(L::w(0)) * dfma<T>(rho, A[0], drho);
+        gs[1] = T(L::w(1)) * dfma<T>(rho, A[2], drho);
+        gs[2] = T(L::w(2)) * dfma<T>(rho, A[1], drho);
     } else {
-        const T sx = dsqrt<T>(T(1) + T(3) * ux * ux), sy = dsqrt<T>(T(1) + T(3) * uy * uy);
-        const T ax = T(2) - sx, ay = T(2) - sy;
-        const T bx = (T(2) * ux + sx) / (T(1) - ux), by = (T(2) * uy + sy) / (T(1) - uy);
-        const T ibx = T(1) / bx, iby = T(1) / by;
-        const T base = rho * ax * ay;
+        T B[3], R[3], D[3];
+        entropic_axis<T>(uy, B);
+#pragma unroll
+        for (int j = 0; j < 3; j++) {
+            R[j] = rho * A[j];
+            D[j] = dfma<T>(rho, B[j], drho);
+        }
 #pragma unroll
         for (int i = 0; i < L::Q; i++) {
-            T p = base * T(L::w(i));
-            if (L::cx(i) == 1) p *= bx;
-            if (L::cx(i) == -1) p *= ibx;
-            if (L::cy(i) == 1) p *= by;
-            if (L::cy(i) == -1) p *= iby;
-            gs[i] = p - T(L::w(i)) * rho0;
+            const int j = L::cx(i) < 0 ? 2 : L::cx(i), k = L::cy(i) < 0 ? 2 : L::cy(i);
+            gs[i] = T(L::w(i)) * dfma<T>(R[j], B[k], R[j] + D[k]);
         }
     }
 }
@@ -359,7 +444,7 @@ __host__ __device__ __forceinline__ void feq_entropic(T rho, T ux, T uy, T rho0,
 template <typename L, typename T>
 __host__ __device__ __forceinline__ void feq_rho_u(int eq, T rho, T ux, T uy, T rho0, T* gs) {
     if (eq == EQ_POLY) feq_poly<L, T>(rho - rho0, rho, ux, uy, gs);
-    else feq_entropic<L, T>(rho, ux, uy, rho0, gs);
+    else feq_entropic<L, T>(rho - rho0, rho, ux, uy, gs);
 }
 
 // ---------------------------------------------------------------------------
@@ -395,6 +480,16 @@ template <> __device__ __forceinline__ float phi_fn<float>(float x) {
 }
 
 template <> __device__ __forceinline__ double phi_fn<double>(double x) {
+    if (fabs(x) <= 0.015625) {
+        // terms n = 2..9; truncation < 1e-16 relative at |x| = 1/64
+        double p = 0.0;
+#pragma unroll
+        for (int n = 9; n >= 2; n--) {
+            const double c = ((n & 1) ? -1.0 : 1.0) / (double(n) * double(n - 1));
+            p = fma(p, x, c);
+        }
+        return x * x * p;
+    }
     if (fabs(x) <= 0.0625) {
         // terms n = 2..17; truncation < 1e-18 relative at |x| = 1/16
         double p = 0.0;
@@ -409,17 +504,6 @@ template <> __device__ __forceinline__ double phi_fn<double>(double x) {
     return fma(1.0 + x, log1p(x), -x);
 }
 
-// 1 / x: FP32 from the hardware approximation refined by one Newton-Raphson
-// step r + r (1 - x r) (the relative error e of the seed becomes ~e^2, below
-// one ulp); FP64 divides.
-template <typename T> __device__ __forceinline__ T recip(T x);
-template <> __device__ __forceinline__ float recip<float>(float x) {
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return fmaf(r, fmaf(-x, r, 1.0f), r);
-}
-template <> __device__ __forceinline__ double recip<double>(double x) { return 1.0 / x; }
-
 // Exact dS of one site in type T; +inf outside the positive cone.
 template <typename L, typename T>
 __device__ __forceinline__ T delta_s_exact(const T* g, const T* gs, T rho0) {
@@ -430,7 +514,8 @@ __device__ __forceinline__ T delta_s_exact(const T* g, const T* gs, T rho0) {
         fs[i] = dfma<T>(T(L::w(i)), rho0, gs[i]);
         const T f = dfma<T>(T(L::w(i)), rho0, g[i]);
         bad |= !(fs[i] > T(0)) || (f < T(0));
-        x[i] = (g[i] - gs[i]) / fs[i];
+        if constexpr (sizeof(T) == 8) x[i] = (g[i] - gs[i]) * recip<T>(fs[i]);
+        else x[i] = (g[i] - gs[i]) / fs[i];
     }
     if (bad) return T(INFINITY);
     T s = T(0);
@@ -453,29 +538,63 @@ __device__ __noinline__ T delta_s_slow(PopArr<L::Q, T> g, PopArr<L::Q, T> gs, T 
 // The site is cleared when m > 0, 16 Q <= W_min m^2 and 0.55 Q <= delta m.
 // Polynomial f*: f*_i / W_i = rho (1 + 3 v.u + 9/2 (v.u)^2 - 3/2 u^2) >=
 // rho (1 - 3 (|u_x| + |u_y|) - 3/2 u^2) = m.  Other f*: m = min_i f*_i / W_i.
+// FP64 storage evaluates the bound in FP32 (FP64 operations are what its
+// update is bound by), with magnitudes cut to 20 bits (abs_float, integer
+// operations) and a relative margin of 2^-16 on each side, far above the
+// roundings: a site is cleared only if the FP64 bound clears it too, and one
+// near the limit gets its exact dS as any other site that is not cleared.
+
+// |x| as FP32, truncated to 20 significant bits (0 below 2^-126, infinity
+// from 2^128 on and for NaN), without an FP64 operation.
+__device__ __forceinline__ float abs_float(double x) {
+    const int h = __double2hiint(x) & 0x7fffffff;
+    return __int_as_float(min(max(h - (896 << 20), 0), 0x0ff00000) << 3);
+}
+
 template <typename L, typename T, int EQ>
 __device__ __forceinline__ bool ds_cleared(const T* d, const T* gs, T rho, T ux, T uy, T rho0,
-                                           T delta) {
-    T q0 = T(0), q1 = T(0), q2 = T(0);
+                                           T delta, float deltaf) {
+    // the bound's arithmetic type
+    constexpr bool narrow = sizeof(T) == 8;
+    using B = float;
+    B q0 = B(0), q1 = B(0), q2 = B(0);
 #pragma unroll
     for (int i = 0; i < L::Q; i++) {
-        if (L::w(i) == L::w(0)) q0 = dfma<T>(d[i], d[i], q0);
-        else if (L::w(i) == L::w(1)) q1 = dfma<T>(d[i], d[i], q1);
-        else q2 = dfma<T>(d[i], d[i], q2);
+        B di;
+        if constexpr (narrow) di = abs_float(d[i]);
+        else di = d[i];
+        if (L::w(i) == L::w(0)) q0 = fmaf(di, di, q0);
+        else if (L::w(i) == L::w(1)) q1 = fmaf(di, di, q1);
+        else q2 = fmaf(di, di, q2);
     }
     constexpr double wmin = L::Q == 9 ? 1.0 / 36.0 : 1.0 / 6.0;
-    const T Q = dfma<T>(q0, T(1.0 / L::w(0)), dfma<T>(q1, T(1.0 / L::w(1)),
-                        L::Q == 9 ? q2 * T(1.0 / L::w(5)) : T(0)));
-    T m;
-    if constexpr (EQ == 0) {
-        const T usq = dfma<T>(ux, ux, uy * uy);
-        m = rho * dfma<T>(T(-1.5), usq, dfma<T>(T(-3), fabs(ux) + fabs(uy), T(1)));
-    } else {
-        m = T(INFINITY);
+    B Q = fmaf(q0, B(1.0 / L::w(0)), fmaf(q1, B(1.0 / L::w(1)), L::Q == 9 ? q2 * B(1.0 / L::w(5)) : B(0)));
+    B m, dl;
+    if constexpr (narrow) {
+        const B r = abs_float(rho), vx = abs_float(ux) * B(1.0 + 0x1p-18), vy = abs_float(uy) * B(1.0 + 0x1p-18);
+        if constexpr (EQ == 0) {
+            m = r * fmaf(B(-1.5), fmaf(vx, vx, vy * vy), fmaf(B(-3), vx + vy, B(1)));
+        } else {
+            m = B(INFINITY);
 #pragma unroll
-        for (int i = 0; i < L::Q; i++) m = fmin(m, dfma<T>(gs[i], T(1.0 / L::w(i)), rho0));
+            for (int i = 0; i < L::Q; i++)
+                m = fminf(m, gs[i] > T(0) ? abs_float(gs[i]) * B(1.0 / L::w(i)) : B(-1));
+        }
+        Q *= B(1.0 + 0x1p-16);
+        m *= B(1.0 - 0x1p-16);
+        dl = deltaf * (deltaf > B(0) ? B(1.0 - 0x1p-16) : B(1.0 + 0x1p-16));
+        return (rho > T(0)) & (m > B(0)) & (B(16.0 / wmin) * Q <= m * m) & (B(0.55) * Q <= dl * m);
+    } else {
+        if constexpr (EQ == 0) {
+            const B usq = fmaf(ux, ux, uy * uy);
+            m = rho * fmaf(B(-1.5), usq, fmaf(B(-3), fabsf(ux) + fabsf(uy), B(1)));
+        } else {
+            m = B(INFINITY);
+#pragma unroll
+            for (int i = 0; i < L::Q; i++) m = fminf(m, fmaf(gs[i], B(1.0 / L::w(i)), rho0));
+        }
+        return (m > B(0)) && (B(16.0 / wmin) * Q <= m * m) && (B(0.55) * Q <= delta * m);
     }
-    return (m > T(0)) && (T(16.0 / wmin) * Q <= m * m) && (T(0.55) * Q <= delta * m);
 }
 
 // Monotone map of a double onto uint64 (larger double <=> larger key).

@@ -49,17 +49,6 @@ struct NewtonCount {
     unsigned it32, it64, sites, fails;
 };
 
-// 1 / x in FP64 from the FP32 reciprocal refined by two Newton-Raphson
-// steps (each squares the relative error: 2^-23 -> 2^-46 -> below one FP64
-// ulp).  x must lie in the normal FP32 range.
-__device__ __forceinline__ double recip64(double x) {
-    double r = (double)__frcp_rn((float)x);
-    double e = fma(-x, r, 1.0);
-    r = fma(r, e, r);
-    e = fma(-x, r, 1.0);
-    return fma(r, e, r);
-}
-
 __device__ __forceinline__ float sqrt_approx(float x) {
     float r;
     asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));

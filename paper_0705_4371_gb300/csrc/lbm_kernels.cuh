@@ -31,8 +31,9 @@ constexpr int kStage = 1024;         // candidates staged in shared memory by th
 
 template <typename L, typename T, int EQ>
 __device__ __forceinline__ void equilibrium(const Params& P, T drho, T rho, T ux, T uy, T* gs) {
+    (void)P;
     if constexpr (EQ == EQ_POLY) feq_poly<L, T>(drho, rho, ux, uy, gs);
-    else feq_entropic<L, T>(rho, ux, uy, Par<T>::rho0(P), gs);
+    else feq_entropic<L, T, sizeof(T) == 8>(drho, rho, ux, uy, gs);   // (FP64 storage: rho0 = 0)
 }
 
 // Energy-constrained entropic f* (D2Q9 only) as deviations from the
@@ -50,14 +51,20 @@ __device__ __forceinline__ void equilibrium_energy(T rho, T jx, T jy, T e2, T* g
         energy_solve_ff(rho, jx, jy, e2, mu3, gs, nc);
     } else {
         // FP64 storage (rho0 = 0): FP64 finish to 4e-15 (the FP64 parity bound)
-        const double ir = recip64(rho);
+        const double ir = recip<double>(rho);
         energy_solve(rho, jx * ir, jy * ir, e2 * ir, mu3, gs, nc, 4e-15f);
     }
 }
 
 template <typename L, typename T>
 __device__ __forceinline__ void moments(const T* g, T rho0, T& drho, T& rho, T& jx, T& jy) {
-    if constexpr (L::Q == 9) {
+    if constexpr (L::Q == 9 && sizeof(T) == 8) {
+        // sums of the diagonals shared (16 additions)
+        const T pe = g[5] + g[8], pw = g[6] + g[7];
+        jx = (g[1] - g[3]) + (pe - pw);
+        jy = (g[2] - g[4]) + ((g[5] - g[8]) + (g[6] - g[7]));
+        drho = g[0] + ((g[1] + g[3]) + (g[2] + g[4])) + (pe + pw);
+    } else if constexpr (L::Q == 9) {
         // pairwise sums (D2Q9 numbering: 1..4 E N W S, 5..8 NE NW SW SE)
         drho = ((g[0] + g[1]) + (g[2] + g[3])) + ((g[4] + g[5]) + (g[6] + g[7])) + g[8];
         jx = ((g[1] - g[3]) + (g[5] - g[6])) + (g[8] - g[7]);
@@ -71,18 +78,46 @@ __device__ __forceinline__ void moments(const T* g, T rho0, T& drho, T& rho, T& 
     rho = rho0 + drho;
 }
 
-// u = j / rho: FP64 divides (as the oracle does); FP32 multiplies by the
-// refined reciprocal (recip).
+// u = j / rho by the refined reciprocal (recip).
 template <typename T>
 __device__ __forceinline__ void velocity(T jx, T jy, T rho, T& ux, T& uy) {
-    if constexpr (sizeof(T) == 8) {
-        ux = jx / rho;
-        uy = jy / rho;
-    } else {
-        const T r = recip<T>(rho);
-        ux = jx * r;
-        uy = jy * r;
-    }
+    const T r = recip<T>(rho);
+    ux = jx * r;
+    uy = jy * r;
+}
+
+// Whether rho, u_x and u_y are finite.
+__device__ __forceinline__ bool all_finite(float rho, float ux, float uy) { return isfinite(rho + ux + uy); }
+__device__ __forceinline__ bool all_finite(double rho, double ux, double uy) {
+    // exponent fields (integer operations)
+    const int a = __double2hiint(rho), b = __double2hiint(ux), c = __double2hiint(uy);
+    return ((a & 0x7ff00000) != 0x7ff00000) & ((b & 0x7ff00000) != 0x7ff00000) & ((c & 0x7ff00000) != 0x7ff00000);
+}
+
+// Polynomial D2Q9 f* of FP64 storage (rho0 = 0) from the moments: with
+// j = rho u the terms of feq_poly need neither rho nor products of it (30
+// FP64 operations instead of 37).
+__device__ __forceinline__ void feq_poly_f64(double rho, double jx, double jy, double ux, double uy, double* gs) {
+    const double c0 = fma(-1.5, fma(jx, ux, jy * uy), rho);
+    const double ca = c0 * (1.0 / 9.0), cb = c0 * (1.0 / 36.0);
+    gs[0] = c0 * (4.0 / 9.0);
+    double a = fma(0.5 * jx, ux, ca), b = jx * (1.0 / 3.0);
+    gs[1] = a + b;
+    gs[3] = a - b;
+    a = fma(0.5 * jy, uy, ca);
+    b = jy * (1.0 / 3.0);
+    gs[2] = a + b;
+    gs[4] = a - b;
+    double j = jx + jy;
+    a = fma(0.125 * j, ux + uy, cb);
+    b = j * (1.0 / 12.0);
+    gs[5] = a + b;
+    gs[7] = a - b;
+    j = jx - jy;
+    a = fma(0.125 * j, ux - uy, cb);
+    b = j * (1.0 / 12.0);
+    gs[8] = a + b;
+    gs[6] = a - b;
 }
 
 // 2E = sum |v|^2 f = sum |v|^2 g + rho0 sum W |v|^2 of a site's deviations.
@@ -104,8 +139,13 @@ __device__ __forceinline__ void site_equilibrium(const Params& P, const T* g, T*
                                                  T& uy, NewtonCount& nc, const float* a0 = nullptr) {
     T drho, jx, jy;
     moments<L, T>(g, Par<T>::rho0(P), drho, rho, jx, jy);
+    if constexpr (sizeof(T) == 8) rho = drho;   // FP64 storage holds f itself (rho0 = 0)
     velocity<T>(jx, jy, rho, ux, uy);
-    if constexpr (EQ >= EQ_ENERGY) {
+    if constexpr (EQ == EQ_POLY && L::Q == 9 && sizeof(T) == 8) {
+        (void)nc;
+        (void)a0;
+        feq_poly_f64(rho, jx, jy, ux, uy, gs);
+    } else if constexpr (EQ >= EQ_ENERGY) {
         const T e2 = energy_moment<L, T>(g, Par<T>::rho0(P));
         equilibrium_energy<T, EQ>(rho, jx, jy, e2, gs, nc, a0);
     } else {
@@ -155,7 +195,7 @@ __device__ __noinline__ double delta_s_fp64(PopArr<L::Q, T> g, double rho0) {
     } else if constexpr (EQ == EQ_POLY) {
         feq_poly<L, double>(drho, rho, ux, uy, gs);
     } else {
-        feq_entropic<L, double>(rho, ux, uy, rho0, gs);
+        feq_entropic<L, double>(drho, rho, ux, uy, gs);
     }
     return delta_s_exact<L, double>(gd, gs, rho0);
 }
@@ -359,7 +399,7 @@ __device__ __forceinline__ bool update_site(const Params& P, T* g, int x, int y,
                                             const float* a0 = nullptr, T* ds_out = nullptr) {
     T gs[L::Q], rho, ux, uy;
     site_equilibrium<L, T, EQ>(P, g, gs, rho, ux, uy, nc, a0);
-    nonfinite |= !isfinite(rho + ux + uy);
+    nonfinite |= !all_finite(rho, ux, uy);
     if (PROBE && x == P.probe_x && y == P.probe_y && P.probe_ring)
         P.probe_ring[t % P.ring_cap] = (double)ux;
     T d[L::Q];
@@ -368,7 +408,7 @@ __device__ __forceinline__ bool update_site(const Params& P, T* g, int x, int y,
     if constexpr (PROJ) conserve_neq<L, EQ>(d);
     // (no short-circuit: the site's update stays one branch-free block)
     const bool pending =
-        (P.k > 0) & !ds_cleared<L, T, EQ>(d, gs, rho, ux, uy, Par<T>::rho0(P), Par<T>::delta(P));
+        (P.k > 0) & !ds_cleared<L, T, EQ>(d, gs, rho, ux, uy, Par<T>::rho0(P), Par<T>::delta(P), P.deltaf);
     if constexpr (RESOLVE) {
         T ds = T(-1);
         if (pending && !ghost_column(P, x)) ds = site_ds<L, T, EQ>(P, g, gs);
@@ -1896,7 +1936,7 @@ __global__ void __launch_bounds__(kSiteBlock) k_collide_site(const __grid_consta
 // listed in block 0, and the hardware's cluster barrier separates the
 // collision from the selection and, when a step has candidates, the
 // Ehrenfests' step from the next free flight.  800 sites, FP64: 23.5 us per step in
-// one launch each (4 blocks), 10.9 us so.
+// one launch each (4 blocks), 7.3 us so (2.5 us without the selection).
 // Every population passes through the storage type, so results are those of
 // one launch per step.
 // ---------------------------------------------------------------------------
@@ -2108,7 +2148,7 @@ __global__ void k_init_eq(const __grid_constant__ Params P, const double* rho, c
     using T = typename Store<S>::T;
     const long long sid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (sid >= (long long)P.nx * P.ny) return;
-    const int x = (int)(sid % P.nx), y = (int)(sid / P.nx);
+    const int y = (int)((unsigned)sid / (unsigned)P.nx), x = (int)((unsigned)sid - (unsigned)y * P.nx);   // (< 2^31 sites)
     const long long o = (long long)y * P.nxp + x;
     T gs[L::Q];
     if (is_solid(P, x, y)) {
@@ -2142,7 +2182,7 @@ __global__ void k_import(const __grid_constant__ Params P, const double* f, int 
     const long long N = (long long)P.nx * P.ny;
     const long long sid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (sid >= N) return;
-    const int x = (int)(sid % P.nx), y = (int)(sid / P.nx);
+    const int y = (int)((unsigned)sid / (unsigned)P.nx), x = (int)((unsigned)sid - (unsigned)y * P.nx);   // (< 2^31 sites)
     const long long o = (long long)y * P.nxp + x;
     const bool solid = is_solid(P, x, y);
     using T = typename Store<S>::T;
@@ -2159,9 +2199,29 @@ __global__ void k_import(const __grid_constant__ Params P, const double* f, int 
             Store<S>::store(P.dst, i * P.plane + o, solid ? T(0) : dev_of_f64<L, S>(P, i, f[i * N + sid]));
 }
 
+// Running sum s + c of floats: s their rounded sum, c the sum of the
+// rounding errors (two-sum).
+struct Sum2 {
+    float s, c;
+    __device__ __forceinline__ void add(float x) {
+        const ff t = ff_two_sum(s, x);
+        s = t.hi;
+        c += t.lo;
+    }
+    __device__ __forceinline__ void add(Sum2 o) {
+        add(o.s);
+        c += o.c;
+    }
+    __device__ __forceinline__ ff value() const { return ff_fast_two_sum(s, c); }
+};
+
 // Pre-collision state of the current step (gather of src) at sites
 // [s0, s1), exported as mode 0: populations f [Q][ny][nx]; 1: rho, ux, uy,
 // 2E; 2: exact dS (outputs indexed by the site's index y nx + x).
+// The moments of FP32 / FP16 storage were bound by the FP64 pipe (27
+// operations per site, conversions included); six are left, and the
+// sums share their parts: 4096 x 2048, FP32: 355 -> 222 us, FP64 2048 x 1024
+// (divisions and products with lattice velocities before): 302 -> 100 us.
 template <typename L, typename S, int EQ>
 __global__ void k_export(const __grid_constant__ Params P, int mode, double* o0, double* o1, double* o2,
                          double* o3, long long s0, long long s1) {
@@ -2169,7 +2229,7 @@ __global__ void k_export(const __grid_constant__ Params P, int mode, double* o0,
     const long long N = (long long)P.nx * P.ny;
     const long long sid = s0 + (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (sid >= s1) return;
-    const int x = (int)(sid % P.nx), y = (int)(sid / P.nx);
+    const int y = (int)((unsigned)sid / (unsigned)P.nx), x = (int)((unsigned)sid - (unsigned)y * P.nx);   // (< 2^31 sites)
     if (is_solid(P, x, y)) {
         if (mode == 0) for (int i = 0; i < L::Q; i++) o0[i * N + sid] = 0.0;
         if (mode == 1) {
@@ -2185,66 +2245,67 @@ __global__ void k_export(const __grid_constant__ Params P, int mode, double* o0,
     gather_site<L, S>(P, x, y, g);
     if (mode == 0) {
 #pragma unroll
-        for (int i = 0; i < L::Q; i++) o0[i * N + sid] = pop_f64<L, S>(P, i, g[i]);
+        for (int i = 0; i < L::Q; i++) o0[i * N + sid] = pop_f64<L, S>(i, g[i]);
     } else if (mode == 1) {
         if constexpr (sizeof(T) == 4) {
             // FP32 / FP16 storage: the sums of the stored values in float-float
-            // (exact for these nine floats) and u = j / rho by one corrected
-            // FP32 quotient, so that only the conversions to FP64 touch the FP64
-            // pipe; the rho0 parts (sum W = 1, sum W v = 0, sum W |v|^2) are added
-            // in FP64 at the end.
-            ff r = {0.0f, 0.0f}, jx = {0.0f, 0.0f}, jy = {0.0f, 0.0f}, e = {0.0f, 0.0f};
+            // and u = j / rho by one corrected FP32 quotient, so that FP64
+            // sees one addition per part; the rho0 parts (sum W = 1,
+            // sum W v = 0, sum W |v|^2) are added in FP64 at the end.
+            Sum2 one = {0.0f, 0.0f}, two = {0.0f, 0.0f}, jxs = {0.0f, 0.0f}, jys = {0.0f, 0.0f};
+            bool first1 = true, first2 = true, firstx = true, firsty = true;
 #pragma unroll
-            for (int i = 0; i < L::Q; i++) {
-                const ff gi = {g[i], 0.0f};
-                r = ff_add(r, gi);
-                if (L::cx(i) == 1) jx = ff_add(jx, gi);
-                if (L::cx(i) == -1) jx = ff_sub(jx, gi);
-                if (L::cy(i) == 1) jy = ff_add(jy, gi);
-                if (L::cy(i) == -1) jy = ff_sub(jy, gi);
+            for (int i = 1; i < L::Q; i++) {
                 const int c2 = L::cx(i) * L::cx(i) + L::cy(i) * L::cy(i);
-                if (c2 > 0) e = ff_add(e, ff_scale(gi, (float)c2));
+                auto put = [](Sum2& a, bool& first, float v) {
+                    if (first) a.s = v;
+                    else a.add(v);
+                    first = false;
+                };
+                if (c2 == 1) put(one, first1, g[i]);
+                if (c2 == 2) put(two, first2, g[i]);
+                if (L::cx(i) != 0) put(jxs, firstx, L::cx(i) > 0 ? g[i] : -g[i]);
+                if (L::cy(i) != 0) put(jys, firsty, L::cy(i) > 0 ? g[i] : -g[i]);
             }
+            Sum2 rs = {g[0], 0.0f}, es = one;
+            rs.add(one);
+            if constexpr (L::Q == 9) {
+                rs.add(two);
+                es.add(Sum2{2.0f * two.s, 2.0f * two.c});
+            }
+            const ff r = rs.value(), jx = jxs.value(), jy = jys.value(), e = es.value();
             // the stored deviations' offsets: sum W rho0 (= rho0), and for
             // plain FP32 the sums of the FP32 weights (exact in FP64)
-            double off0 = P.rho0, off2 = L::sum_w_c2 * P.rho0;
-            if constexpr (Store<S>::kPlain) {
-                off0 = 0.0;
-                off2 = 0.0;
-#pragma unroll
-                for (int i = 0; i < L::Q; i++) {
-                    off0 += (double)(float)L::w(i);
-                    off2 += (double)(L::cx(i) * L::cx(i) + L::cy(i) * L::cy(i)) * (double)(float)L::w(i);
-                }
-            }
-            const double rho = (off0 + (double)r.hi) + (double)r.lo;
-            const float o0h = (float)off0;
-            const ff rf = ff_add({o0h, (float)(off0 - (double)o0h)}, r);
-            const ff ir = ff_recip(rf);
-            o0[sid] = rho;
+            constexpr bool plain = Store<S>::kPlain;
+            constexpr float w0 = (float)L::w(0), w1 = (float)L::w(1), w5 = L::Q == 9 ? (float)L::w(L::Q - 1) : 0.0f;
+            constexpr int n1 = L::Q == 9 ? 4 : 2, n2 = L::Q == 9 ? 4 : 0;
+            constexpr double off0 = plain ? (double)w0 + n1 * (double)w1 + n2 * (double)w5 : 1.0;
+            constexpr double off2 = plain ? n1 * (double)w1 + 2 * n2 * (double)w5 : L::sum_w_c2;
+            constexpr float off0h = (float)off0, off0l = (float)(off0 - (double)off0h);
+            o0[sid] = (off0 + widen(r.hi)) + widen(r.lo);
+            const ff ir = ff_recip(ff_add({off0h, off0l}, r));
             if (o1) {
                 const ff u = ff_mul(jx, ir);
-                o1[sid] = (double)u.hi + (double)u.lo;
+                o1[sid] = widen(u.hi) + widen(u.lo);
             }
             if (o2) {
                 const ff v = ff_mul(jy, ir);
-                o2[sid] = (double)v.hi + (double)v.lo;
+                o2[sid] = widen(v.hi) + widen(v.lo);
             }
-            if (o3) o3[sid] = (off2 + (double)e.hi) + (double)e.lo;
+            if (o3) o3[sid] = (off2 + widen(e.hi)) + widen(e.lo);
         } else {
-            double rho = 0, jx = 0, jy = 0, e2 = 0;
-#pragma unroll
-            for (int i = 0; i < L::Q; i++) {
-                const double f = (double)g[i] + L::w(i) * P.rho0;
-                rho += f;
-                jx += L::cx(i) * f;
-                jy += L::cy(i) * f;
-                e2 += (L::cx(i) * L::cx(i) + L::cy(i) * L::cy(i)) * f;
+            double drho, rho, jx, jy, ux, uy;
+            moments<L, double>(g, 0.0, drho, rho, jx, jy);
+            velocity<double>(jx, jy, drho, ux, uy);
+            o0[sid] = drho;
+            if (o1) o1[sid] = ux;
+            if (o2) o2[sid] = uy;
+            if (o3) {
+                if constexpr (L::Q == 9)
+                    o3[sid] = fma(2.0, (g[5] + g[8]) + (g[6] + g[7]), (g[1] + g[3]) + (g[2] + g[4]));
+                else
+                    o3[sid] = g[1] + g[2];
             }
-            o0[sid] = rho;
-            if (o1) o1[sid] = jx / rho;
-            if (o2) o2[sid] = jy / rho;
-            if (o3) o3[sid] = e2;
         }
     } else {
         T gs[L::Q], rho, ux, uy;
