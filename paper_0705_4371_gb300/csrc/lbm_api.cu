@@ -47,27 +47,30 @@ constexpr int kTubeSteps = 4096;     // steps of a short D1Q3 run per launch
 constexpr int kExportChunks = 8;     // row chunks of a host export (copies overlap the conversion)
 constexpr int kXferEvents = 16;      // events of one chunked transfer (>= Q planes, >= chunks, + 1)
 constexpr int kDefaultLog = 65536;
-// Default tile shapes, the fastest measured on GB300: FP32 and FP16 storage
-// (plain and deviation) stage 6-row tiles with 2 more in flight per block
-// (shape 5; FP16 at 1000 steps of the 4096 x 2048 cylinder: 90.8 k MLUPS
-// against 86.8 k with 8-row tiles at three blocks per SM); FP64 storage
-// 8-row tiles with 1 more (shape 4).  Small polynomial-f* FP32 grids (up to 600 000 sites:
-// one or two staged tiles per resident block, a step of ~20 us dominated by
-// latency) run faster register-fed (shape 1): the 600 x 500 channel 15.7 k
-// against 13.0 k MLUPS, 1024 x 512 23.2 k against 22.2 k; from 1536 x 768
-// on shape 5 is ahead (34.3 k against 31.1 k), and FP16 storage is fastest
-// on shape 5 at every size measured.  The energy forms: FP64 storage's FP64
+// Default tile shapes by measurement on GB300 (us per step of two runs side by
+// side).  Up to 600 000 sites (one or two tiles per resident block, a step
+// dominated by latency): register-fed tiles for polynomial-f* FP32 (shape 1;
+// alone 600 x 500 takes 13.4 us, 12.7 - 14.3 staged), 6-row staged tiles for
+// the others (shape 5; FP16 500 x 256: 7.1 against 8.6 on shape 4).  Above,
+// the 8-row tiles' warps win wherever arithmetic is what bounds a step (shape
+// 4; 4096 x 2048: entropic FP32 115 against 131; 2048 x 1024 ELBM 91 against
+// 125) and, less, where memory does (polynomial FP32: 94 against 97 at
+// 4096 x 2048, 13.1 against 14.3 at 1280 x 640; between 600 000 and 800 000
+// sites it keeps shape 5).  FP16 gains from 1e6 sites on (1024 x 600: 10.7
+// against 9.4; 2048 x 1024: 20 against 24; 4096 x 2048: 68 against 84).
+// FP64 storage: 8-row tiles.  The energy forms: FP64 storage's
 // solve wants the most resident warps (register-fed shape 1); the
 // float-float solve of FP32 / FP16 storage and the network's warm start run
 // best in the staged shape 4 (measured at 2048 x 1024: Newton start 89 us
 // per step against 235 on shape 0 and 93 on shape 5; warm start 211 against
 // 263 and 233).
-int default_tile_shape(int lattice, int eq, int precision, long long sites) {
+int default_tile_shape(int lattice, int eq, int precision, long long sites, bool elbm) {
     if (lattice != LB_D2Q9) return 0;
     if (eq < LB_EQ_ENTROPIC_ENERGY) {
-        if (precision == LB_F64) return 4;
-        if (eq == LB_EQ_POLY && precision != LB_F16_DEV && sites <= 600000) return 1;
-        return 5;
+        if (precision == LB_F64 || elbm) return 4;
+        if (precision == LB_F16_DEV) return sites <= 1000000 ? 5 : 4;
+        if (eq == LB_EQ_POLY && sites <= 600000) return 1;
+        return sites <= (eq == LB_EQ_POLY ? 800000 : 600000) ? 5 : 4;
     }
     if (precision == LB_F64) return 1;
     return 4;
@@ -166,6 +169,7 @@ struct lb_handle {
     unsigned* ticket;
     int tile_shape;
     int grid_blocks, sm_count, blocks_per_sm;
+    bool shape_set;           // the caller chose the tile shape
     bool tube;                // short D1Q3 run: many steps per cluster launch
     // tensor maps of the two population buffers (shared-memory-staged shapes)
     CUtensorMap tmap[2];
@@ -413,6 +417,13 @@ int size_grid(lb_handle* h) {
     return LB_OK;
 }
 
+// Take a tile shape (the run's stream is idle, its graphs are dropped).
+int use_tile_shape(lb_handle* h, int shape) {
+    h->tile_shape = shape;
+    const int rc = size_grid(h);
+    return rc != LB_OK ? rc : make_tensor_maps(h);
+}
+
 }  // namespace
 
 // ---------------------------------------------------------------------------
@@ -565,7 +576,7 @@ int lb_create(int lattice, int nx, int ny, int equilibrium, double nu, double de
     h->bc = b;
     h->plane = (long long)ny * h->nxp;
     h->probe_x = h->probe_y = -1;
-    h->tile_shape = default_tile_shape(lattice, equilibrium, precision, (long long)nx * ny);
+    h->tile_shape = default_tile_shape(lattice, equilibrium, precision, (long long)nx * ny, false);
     h->ring_cap = kDefaultLog;
     h->replay_t0 = -1;
     if (precision == LB_F64) h->L = launchers_f64(lattice, equilibrium);
@@ -1038,6 +1049,8 @@ int lb_set_collision(lb_handle* h, int collision) {
     CK(cudaStreamSynchronize(h->stream));
     h->elbm = collision == LB_COLLISION_ELBM;
     drop_graphs(h);
+    const int shape = default_tile_shape(h->lattice, h->eq, h->prec, (long long)h->nx * h->ny, h->elbm);
+    if (!h->shape_set && shape != h->tile_shape) return use_tile_shape(h, shape);
     return LB_OK;
 }
 
@@ -1108,11 +1121,10 @@ int lb_set_tile_shape(lb_handle* h, int shape) {
     if (shape == 6 && h->eq >= LB_EQ_ENTROPIC_ENERGY)
         return fail(LB_ERR_ARG, "the energy forms take tile shapes 0-5");
     CK(cudaStreamSynchronize(h->stream));
-    h->tile_shape = shape;
     drop_graphs(h);
-    const int rc = size_grid(h);
-    if (rc != LB_OK) return rc;
-    return make_tensor_maps(h);
+    const int rc = use_tile_shape(h, shape);
+    if (rc == LB_OK) h->shape_set = true;
+    return rc;
 }
 
 // ---------------------------------------------------------------------------
