@@ -62,8 +62,8 @@ constexpr int kDefaultLog = 65536;
 // solve wants the most resident warps (register-fed shape 1); the
 // float-float solve of FP32 / FP16 storage and the network's warm start run
 // best in the staged shape 4 (measured at 2048 x 1024: Newton start 89 us
-// per step against 235 on shape 0 and 93 on shape 5; warm start 211 against
-// 263 and 233).
+// per step against 235 on shape 0 and 93 on shape 5; warm start 131 against
+// 209 on shape 5).
 int default_tile_shape(int lattice, int eq, int precision, long long sites, bool elbm) {
     if (lattice != LB_D2Q9) return 0;
     if (eq < LB_EQ_ENTROPIC_ENERGY) {

@@ -37,15 +37,13 @@ __device__ __forceinline__ void equilibrium(const Params& P, T drho, T rho, T ux
 }
 
 // Energy-constrained entropic f* (D2Q9 only) as deviations from the
-// moments (drho, j, 2E); Newton from the start point a0 (the network's
-// warm start in the learned form) or, when a0 is null, from the polynomial
-// start point (3 u_x, 3 u_y, 0) (the multipliers of the first-order
-// expansion about rest).  The momentum multipliers are eliminated in closed
-// form, so only the energy multiplier's start enters the iteration.
+// moments (drho, j, 2E); Newton from the energy multiplier's start mu3 (the
+// network's warm start in the learned form, else 0: the polynomial start
+// point (3 u_x, 3 u_y, 0), the multipliers of the first-order expansion about
+// rest; the momentum multipliers follow in closed form).
 template <typename T, int EQ>
 __device__ __forceinline__ void equilibrium_energy(T rho, T jx, T jy, T e2, T* gs, NewtonCount& nc,
-                                                   const float* a0 = nullptr) {
-    const float mu3 = a0 ? a0[2] : 0.0f;
+                                                   float mu3 = 0.0f) {
     if constexpr (sizeof(T) == 4) {
         // FP32 / FP16 storage: the float-float finish (no FP64 work)
         energy_solve_ff(rho, jx, jy, e2, mu3, gs, nc);
@@ -132,25 +130,25 @@ __device__ __forceinline__ T energy_moment(const T* g, T rho0) {
 }
 
 // Quasiequilibrium of a gathered site (shared by the collision, the
-// Ehrenfests' step and the exports so that all round identically).  a0:
-// Newton start point of the energy forms (null: the polynomial start).
+// Ehrenfests' step and the exports so that all round identically).  mu3:
+// start of the energy forms' multiplier (0: the polynomial start).
 template <typename L, typename T, int EQ>
 __device__ __forceinline__ void site_equilibrium(const Params& P, const T* g, T* gs, T& rho, T& ux,
-                                                 T& uy, NewtonCount& nc, const float* a0 = nullptr) {
+                                                 T& uy, NewtonCount& nc, float mu3 = 0.0f) {
     T drho, jx, jy;
     moments<L, T>(g, Par<T>::rho0(P), drho, rho, jx, jy);
     if constexpr (sizeof(T) == 8) rho = drho;   // FP64 storage holds f itself (rho0 = 0)
     velocity<T>(jx, jy, rho, ux, uy);
     if constexpr (EQ == EQ_POLY && L::Q == 9 && sizeof(T) == 8) {
         (void)nc;
-        (void)a0;
+        (void)mu3;
         feq_poly_f64(rho, jx, jy, ux, uy, gs);
     } else if constexpr (EQ >= EQ_ENERGY) {
         const T e2 = energy_moment<L, T>(g, Par<T>::rho0(P));
-        equilibrium_energy<T, EQ>(rho, jx, jy, e2, gs, nc, a0);
+        equilibrium_energy<T, EQ>(rho, jx, jy, e2, gs, nc, mu3);
     } else {
         (void)nc;
-        (void)a0;
+        (void)mu3;
         equilibrium<L, T, EQ>(P, drho, rho, ux, uy, gs);
     }
 }
@@ -396,9 +394,9 @@ __device__ __forceinline__ bool ghost_column(const Params& P, int x) {
 template <typename L, typename T, int EQ, bool PROJ, bool PROBE = true, bool RESOLVE = false>
 __device__ __forceinline__ bool update_site(const Params& P, T* g, int x, int y, long long t,
                                             bool& nonfinite, NewtonCount& nc,
-                                            const float* a0 = nullptr, T* ds_out = nullptr) {
+                                            float mu3 = 0.0f, T* ds_out = nullptr) {
     T gs[L::Q], rho, ux, uy;
-    site_equilibrium<L, T, EQ>(P, g, gs, rho, ux, uy, nc, a0);
+    site_equilibrium<L, T, EQ>(P, g, gs, rho, ux, uy, nc, mu3);
     nonfinite |= !all_finite(rho, ux, uy);
     if (PROBE && x == P.probe_x && y == P.probe_y && P.probe_ring)
         P.probe_ring[t % P.ring_cap] = (double)ux;
@@ -432,11 +430,23 @@ __device__ __forceinline__ bool update_site(const Params& P, T* g, int x, int y,
     return pending;
 }
 
-// Learned form: the network's Newton start point for the warp's 32 sites
-// (lane l: its gathered site g, or valid = false).  Every lane must call it.
+// Shared copy of the network in the learned form's kernels (empty otherwise).
+template <int EQ> struct MlpSlot {
+    __device__ void fill(const Params&) {}
+};
+template <> struct MlpSlot<EQ_ENERGY_MLP> {
+    MlpSmemQ s;
+    __device__ void fill(const Params& P) {
+        mlp_fill(s, P.mlp);
+        mlp_fill_quads(s, P.mlp);
+    }
+};
+
+// Learned form: the network's start of the energy multiplier for the warp's
+// 32 sites (lane l: its gathered site g, or valid = false).  Every lane must
+// call it.
 template <typename T>
-__device__ __forceinline__ void mlp_site_start(const Params& P, const MlpSmem& ms, bool valid,
-                                               const T* g, float* a) {
+__device__ __forceinline__ float mlp_site_start(const Params& P, const MlpSmemQ& ms, bool valid, const T* g) {
     float rho = 1.0f, ux = 0.0f, uy = 0.0f, e2 = 0.0f;
     if (valid) {
         T drho, r, jx, jy;
@@ -448,17 +458,8 @@ __device__ __forceinline__ void mlp_site_start(const Params& P, const MlpSmem& m
         e2 = (float)energy_moment<D2Q9, T>(g, Par<T>::rho0(P));
         valid = rho > 0.0f && isfinite(rho + ux + uy + e2);
     }
-    mlp_warm_start(ms, valid, rho, ux, uy, e2, a);
+    return mlp_start(ms, rho, ux, uy, e2, valid);
 }
-
-// Shared copy of the network in the learned form's kernels (empty otherwise).
-template <int EQ> struct MlpSlot {
-    __device__ void fill(const Params&) {}
-};
-template <> struct MlpSlot<EQ_ENERGY_MLP> {
-    MlpSmem s;
-    __device__ void fill(const Params& P) { mlp_fill(s, P.mlp); }
-};
 
 // Exact dS of site (x, y) with the pre-collision state re-gathered from the
 // source field (not written during a step); -1 on a slab's ghost column.
@@ -1102,11 +1103,10 @@ __global__ void __launch_bounds__(32 * WARPS, MINB) k_collide_d2q9(const __grid_
 #pragma unroll
             for (int s = 0; s < VEC; s++) {
                 NewtonCount one = nc;
-                float a0[3];
-                if constexpr (EQ == EQ_ENERGY_MLP) mlp_site_start<T>(P, mslot.s, true, g[s], a0);
+                float mu3 = 0.0f;
+                if constexpr (EQ == EQ_ENERGY_MLP) mu3 = mlp_site_start<T>(P, mslot.s, true, g[s]);
                 const bool p = update_site<L, T, EQ, Store<S>::kProject>(P, g[s], (fluid >> s) & 1u ? xs + s : -2, y, t,
-                                                                         nonfinite, one,
-                                                                         EQ == EQ_ENERGY_MLP ? a0 : nullptr);
+                                                                         nonfinite, one, mu3);
                 if ((fluid >> s) & 1u) {
                     nc = one;
                     if (p) pend |= 1u << s;
@@ -1402,18 +1402,14 @@ __device__ __noinline__ TileState<Sink> tma_tile_general(const Params& P, const 
             } else {
                 gather_site_smem<S, R, TX>(P, box, x0, y0, x, y, g);
             }
+            float mu3 = 0.0f;
             if constexpr (EQ == EQ_ENERGY_MLP) {
-                float a0[3];
                 __syncwarp();
-                mlp_site_start<T>(P, mslot.s, fluid, g, a0);
-                if (fluid)
-                    update_site<L, T, EQ, Store<S>::kProject, true, true>(P, g, x, y, t, state.nonfinite, state.nc,
-                                                                          a0, &ds);
-            } else {
-                if (fluid)
-                    update_site<L, T, EQ, Store<S>::kProject, true, true>(P, g, x, y, t, state.nonfinite, state.nc,
-                                                                          nullptr, &ds);
+                mu3 = mlp_site_start<T>(P, mslot.s, fluid, g);
             }
+            if (fluid)
+                update_site<L, T, EQ, Store<S>::kProject, true, true>(P, g, x, y, t, state.nonfinite, state.nc, mu3,
+                                                                      &ds);
             if (inside) {
 #pragma unroll
                 for (int i = 0; i < L::Q; i++)
@@ -1451,16 +1447,10 @@ __device__ __noinline__ TileState<Sink> edge_item(const Params& P, int item, lon
         for (int i = 0; i < L::Q; i++) g[i] = T(0);
     }
     T ds = T(-1);
-    if constexpr (EQ == EQ_ENERGY_MLP) {
-        float a0[3];
-        mlp_site_start<T>(P, mslot.s, fluid, g, a0);
-        if (fluid)
-            update_site<L, T, EQ, Store<S>::kProject, true, true>(P, g, x, y, t, state.nonfinite, state.nc, a0, &ds);
-    } else {
-        if (fluid)
-            update_site<L, T, EQ, Store<S>::kProject, true, true>(P, g, x, y, t, state.nonfinite, state.nc, nullptr,
-                                                                  &ds);
-    }
+    float mu3 = 0.0f;
+    if constexpr (EQ == EQ_ENERGY_MLP) mu3 = mlp_site_start<T>(P, mslot.s, fluid, g);
+    if (fluid)
+        update_site<L, T, EQ, Store<S>::kProject, true, true>(P, g, x, y, t, state.nonfinite, state.nc, mu3, &ds);
     if (inside) {
         S* dst = static_cast<S*>(P.dst);
         const long long o = (long long)y * P.nxp + x;
@@ -1687,22 +1677,16 @@ __device__ __forceinline__ void tma_tile(const Params& P, S* box, int x0, int y0
         bool pa, pb;
         // (the sites that are not the row's do not count as solved)
         NewtonCount na = state.nc;
+        float ma = 0.0f, mb = 0.0f;
         if constexpr (EQ == EQ_ENERGY_MLP) {
-            float a0[3];
-            mlp_site_start<T>(P, mslot.s, true, ga, a0);
-            pa = update_site<L, T, EQ, Store<S>::kProject, false>(P, ga, x0 + c, y, t, state.nonfinite, na, a0);
-            if (!ea) state.nc = na;
-            na = state.nc;
-            mlp_site_start<T>(P, mslot.s, true, gb, a0);
-            pb = update_site<L, T, EQ, Store<S>::kProject, false>(P, gb, x0 + c + 1, y, t, state.nonfinite, na, a0);
-            if (!eb) state.nc = na;
-        } else {
-            pa = update_site<L, T, EQ, Store<S>::kProject, false>(P, ga, x0 + c, y, t, state.nonfinite, na);
-            if (EQ >= EQ_ENERGY && !ea) state.nc = na;
-            na = state.nc;
-            pb = update_site<L, T, EQ, Store<S>::kProject, false>(P, gb, x0 + c + 1, y, t, state.nonfinite, na);
-            if (EQ >= EQ_ENERGY && !eb) state.nc = na;
+            ma = mlp_site_start<T>(P, mslot.s, true, ga);
+            mb = mlp_site_start<T>(P, mslot.s, true, gb);
         }
+        pa = update_site<L, T, EQ, Store<S>::kProject, false>(P, ga, x0 + c, y, t, state.nonfinite, na, ma);
+        if (EQ >= EQ_ENERGY && !ea) state.nc = na;
+        na = state.nc;
+        pb = update_site<L, T, EQ, Store<S>::kProject, false>(P, gb, x0 + c + 1, y, t, state.nonfinite, na, mb);
+        if (EQ >= EQ_ENERGY && !eb) state.nc = na;
         if (!(ea | eb)) {
 #pragma unroll
             for (int i = 0; i < L::Q; i++)
@@ -2029,7 +2013,7 @@ __global__ void __launch_bounds__(kTubeThreads) k_tube(const __grid_constant__ P
                     }
                 }
             }
-            update_site<L, T, EQ, Store<S>::kProject, true, true>(P, g, x, 0, t, nonfinite, nc, nullptr, &ds);
+            update_site<L, T, EQ, Store<S>::kProject, true, true>(P, g, x, 0, t, nonfinite, nc, 0.0f, &ds);
 #pragma unroll
             for (int i = 0; i < L::Q; i++) Store<S>::store(nxt + i * per + tid, 0, store_round<L, S>(i, g[i]));
         }

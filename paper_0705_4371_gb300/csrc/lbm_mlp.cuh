@@ -204,30 +204,116 @@ __device__ __forceinline__ void mlp_warp_forward(const MlpSmem& s, unsigned p01,
     }
 }
 
-// Warm start of the energy Newton solve: multipliers a = (mu_x, mu_y, mu_c)
-// of the normalised form from the network, for the warp's 32 sites (every
-// lane calls; valid = false lanes get the polynomial start).  Outputs that
-// are not finite or implausibly large (|a| > 8) fall back to the polynomial
-// start.
-__device__ __forceinline__ void mlp_warm_start(const MlpSmem& s, bool valid, float rho, float ux,
-                                               float uy, float e2, float* a) {
-    const float th = valid ? e2 / rho - ux * ux - uy * uy : 0.0f;
-    unsigned p01 = 0u, p23 = 0u;
-    if (valid) mlp_inputs(s, rho, ux, uy, th, p01, p23);
-    float y[kMlpOut] = {0.0f, 0.0f, 0.0f, 0.0f};
-    mlp_warp_forward(s, p01, p23, y);
-    a[0] = 3.0f * ux;
-    a[1] = 3.0f * uy;
-    a[2] = 0.0f;
-    if (!valid) return;
-    const float c0 = a[0] + s.oscale[1] * y[1];
-    const float c1 = a[1] + s.oscale[2] * y[2];
-    const float c2 = s.oscale[3] * y[3];
-    if (fabsf(c0) <= 8.0f && fabsf(c1) <= 8.0f && fabsf(c2) <= 8.0f) {   // false for NaN
-        a[0] = c0;
-        a[1] = c1;
-        a[2] = c2;
+// The network as the collide kernels hold it: the biases also as
+// accumulator fragments (quad t of n-tile nt: columns 8 nt + 2 t, + 1 of both
+// row halves).
+struct MlpSmemQ : MlpSmem {
+    float4 q1[8][4], q2[8][4];
+};
+
+__device__ __forceinline__ void mlp_fill_quads(MlpSmemQ& s, const float* __restrict__ p) {
+    for (int e = threadIdx.x; e < 32; e += blockDim.x) {
+        const int nt = e >> 2, t = e & 3, c = 8 * nt + 2 * t;
+        s.q1[nt][t] = make_float4(p[kMlpB1 + c], p[kMlpB1 + c + 1], p[kMlpB1 + c], p[kMlpB1 + c + 1]);
+        s.q2[nt][t] = make_float4(p[kMlpB2 + c], p[kMlpB2 + c + 1], p[kMlpB2 + c], p[kMlpB2 + c + 1]);
     }
+}
+
+// D = A B + C, as mma_bf16, with an accumulator input of its own.
+__device__ __forceinline__ void mma_bf16_from(float* d, float4 c, unsigned a0, unsigned a1, unsigned a2, unsigned a3,
+                                              unsigned b0, unsigned b1) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 "
+        "{%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%10, %11, %12, %13};"
+        : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(c.x), "f"(c.y), "f"(c.z), "f"(c.w));
+}
+
+// Warm start of the energy Newton solve for the warp's 32 sites (lane l: one
+// site's rho, u, 2E): the energy multiplier mu_3 of the network's prediction
+// (mu_1 and mu_2 follow from it in closed form).  Lanes without a valid site
+// and predictions that are not finite or implausibly large (some |mu| > 8)
+// get the polynomial start, 0.  Every lane of the warp must call it.
+// Bound by the tensor pipe: 88 MMAs per warp at 8.7 cycles each per SM
+// quarter.  Both 16-site tiles of the warp take every weight fragment as it
+// is read (one shared-memory read for two MMAs), the biases enter as the first
+// MMA's accumulators without a move, and the routine is out of line: inlined
+// in the update twice it spilled 860 bytes per thread.  2048 x 1024: the
+// network's share of a step 119 -> 62 us.
+static __device__ __noinline__ float mlp_start(const MlpSmemQ& s, float rho, float ux, float uy, float e2, bool valid) {
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31, g = lane >> 2, tig = lane & 3;
+    unsigned p01 = 0u, p23 = 0u;
+    if (valid) mlp_inputs(s, rho, ux, uy, e2 / rho - ux * ux - uy * uy, p01, p23);
+    unsigned a[2][2];   // input columns 2 tig, 2 tig + 1 of rows g and g + 8 of tile m
+#pragma unroll
+    for (int m = 0; m < 2; m++)
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+            const int r = 16 * m + 8 * h + g;
+            const unsigned lo = __shfl_sync(FULL, p01, r), hi = __shfl_sync(FULL, p23, r);
+            a[m][h] = tig == 0 ? lo : (tig == 1 ? hi : 0u);
+        }
+    unsigned A2[2][4][4];
+#pragma unroll
+    for (int nt = 0; nt < 8; nt++) {
+        const unsigned w = s.w1[nt][lane];
+        const float4 b = s.q1[nt][tig];
+#pragma unroll
+        for (int m = 0; m < 2; m++) {
+            float c[4];
+            mma_bf16_from(c, b, a[m][0], a[m][1], 0u, 0u, w, 0u);
+            A2[m][nt >> 1][(nt & 1) * 2 + 0] = bf16_pack_relu(c[0], c[1]);
+            A2[m][nt >> 1][(nt & 1) * 2 + 1] = bf16_pack_relu(c[2], c[3]);
+        }
+    }
+    float yc[2][4];
+#pragma unroll
+    for (int m = 0; m < 2; m++) {
+        yc[m][0] = yc[m][2] = s.b3[2 * tig];
+        yc[m][1] = yc[m][3] = s.b3[2 * tig + 1];
+    }
+#pragma unroll
+    for (int jp = 0; jp < 4; jp++) {
+        unsigned A3[2][4];
+#pragma unroll
+        for (int hh = 0; hh < 2; hh++) {
+            const int nt = 2 * jp + hh;
+            const float4 b = s.q2[nt][tig];
+            float c[2][4];
+#pragma unroll
+            for (int j = 0; j < 4; j++) {
+                const uint2 w = s.w2[nt][j][lane];
+#pragma unroll
+                for (int m = 0; m < 2; m++) {
+                    if (j == 0) mma_bf16_from(c[m], b, A2[m][j][0], A2[m][j][1], A2[m][j][2], A2[m][j][3], w.x, w.y);
+                    else mma_bf16(c[m], A2[m][j][0], A2[m][j][1], A2[m][j][2], A2[m][j][3], w.x, w.y);
+                }
+            }
+#pragma unroll
+            for (int m = 0; m < 2; m++) {
+                A3[m][2 * hh] = bf16_pack_relu(c[m][0], c[m][1]);
+                A3[m][2 * hh + 1] = bf16_pack_relu(c[m][2], c[m][3]);
+            }
+        }
+        const uint2 w = s.w3[jp][lane];
+#pragma unroll
+        for (int m = 0; m < 2; m++) mma_bf16(yc[m], A3[m][0], A3[m][1], A3[m][2], A3[m][3], w.x, w.y);
+    }
+    // outputs 1 .. 3 to the site's lane, as in mlp_warp_forward
+    float y[kMlpOut];
+#pragma unroll
+    for (int j = 1; j < kMlpOut; j++) {
+        const int src = 4 * (lane & 7) + (j >> 1);
+#pragma unroll
+        for (int m = 0; m < 2; m++) {
+            const float lo = __shfl_sync(FULL, yc[m][j & 1], src);
+            const float hi = __shfl_sync(FULL, yc[m][2 + (j & 1)], src);
+            if ((lane >> 4) == m) y[j] = (lane & 8) ? hi : lo;
+        }
+    }
+    const float c0 = 3.0f * ux + s.oscale[1] * y[1], c1 = 3.0f * uy + s.oscale[2] * y[2], c2 = s.oscale[3] * y[3];
+    return valid && fabsf(c0) <= 8.0f && fabsf(c1) <= 8.0f && fabsf(c2) <= 8.0f ? c2 : 0.0f;   // (false for NaN)
 }
 
 }  // namespace lbm
