@@ -354,15 +354,19 @@ __device__ __noinline__ T elbm_factor(PopArr<L::Q, T> g, PopArr<L::Q, T> gs, T r
 // Returns dS in T (NaN for a non-finite state).  Out of line: the sites the
 // bound does not clear are few, and the update path keeps its registers.
 template <typename L, typename T, int EQ>
-__device__ __noinline__ T resolved_ds(PopArr<L::Q, T> g, PopArr<L::Q, T> gs, T rho0, T dl, double delta,
-                                      double rho0d, double band, int recheck) {
-    T ds = delta_s_exact<L, T>(g.v, gs.v, rho0);
+__device__ __forceinline__ T recheck_ds(const PopArr<L::Q, T>& g, T ds, T dl, double delta, double rho0d, double band,
+                                        int recheck) {
     if (recheck && isfinite(ds) && fabs((double)ds - delta) <= band) {
         const double d64 = delta_s_fp64<L, T, EQ>(g, rho0d);
         if (d64 > delta) ds = (T)d64 > dl ? (T)d64 : nextafter(dl, T(INFINITY));
         else ds = T(-1);
     }
     return ds;
+}
+template <typename L, typename T, int EQ>
+__device__ __noinline__ T resolved_ds(PopArr<L::Q, T> g, PopArr<L::Q, T> gs, T rho0, T dl, double delta,
+                                      double rho0d, double band, int recheck) {
+    return recheck_ds<L, T, EQ>(g, delta_s_exact<L, T>(g.v, gs.v, rho0), dl, delta, rho0d, band, recheck);
 }
 
 // The same from the site's pre-collision deviations g and quasiequilibrium
@@ -390,16 +394,21 @@ __device__ __forceinline__ bool ghost_column(const Params& P, int x) {
 // the storage's rounding (store_round).  RESOLVE: a site the bound does not
 // clear has its dS evaluated here, from the pre-collision g and f* at hand
 // (site_ds), and stored to *ds_out (-1 for every other site, and for a
-// slab's ghost columns).
+// slab's ghost columns).  gs_out (optional): f*, for a caller that resolves
+// the site itself.
 template <typename L, typename T, int EQ, bool PROJ, bool PROBE = true, bool RESOLVE = false>
 __device__ __forceinline__ bool update_site(const Params& P, T* g, int x, int y, long long t,
                                             bool& nonfinite, NewtonCount& nc,
-                                            float mu3 = 0.0f, T* ds_out = nullptr) {
+                                            float mu3 = 0.0f, T* ds_out = nullptr, T* gs_out = nullptr) {
     T gs[L::Q], rho, ux, uy;
     site_equilibrium<L, T, EQ>(P, g, gs, rho, ux, uy, nc, mu3);
     nonfinite |= !all_finite(rho, ux, uy);
     if (PROBE && x == P.probe_x && y == P.probe_y && P.probe_ring)
         P.probe_ring[t % P.ring_cap] = (double)ux;
+    if (gs_out) {
+#pragma unroll
+        for (int i = 0; i < L::Q; i++) gs_out[i] = gs[i];
+    }
     T d[L::Q];
 #pragma unroll
     for (int i = 0; i < L::Q; i++) d[i] = g[i] - gs[i];
@@ -1916,11 +1925,14 @@ __global__ void __launch_bounds__(kSiteBlock) k_collide_site(const __grid_consta
 // chain -- launch, loads, the FP64 update (two FP64 operations per SM and
 // clock), the exact dS of the sites near the front, the selection -- so the
 // state stays in the shared memory of a cluster of 16 blocks (16 SMs' FP64
-// pipes), neighbours read each other's edge sites there, the candidates are
-// listed in block 0, and the hardware's cluster barrier separates the
-// collision from the selection and, when a step has candidates, the
-// Ehrenfests' step from the next free flight.  800 sites, FP64: 23.5 us per step in
-// one launch each (4 blocks), 7.3 us so (2.5 us without the selection).
+// pipes), neighbours read each other's edge sites there, every block lists its
+// candidates, and the hardware's cluster barrier separates the collision from
+// the selection and, when a step has candidates, the Ehrenfests' step from
+// the next free flight.  The exact dS of a warp's pending sites takes a lane
+// per population (its series and logarithms are the longest FP64 chain of a
+// step), and a candidate's f* is evaluated while the barrier completes.
+// 800 sites, FP64: 23.5 us per step in one launch each (4 blocks), 5.9 us so
+// (2.5 us without the selection).
 // Every population passes through the storage type, so results are those of
 // one launch per step.
 // ---------------------------------------------------------------------------
@@ -1928,16 +1940,73 @@ constexpr int kTubeBlocks = 16;          // cluster size
 constexpr int kTubeThreads = 256;        // most sites per block
 constexpr int kTubeRank = 128;           // candidates ranked by counting
 
+template <typename T>
 struct TubeShared {
     TopkScratch sc;
     Thresh th;
-    unsigned count[3];                   // candidates of step t in block 0's count[t mod 3]
+    unsigned count[3];                   // the block's candidates of step t in count[t mod 3]
+    unsigned long long key[kTubeThreads];
+    unsigned idx[kTubeThreads];
+    T pend[kTubeThreads / 32][32][6];    // per warp: g and f* of its pending sites, then dS
 };
 
 template <typename S>
 constexpr size_t tube_smem_bytes(int n) {
     const int per = (n + kTubeBlocks - 1) / kTubeBlocks;
     return (size_t)n * 12 + 16 + 6 * (size_t)per * sizeof(S);
+}
+
+// Exact dS (delta_s_exact, the same operations) of the warp's pending sites,
+// a lane per population: slot[j] holds g and f* of the warp's j-th pending
+// site.  Every lane calls; returns the lane's dS (-1: not pending).
+template <typename T>
+__device__ __forceinline__ T warp_delta_s(bool pending, const T* g, const T* gs, T rho0, T (*slot)[6]) {
+    using L = D1Q3;
+    const int lane = threadIdx.x & 31;
+    const unsigned mask = __ballot_sync(0xffffffffu, pending);
+    const int n = __popc(mask), own = __popc(mask & ((1u << lane) - 1u));
+    if (pending)
+#pragma unroll
+        for (int i = 0; i < L::Q; i++) {
+            slot[own][i] = g[i];
+            slot[own][3 + i] = gs[i];
+        }
+    __syncwarp();
+    const int part = lane % 3;
+    const T w = part == 0 ? T(L::w(0)) : T(L::w(1));
+    for (int b = 0; b < n; b += 10) {
+        const int j = b + lane / 3;
+        const bool on = lane < 30 && j < n;
+        T fs = T(1), x = T(0);
+        bool bad = false;
+        if (on) {
+            const T gi = slot[j][part], si = slot[j][3 + part];
+            fs = dfma<T>(w, rho0, si);
+            const T f = dfma<T>(w, rho0, gi);
+            bad = !(fs > T(0)) || (f < T(0));
+            if constexpr (sizeof(T) == 8) x = (gi - si) * recip<T>(fs);
+            else x = (gi - si) / fs;
+        }
+        const T phi = bad ? T(0) : phi_fn<T>(x);
+        const T fs1 = __shfl_down_sync(0xffffffffu, fs, 1), fs2 = __shfl_down_sync(0xffffffffu, fs, 2);
+        const T phi1 = __shfl_down_sync(0xffffffffu, phi, 1), phi2 = __shfl_down_sync(0xffffffffu, phi, 2);
+        const unsigned bads = __ballot_sync(0xffffffffu, bad);
+        if (on && part == 0) {
+            const T ds = dfma<T>(fs2, phi2, dfma<T>(fs1, phi1, dfma<T>(fs, phi, T(0))));
+            slot[j][0] = (bads >> lane) & 7u ? T(INFINITY) : ds;
+        }
+        __syncwarp();
+    }
+    return pending ? slot[own][0] : T(-1);
+}
+
+__device__ __forceinline__ void cluster_arrive() {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+    __syncwarp();
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
 template <typename S, int EQ>
@@ -1947,30 +2016,27 @@ __global__ void __launch_bounds__(kTubeThreads) k_tube(const __grid_constant__ P
     namespace cg = cooperative_groups;
     cg::cluster_group cluster = cg::this_cluster();
     extern __shared__ __align__(16) unsigned char tube_raw[];
-    __shared__ TubeShared sh;
+    __shared__ TubeShared<T> sh;
     const int n = P.nx, per = (n + kTubeBlocks - 1) / kTubeBlocks;
-    const int rank = (int)cluster.block_rank(), tid = threadIdx.x;
+    const int rank = (int)cluster.block_rank(), tid = threadIdx.x, lane = tid & 31;
     const int x = rank * per + tid;
     const bool mine = tid < per && x < n;
-    // block 0: the step's candidates; every block: its sites' post-collision
-    // populations [parity][plane][per]
+    // block 0: a step's candidates when they are ranked by radix; every block:
+    // its sites' post-collision populations [parity][plane][per]
     unsigned long long* key = reinterpret_cast<unsigned long long*>(tube_raw);
     unsigned* idx = reinterpret_cast<unsigned*>(tube_raw + (size_t)n * 8);
     S* f = reinterpret_cast<S*>(tube_raw + ((size_t)n * 12 + 15) / 16 * 16);
-    unsigned long long* key0 = cluster.map_shared_rank(key, 0);
-    unsigned* idx0 = cluster.map_shared_rank(idx, 0);
-    unsigned* count0 = cluster.map_shared_rank(sh.count, 0);
     if (tid < 3) sh.count[tid] = 0u;
     if (mine)
 #pragma unroll
         for (int i = 0; i < L::Q; i++) f[i * per + tid] = static_cast<const S*>(P.src)[i * P.plane + x];
     const long long t0 = *P.step;
-    const T delta = Par<T>::delta(P);
+    const T delta = Par<T>::delta(P), rho0 = Par<T>::rho0(P);
     bool nonfinite = false;
     NewtonCount nc = {0, 0, 0, 0};
+    int c = (int)(t0 % 3), ring = (int)(t0 % P.ring_cap);
     cluster.sync();
     for (int s = 0; s < steps; s++) {
-        const long long t = t0 + s;
         S* cur = f + (s & 1) * 3 * per;
         S* nxt = f + ((s + 1) & 1) * 3 * per;
         // population i of site xx after the previous step
@@ -1979,8 +2045,8 @@ __global__ void __launch_bounds__(kTubeThreads) k_tube(const __grid_constant__ P
             const S* q = b == rank ? cur : cluster.map_shared_rank(cur, b);
             return Store<S>::load(q + i * per + xx - b * per, 0);
         };
-        const unsigned c = (unsigned)(t % 3);
-        T ds = T(-1), g[L::Q];
+        bool pending = false;
+        T g[L::Q], pre[L::Q], gs[L::Q];
         if (mine) {
             if (s == 0 && P.prestream) {
 #pragma unroll
@@ -1990,7 +2056,11 @@ __global__ void __launch_bounds__(kTubeThreads) k_tube(const __grid_constant__ P
                 g[0] = at(0, x);
 #pragma unroll
                 for (int i = 1; i < L::Q; i++) {
-                    const int sx = x - L::cx(i);
+                    const int sx = x - L::cx(i), local = tid - L::cx(i);
+                    if (local >= 0 && local < per && sx < n) {
+                        g[i] = Store<S>::load(cur + i * per + local, 0);
+                        continue;
+                    }
                     if (sx >= 0 && sx < n) {
                         g[i] = at(i, sx);
                         continue;
@@ -2013,36 +2083,83 @@ __global__ void __launch_bounds__(kTubeThreads) k_tube(const __grid_constant__ P
                     }
                 }
             }
-            update_site<L, T, EQ, Store<S>::kProject, true, true>(P, g, x, 0, t, nonfinite, nc, 0.0f, &ds);
+#pragma unroll
+            for (int i = 0; i < L::Q; i++) pre[i] = g[i];
+            pending = update_site<L, T, EQ, Store<S>::kProject>(P, g, x, 0, t0 + s, nonfinite, nc, 0.0f, nullptr, gs);
 #pragma unroll
             for (int i = 0; i < L::Q; i++) Store<S>::store(nxt + i * per + tid, 0, store_round<L, S>(i, g[i]));
         }
-        // the counter of the step after next's predecessor: last read before
-        // the previous step's barrier, next used after this one's
-        if (rank == 0 && tid == 0) sh.count[(c + 1u) % 3u] = 0u;
+        T ds = T(-1);
+        if (__any_sync(0xffffffffu, pending)) {
+            ds = warp_delta_s<T>(pending, pre, gs, rho0, sh.pend[tid >> 5]);
+            if (pending) {
+                PopArr<L::Q, T> pa;
+#pragma unroll
+                for (int i = 0; i < L::Q; i++) pa.v[i] = pre[i];
+                ds = recheck_ds<L, T, EQ>(pa, ds, delta, P.delta, P.rho0, P.recheck_band, P.recheck);
+            }
+        }
         const bool cand = ds > delta;
         const unsigned long long k = cand ? ds_key((double)ds) : 0ull;
         unsigned slot = 0u;
         if (cand) {
-            slot = atomicAdd(count0 + c, 1u);
-            key0[slot] = k;
-            idx0[slot] = (unsigned)x;
+            slot = atomicAdd(sh.count + c, 1u);
+            sh.key[slot] = k;
+            sh.idx[slot] = (unsigned)x;
         }
-        cluster.sync();
-        const int m = (int)count0[c];        // candidates (the same for every thread)
-        const int sel = min(m, P.k);
+        // the next step's counter: last read two steps ago, before the
+        // previous step's barrier
+        const int cn = c == 2 ? 0 : c + 1;
+        if (tid == 0) sh.count[cn] = 0u;
+        cluster_arrive();
+        T h[L::Q];
+        if (cand) {
+            // f* from the stored post-collision populations, in case
+#pragma unroll
+            for (int i = 0; i < L::Q; i++) h[i] = Store<S>::load(nxt + i * per + tid, 0);
+            ehrenfest_value<L, S, EQ>(P, h);
+        }
+        cluster_wait();
+        // every block's count, in lanes 0 .. 15; m: the step's candidates
+        // (the same for every thread)
+        int m = 0;
+        unsigned cnt = 0u;
+        if (P.k > 0) {
+            if (lane < kTubeBlocks) cnt = cluster.map_shared_rank(sh.count, lane)[c];
+            m = (int)__reduce_add_sync(0xffffffffu, cnt);
+        }
         if (m > 0) {
             bool take = cand;
-            if (m > P.k && m <= kTubeRank) {
-                slot = 0u;
-                if (cand)
-                    for (int e = 0; e < m; e++) {
-                        const unsigned long long ke = key0[e];
-                        slot += ke > k || (ke == k && idx0[e] < (unsigned)x);
+            if (m <= P.k) {
+                slot += __reduce_add_sync(0xffffffffu, lane < rank ? cnt : 0u);
+            } else if (m <= kTubeRank) {
+                if (__any_sync(0xffffffffu, cand)) {
+                    slot = 0u;
+                    for (int b = 0; b < kTubeBlocks; b++) {
+                        const int nb = (int)__shfl_sync(0xffffffffu, cnt, b);
+                        const unsigned long long* kb = cluster.map_shared_rank(sh.key, b);
+                        const unsigned* ib = cluster.map_shared_rank(sh.idx, b);
+                        for (int e = 0; e < nb; e++) {
+                            const unsigned long long ke = kb[e];
+                            slot += ke > k || (ke == k && ib[e] < (unsigned)x);
+                        }
                     }
-                take = cand && slot < (unsigned)P.k;
-            } else if (m > P.k) {
+                    take = cand && slot < (unsigned)P.k;
+                }
+            } else {
                 if (rank == 0) {
+                    int base = 0;
+                    for (int b = 0; b < kTubeBlocks; b++) {
+                        const int nb = (int)__shfl_sync(0xffffffffu, cnt, b);
+                        const unsigned long long* kb = cluster.map_shared_rank(sh.key, b);
+                        const unsigned* ib = cluster.map_shared_rank(sh.idx, b);
+                        for (int e = tid; e < nb; e += blockDim.x) {
+                            key[base + e] = kb[e];
+                            idx[base + e] = ib[e];
+                        }
+                        base += nb;
+                    }
+                    __syncthreads();
                     const Thresh th = block_topk(sh.sc, m, P.k, [&](int e) { return key[e]; },
                                                  [&](int e) { return idx[e]; });
                     if (tid == 0) sh.th = th;
@@ -2050,35 +2167,31 @@ __global__ void __launch_bounds__(kTubeThreads) k_tube(const __grid_constant__ P
                 cluster.sync();
                 const Thresh th = *cluster.map_shared_rank(&sh.th, 0);
                 take = cand && th.selected(k, (unsigned)x);
-            }
-            if (take) {
-                // f' <- f* from the stored post-collision populations
-                T h[L::Q];
-#pragma unroll
-                for (int i = 0; i < L::Q; i++) h[i] = Store<S>::load(nxt + i * per + tid, 0);
-                ehrenfest_value<L, S, EQ>(P, h);
-#pragma unroll
-                for (int i = 0; i < L::Q; i++) Store<S>::store(nxt + i * per + tid, 0, store_round<L, S>(i, h[i]));
-            }
-            if (s == steps - 1) {
-                // the last step's list (order unspecified); by radix: a
-                // selected site's place is its rank among the selected
-                if (m > P.k && m > kTubeRank && take) {
-                    const Thresh th = *cluster.map_shared_rank(&sh.th, 0);
+                if (take && s == steps - 1) {
+                    // its place in the list: its rank among the selected
+                    const unsigned long long* key0 = cluster.map_shared_rank(key, 0);
+                    const unsigned* idx0 = cluster.map_shared_rank(idx, 0);
                     slot = 0u;
                     for (int e = 0; e < m; e++) slot += idx0[e] < (unsigned)x && th.selected(key0[e], idx0[e]);
                 }
-                if (take) P.sel_idx[slot] = x;
             }
-            cluster.sync();
+            if (take) {
+#pragma unroll
+                for (int i = 0; i < L::Q; i++) Store<S>::store(nxt + i * per + tid, 0, store_round<L, S>(i, h[i]));
+                if (s == steps - 1) P.sel_idx[slot] = x;   // (order unspecified)
+            }
+            cluster_arrive();
+            cluster_wait();
         }
         if (rank == 0 && tid == 0) {
-            P.count_ring[t % P.ring_cap] = sel;
+            P.count_ring[ring] = min(m, P.k);
             if (s == steps - 1) {
-                *P.sel_count = sel;
-                *P.step = t + 1;
+                *P.sel_count = min(m, P.k);
+                *P.step = t0 + steps;
             }
         }
+        c = cn;
+        ring = ring + 1 == P.ring_cap ? 0 : ring + 1;
     }
     if (mine) {
         const S* last = f + (steps & 1) * 3 * per;
