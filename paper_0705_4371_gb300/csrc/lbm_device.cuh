@@ -182,9 +182,73 @@ __device__ __forceinline__ bool is_solid(const Params& P, int x, int y) {
 // The library is compiled without automatic multiply-add contraction; every
 // fused multiply-add is written out, so each kernel that evaluates these
 // functions produces the same bits (bit-exact checkpoint / resume).
+template <typename T> constexpr bool kF64 = false;
+template <> constexpr bool kF64<double> = true;
+
+// Two FP32 values, one per site of a pair, worked on by the packed FP32
+// instructions of sm_100 on (add, mul and fma .f32x2): each half is rounded as
+// the scalar instruction rounds it, so a pair gives the bits of two scalar
+// evaluations.  They take one issue slot for two results (measured 64
+// instructions per SM and clock against 117 - 128 scalar ones: the FP32
+// pipes' rate is the same), which leaves the other slots to loads,
+// conversions and integer work.
+// (The host versions only let the shared templates compile.)
+#define LBM_HD __host__ __device__ __forceinline__
+struct __align__(8) f2 {
+    float x, y;
+    f2() = default;
+    LBM_HD f2(float a, float b) : x(a), y(b) {}
+    LBM_HD explicit f2(float a) : x(a), y(a) {}
+    LBM_HD explicit f2(double a) : x((float)a), y((float)a) {}
+    LBM_HD explicit f2(int a) : x((float)a), y((float)a) {}
+};
+#ifdef __CUDA_ARCH__
+__device__ __forceinline__ unsigned long long f2_pack(f2 a) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a.x), "f"(a.y));
+    return r;
+}
+__device__ __forceinline__ f2 f2_unpack(unsigned long long r) {
+    f2 a;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a.x), "=f"(a.y) : "l"(r));
+    return a;
+}
+#endif
+LBM_HD f2 f2_fma(f2 a, f2 b, f2 c) {
+#ifdef __CUDA_ARCH__
+    unsigned long long d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(f2_pack(a)), "l"(f2_pack(b)), "l"(f2_pack(c)));
+    return f2_unpack(d);
+#else
+    return f2(fmaf(a.x, b.x, c.x), fmaf(a.y, b.y, c.y));
+#endif
+}
+LBM_HD f2 operator+(f2 a, f2 b) {
+#ifdef __CUDA_ARCH__
+    unsigned long long d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(f2_pack(a)), "l"(f2_pack(b)));
+    return f2_unpack(d);
+#else
+    return f2(a.x + b.x, a.y + b.y);
+#endif
+}
+LBM_HD f2 operator*(f2 a, f2 b) {
+#ifdef __CUDA_ARCH__
+    unsigned long long d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(f2_pack(a)), "l"(f2_pack(b)));
+    return f2_unpack(d);
+#else
+    return f2(a.x * b.x, a.y * b.y);
+#endif
+}
+LBM_HD f2 operator-(f2 a, f2 b) { return f2_fma(b, f2(-1.0f), a); }   // a - b, rounded once
+LBM_HD f2 operator-(f2 a) { return a * f2(-1.0f); }
+#undef LBM_HD
+
 template <typename T> __host__ __device__ __forceinline__ T dfma(T a, T b, T c);
 template <> __host__ __device__ __forceinline__ float dfma<float>(float a, float b, float c) { return fmaf(a, b, c); }
 template <> __host__ __device__ __forceinline__ double dfma<double>(double a, double b, double c) { return fma(a, b, c); }
+template <> __host__ __device__ __forceinline__ f2 dfma<f2>(f2 a, f2 b, f2 c) { return f2_fma(a, b, c); }
 
 // v . u for lattice velocity components in {-1, 0, 1}: additions only.
 template <typename L, typename T>
@@ -297,38 +361,38 @@ __device__ __forceinline__ typename Store<S>::T store_round(int i, typename Stor
 // energy constraint; D1Q3: sum W v^2 = 1/3).  The sums are of the small
 // nonequilibrium parts, so the conserved moments of the result are exact to
 // their rounding; in exact arithmetic nothing changes.
-template <typename L, int EQ>
-__device__ __forceinline__ void conserve_neq(float* d) {
+template <typename L, int EQ, typename T>
+__device__ __forceinline__ void conserve_neq(T* d) {
     if constexpr (L::Q == 9) {
-        const float D0 = ((d[0] + d[1]) + (d[2] + d[3])) + ((d[4] + d[5]) + (d[6] + d[7])) + d[8];
-        const float Dx = ((d[1] - d[3]) + (d[5] - d[6])) + (d[8] - d[7]);
-        const float Dy = ((d[2] - d[4]) + (d[5] - d[8])) + (d[6] - d[7]);
-        float a = D0, e = 0.0f;
+        const T D0 = ((d[0] + d[1]) + (d[2] + d[3])) + ((d[4] + d[5]) + (d[6] + d[7])) + d[8];
+        const T Dx = ((d[1] - d[3]) + (d[5] - d[6])) + (d[8] - d[7]);
+        const T Dy = ((d[2] - d[4]) + (d[5] - d[8])) + (d[6] - d[7]);
+        T a = D0, e = T(0.0f);
         if constexpr (EQ >= EQ_ENERGY) {
-            const float DE = ((d[1] + d[2]) + (d[3] + d[4])) + 2.0f * ((d[5] + d[6]) + (d[7] + d[8]));
-            a = fmaf(-1.5f, DE, 2.0f * D0);     // a = 2 D0 - 3/2 DE
-            e = fmaf(2.25f, DE, -1.5f * D0);    // e = 9/4 DE - 3/2 D0
+            const T DE = ((d[1] + d[2]) + (d[3] + d[4])) + T(2.0f) * ((d[5] + d[6]) + (d[7] + d[8]));
+            a = dfma<T>(T(-1.5f), DE, T(2.0f) * D0);     // a = 2 D0 - 3/2 DE
+            e = dfma<T>(T(2.25f), DE, T(-1.5f) * D0);    // e = 9/4 DE - 3/2 D0
         }
         // W_i (a + 3 v_i . D + e |v_i|^2), weights 4/9, 1/9, 1/36
-        const float m1 = (a + e) * (1.0f / 9.0f), px = Dx * (1.0f / 3.0f), py = Dy * (1.0f / 3.0f);
-        const float m5 = fmaf(2.0f, e, a) * (1.0f / 36.0f), qx = Dx * (1.0f / 12.0f), qy = Dy * (1.0f / 12.0f);
-        d[0] -= a * (4.0f / 9.0f);
-        d[1] -= m1 + px;
-        d[3] -= m1 - px;
-        d[2] -= m1 + py;
-        d[4] -= m1 - py;
-        const float s1 = m5 + qy, s2 = m5 - qy;
-        d[5] -= s1 + qx;
-        d[6] -= s1 - qx;
-        d[7] -= s2 - qx;
-        d[8] -= s2 + qx;
+        const T m1 = (a + e) * T(1.0f / 9.0f), px = Dx * T(1.0f / 3.0f), py = Dy * T(1.0f / 3.0f);
+        const T m5 = dfma<T>(T(2.0f), e, a) * T(1.0f / 36.0f), qx = Dx * T(1.0f / 12.0f), qy = Dy * T(1.0f / 12.0f);
+        d[0] = d[0] - a * T(4.0f / 9.0f);
+        d[1] = d[1] - (m1 + px);
+        d[3] = d[3] - (m1 - px);
+        d[2] = d[2] - (m1 + py);
+        d[4] = d[4] - (m1 - py);
+        const T s1 = m5 + qy, s2 = m5 - qy;
+        d[5] = d[5] - (s1 + qx);
+        d[6] = d[6] - (s1 - qx);
+        d[7] = d[7] - (s2 - qx);
+        d[8] = d[8] - (s2 + qx);
     } else {
-        const float D0 = (d[0] + d[1]) + d[2];
-        const float Dx = d[2] - d[1];
-        const float m = D0 * (1.0f / 6.0f), p = Dx * 0.5f;   // W (D0 + 3 v Dx), W = 1/6
-        d[0] -= D0 * (2.0f / 3.0f);
-        d[1] -= m - p;
-        d[2] -= m + p;
+        const T D0 = (d[0] + d[1]) + d[2];
+        const T Dx = d[2] - d[1];
+        const T m = D0 * T(1.0f / 6.0f), p = Dx * T(0.5f);   // W (D0 + 3 v Dx), W = 1/6
+        d[0] = d[0] - D0 * T(2.0f / 3.0f);
+        d[1] = d[1] - (m - p);
+        d[2] = d[2] - (m + p);
     }
 }
 
@@ -358,6 +422,10 @@ template <> __host__ __device__ __forceinline__ double recip<double>(double x) {
 #endif
 }
 
+template <> __host__ __device__ __forceinline__ f2 recip<f2>(f2 x) {
+    return f2(recip<float>(x.x), recip<float>(x.y));
+}
+
 // sqrt(x), x > 0: FP32 correctly rounded; FP64 from the hardware's
 // approximation r of 1 / sqrt(x): s = x r, with e = 1 - s r:
 // s + s e (1/2 + 3/8 e), whose error ~ 5/16 e^3 is below 2^-57 -- five FP64
@@ -375,6 +443,8 @@ template <> __host__ __device__ __forceinline__ double dsqrt<double>(double x) {
 #endif
 }
 
+template <> __host__ __device__ __forceinline__ f2 dsqrt<f2>(f2 x) { return f2(sqrtf(x.x), sqrtf(x.y)); }
+
 // Entropic for mass and momentum, by axis.  Sec. 4.1's closed form (with the
 // left/right labels read so that the momentum is +rho u) is rho times
 //   rest (2/3)(2 - s), moving (1/6)(2 s - 1 +- 3 u), s = sqrt(1 + 3 u^2),
@@ -391,7 +461,7 @@ __host__ __device__ __forceinline__ void entropic_axis(T u, T* A) {
     const T q = u3 * u;
     const T s = dsqrt<T>(T(1) + q);
     T sigma;
-    if constexpr (sizeof(T) == 8) sigma = s - T(1);
+    if constexpr (kF64<T>) sigma = s - T(1);
     else sigma = q * recip<T>(T(1) + s);
     A[0] = -sigma;
     const T two = sigma + sigma;
@@ -401,7 +471,7 @@ __host__ __device__ __forceinline__ void entropic_axis(T u, T* A) {
 // ZERO0: the caller's rho0 is zero (FP64 storage; drho = rho).
 template <typename L, typename T, bool ZERO0 = false>
 __host__ __device__ __forceinline__ void feq_entropic(T drho, T rho, T ux, T uy, T* gs) {
-    if constexpr (L::Q == 3 && sizeof(T) == 8) {
+    if constexpr (L::Q == 3 && kF64<T>) {
         // the printed form on rho / 6, correctly rounded (quotient, residual,
         // correction): a rounded weight's error would be the same at every
         // site and step, a drift of the mass (5e-14 after 500 steps)
@@ -514,7 +584,7 @@ __device__ __forceinline__ T delta_s_exact(const T* g, const T* gs, T rho0) {
         fs[i] = dfma<T>(T(L::w(i)), rho0, gs[i]);
         const T f = dfma<T>(T(L::w(i)), rho0, g[i]);
         bad |= !(fs[i] > T(0)) || (f < T(0));
-        if constexpr (sizeof(T) == 8) x[i] = (g[i] - gs[i]) * recip<T>(fs[i]);
+        if constexpr (kF64<T>) x[i] = (g[i] - gs[i]) * recip<T>(fs[i]);
         else x[i] = (g[i] - gs[i]) / fs[i];
     }
     if (bad) return T(INFINITY);
@@ -555,7 +625,7 @@ template <typename L, typename T, int EQ>
 __device__ __forceinline__ bool ds_cleared(const T* d, const T* gs, T rho, T ux, T uy, T rho0,
                                            T delta, float deltaf) {
     // the bound's arithmetic type
-    constexpr bool narrow = sizeof(T) == 8;
+    constexpr bool narrow = kF64<T>;
     using B = float;
     B q0 = B(0), q1 = B(0), q2 = B(0);
 #pragma unroll
@@ -595,6 +665,37 @@ __device__ __forceinline__ bool ds_cleared(const T* d, const T* gs, T rho, T ux,
         }
         return (m > B(0)) && (B(16.0 / wmin) * Q <= m * m) && (B(0.55) * Q <= delta * m);
     }
+}
+
+// The bound for a pair of sites, the same operations half by half: bit 0 and
+// bit 1 set where the pair's first and second site are cleared.
+template <typename L, int EQ>
+__device__ __forceinline__ unsigned ds_cleared_pair(const f2* d, const f2* gs, f2 rho, f2 ux, f2 uy, float rho0,
+                                                    float delta) {
+    f2 q0(0.0f), q1(0.0f), q2(0.0f);
+#pragma unroll
+    for (int i = 0; i < L::Q; i++) {
+        if (L::w(i) == L::w(0)) q0 = f2_fma(d[i], d[i], q0);
+        else if (L::w(i) == L::w(1)) q1 = f2_fma(d[i], d[i], q1);
+        else q2 = f2_fma(d[i], d[i], q2);
+    }
+    constexpr double wmin = 1.0 / 36.0;
+    const f2 Q = f2_fma(q0, f2(1.0 / L::w(0)), f2_fma(q1, f2(1.0 / L::w(1)), q2 * f2(1.0 / L::w(5))));
+    f2 m;
+    if constexpr (EQ == 0) {
+        const f2 usq = f2_fma(ux, ux, uy * uy), a(fabsf(ux.x), fabsf(ux.y)), b(fabsf(uy.x), fabsf(uy.y));
+        m = rho * f2_fma(f2(-1.5f), usq, f2_fma(f2(-3.0f), a + b, f2(1.0f)));
+    } else {
+        m = f2(INFINITY);
+#pragma unroll
+        for (int i = 0; i < L::Q; i++) {
+            const f2 v = f2_fma(gs[i], f2(1.0 / L::w(i)), f2(rho0));
+            m = f2(fminf(m.x, v.x), fminf(m.y, v.y));
+        }
+    }
+    const f2 a = f2((float)(16.0 / wmin)) * Q, b = m * m, c = f2(0.55f) * Q, e = f2(delta) * m;
+    return ((m.x > 0.0f) & (a.x <= b.x) & (c.x <= e.x) ? 1u : 0u) |
+           ((m.y > 0.0f) & (a.y <= b.y) & (c.y <= e.y) ? 2u : 0u);
 }
 
 // Monotone map of a double onto uint64 (larger double <=> larger key).
