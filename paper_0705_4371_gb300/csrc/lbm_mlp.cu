@@ -36,6 +36,7 @@ constexpr int kGradRows = 32;                    // samples a block takes at a t
 constexpr int kGradThreads = 256;
 constexpr int kLd = kMlpHid + 4;                 // activation row: 16-byte aligned, rows on different banks
 constexpr int kPartial = kMlpTrainable + 1;      // per-block gradient sums and the loss
+constexpr int kPartialLd = (kPartial + 3) / 4 * 4;   // a block's row of them (16-byte aligned)
 constexpr int kReduceThreads = 256;
 // Adam's constants; 1 - b is stored as its own correctly rounded FP32 value
 // (1.0f - 0.999f differs from 0.001 by 1.3e-5 relative)
@@ -412,13 +413,13 @@ __device__ __forceinline__ void grad_zero(GradAcc& acc) {
     for (int j = 0; j < 5; j++) acc.ex[j] = 0.0f;
 }
 
-// The thread's sums to the block's row of partial[blocks][kPartial].
+// The thread's sums to the block's row of partial[blocks][kPartialLd].
 __device__ __forceinline__ void grad_store(const GradAcc& acc, float* __restrict__ out) {
     const int tid = threadIdx.x, k = 4 * (tid & 15), n = 4 * (tid >> 4);
 #pragma unroll
     for (int a = 0; a < 4; a++)
-#pragma unroll
-        for (int b = 0; b < 4; b++) out[kMlpW2 + (n + a) * kMlpHid + k + b] = acc.w2[a][b];
+        *reinterpret_cast<float4*>(out + kMlpW2 + (n + a) * kMlpHid + k) =
+            make_float4(acc.w2[a][0], acc.w2[a][1], acc.w2[a][2], acc.w2[a][3]);
     if (tid < 64) {
 #pragma unroll
         for (int j = 0; j < 4; j++) out[kMlpW1 + tid * kMlpIn + j] = acc.ex[j];
@@ -448,7 +449,7 @@ __global__ void __launch_bounds__(kGradThreads) k_mlp_grad(const float* __restri
     grad_zero(acc);
     for (int g = blockIdx.x; g < (n + kGradRows - 1) / kGradRows; g += gridDim.x)
         grad_group(s, grad_load(feat, dmu, 0, n, g), n - g * kGradRows, inv_count, acc);
-    grad_store(acc, partial + (size_t)blockIdx.x * kPartial);
+    grad_store(acc, partial + (size_t)blockIdx.x * kPartialLd);
 }
 
 // Gradient and loss from the block partials, added in block order.
@@ -461,7 +462,7 @@ __global__ void __launch_bounds__(kReduceThreads) k_mlp_reduce(const float* __re
     if (e < kMlpTrainable || loss) {
         const float* at = partial + (loss ? kMlpTrainable : e);
 #pragma unroll 16
-        for (int b = 0; b < nblk; b++) g += at[(size_t)b * kPartial];
+        for (int b = 0; b < nblk; b++) g += at[(size_t)b * kPartialLd];
     }
     if (e < kMlpParams) grad[e] = g;
     else if (loss && loss_out) *loss_out = g * loss_scale;
@@ -478,7 +479,7 @@ __global__ void __launch_bounds__(kReduceThreads) k_mlp_reduce(const float* __re
 // two launches per step this saves the launches, their ramps, and the
 // parameters' and moments' way through memory; a step's samples are loaded
 // before the barrier that ends the previous one.  4096 samples per step,
-// 2^18 samples: 13.5 us per step against 57 us for the two launches
+// 2^18 samples: 12.2 us per step against 57 us for the two launches
 // of one thread per sample and one thread per entry it replaces.
 // ---------------------------------------------------------------------------
 struct __align__(16) StepScale {
@@ -493,7 +494,8 @@ struct TrainArgs {
     long long t0;               // steps done before this launch
     int steps;                  // steps of this launch
     const StepScale* scale;     // [steps]
-    float *partial, *m, *v;     // [blocks][kPartial], Adam moments [kMlpParams]
+    float *partial, *m, *v;     // [sum_blocks][kPartialLd], Adam moments [kMlpParams]
+    int sum_blocks;             // blocks with samples (every block reduces)
     float* loss_log;            // mean batch loss of each epoch (may be null)
     unsigned long long* barrier;   // arrivals (zero at launch)
 };
@@ -524,12 +526,12 @@ __host__ __device__ constexpr int train_segs(int G) { return G < kGradThreads / 
 __global__ void __launch_bounds__(kGradThreads) k_mlp_train(const TrainArgs A) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     GradSmem& s = *reinterpret_cast<GradSmem*>(smem_raw);
-    const int tid = threadIdx.x, G = gridDim.x;
+    const int tid = threadIdx.x, G = gridDim.x, B = A.sum_blocks;
     const int per = (kPartial + G - 1) / G, e0 = blockIdx.x * per, ne = max(0, min(per, kPartial - e0));
     // the block's entries of p, m, v and the segments' sums, after the tiles
     float* own = reinterpret_cast<float*>(smem_raw + sizeof(GradSmem));
     float *own_p = own, *own_m = own + per, *own_v = own + 2 * per, *red = own + 3 * per;   // red[segs][per]
-    const int segs = train_segs(G);
+    const int segs = train_segs(B);
     __shared__ int ok;
     for (int e = tid; e < ne; e += kGradThreads) {
         const bool w = e0 + e < kMlpTrainable;
@@ -544,16 +546,18 @@ __global__ void __launch_bounds__(kGradThreads) k_mlp_train(const TrainArgs A) {
         const long long i0 = b * A.batch;
         const int n = (int)min((long long)A.batch, A.n - i0);
         const float inv = 1.0f / (4.0f * (float)n);
-        grad_fill(s, A.p);
-        __syncthreads();
-        GradAcc acc;
-        grad_zero(acc);
-        for (int g = blockIdx.x; g < (n + kGradRows - 1) / kGradRows; g += G) {
-            const GradIn cur = in;
-            in = grad_load(A.feat, A.dmu, i0, n, g + G);   // the next group's (zeros beyond the batch)
-            grad_group(s, cur, n - g * kGradRows, inv, acc);
+        if ((int)blockIdx.x < B) {
+            grad_fill(s, A.p);
+            __syncthreads();
+            GradAcc acc;
+            grad_zero(acc);
+            for (int g = blockIdx.x; g < (n + kGradRows - 1) / kGradRows; g += B) {
+                const GradIn cur = in;
+                in = grad_load(A.feat, A.dmu, i0, n, g + B);   // the next group's (zeros beyond the batch)
+                grad_group(s, cur, n - g * kGradRows, inv, acc);
+            }
+            grad_store(acc, A.partial + (size_t)blockIdx.x * kPartialLd);
         }
-        grad_store(acc, A.partial + (size_t)blockIdx.x * kPartial);
         const long long bn = b + 1 == A.nb ? 0 : b + 1;
         const StepScale sc = A.scale[t];
         in = grad_load(A.feat, A.dmu, bn * A.batch, (int)min((long long)A.batch, A.n - bn * A.batch), blockIdx.x);
@@ -565,7 +569,7 @@ __global__ void __launch_bounds__(kGradThreads) k_mlp_train(const TrainArgs A) {
                 float g = 0.0f;
                 const float* at = A.partial + e0 + e;
 #pragma unroll 16
-                for (int q = seg; q < G; q += segs) g += __ldcg(at + (size_t)q * kPartial);
+                for (int q = seg; q < B; q += segs) g += __ldcg(at + (size_t)q * kPartialLd);
                 red[seg * per + e] = g;
             }
         __syncthreads();
@@ -635,10 +639,10 @@ int grad_grid(long long n, int most) {
     return (int)std::max(1ll, std::min<long long>((n + kGradRows - 1) / kGradRows, most));
 }
 
-// Shared memory of the training kernel with G blocks.
-size_t train_smem(int G) {
+// Shared memory of the training kernel with G blocks, B of them with samples.
+size_t train_smem(int G, int B) {
     const int per = (kPartial + G - 1) / G;
-    return sizeof(GradSmem) + (size_t)(3 + train_segs(G)) * per * sizeof(float);
+    return sizeof(GradSmem) + (size_t)(3 + train_segs(B)) * per * sizeof(float);
 }
 
 // Adam's bias corrections 1 / (1 - b^t)
@@ -730,7 +734,7 @@ int lb_mlp_grad(const float* params, const float* feat, const float* dmu, int n,
     CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const int nblk = grad_grid(n, 2 * sms);
     float* partial = nullptr;
-    CK(cudaMallocAsync(&partial, (size_t)nblk * kPartial * sizeof(float), st));
+    CK(cudaMallocAsync(&partial, (size_t)nblk * kPartialLd * sizeof(float), st));
     const float inv = 1.0f / (4.0f * (float)n);
     k_mlp_grad<<<nblk, kGradThreads, sizeof(GradSmem), st>>>(params, feat, dmu, n, inv, partial);
     cudaError_t e = cudaGetLastError();
@@ -770,9 +774,10 @@ int lb_mlp_train(float* params, const float* feat, const float* dmu, long long n
     CK(cudaGetDevice(&dev));
     CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     // one block per SM: a step's chain of latencies is the same with more,
-    // and the reduction has fewer partials to add
-    const int G = grad_grid(std::min<long long>(n, batch), sms);
-    const size_t smem = train_smem(G);
+    // and the reduction has fewer partials to add; every SM takes part in the
+    // reduction (152 blocks: 32 entries each, one per lane)
+    const int A_blocks = grad_grid(std::min<long long>(n, batch), sms), G = sms;
+    const size_t smem = train_smem(G, A_blocks);
     CK(cudaFuncSetAttribute(k_mlp_train, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_mlp_train, kGradThreads, smem));
     if (per_sm < 1) return fail(LB_ERR_CUDA, "the training kernel does not fit on this device");
@@ -780,14 +785,14 @@ int lb_mlp_train(float* params, const float* feat, const float* dmu, long long n
     constexpr long long kChunk = 1 << 16;   // steps per launch
     const size_t scale_b = (size_t)std::min(std::max(total, 1ll), kChunk) * sizeof(StepScale);
     const size_t mv_b = 2 * (size_t)kMlpParams * sizeof(float);
-    const size_t part_b = (size_t)G * kPartial * sizeof(float);
+    const size_t part_b = (size_t)A_blocks * kPartialLd * sizeof(float);
     unsigned char* mem = nullptr;
     CK(cudaMallocAsync(&mem, scale_b + mv_b + 16 + part_b, st));
     float* m = reinterpret_cast<float*>(mem + scale_b);
     cudaError_t e = cudaMemsetAsync(mem + scale_b, 0, mv_b + 16, st);
     if (e == cudaSuccess && loss_log) e = cudaMemsetAsync(loss_log, 0, (size_t)epochs * sizeof(float), st);
     TrainArgs A = {params, feat, dmu, n, nb, batch, 0, 0, reinterpret_cast<StepScale*>(mem),
-                   reinterpret_cast<float*>(mem + scale_b + mv_b + 16), m, m + kMlpParams, loss_log,
+                   reinterpret_cast<float*>(mem + scale_b + mv_b + 16), m, m + kMlpParams, A_blocks, loss_log,
                    reinterpret_cast<unsigned long long*>(mem + scale_b + mv_b)};
     for (long long t = 0; t < total && e == cudaSuccess; t += kChunk) {
         A.t0 = t;

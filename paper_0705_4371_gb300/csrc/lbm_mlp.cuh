@@ -144,7 +144,22 @@ __device__ __forceinline__ void mlp_tile_forward(const MlpSmem& s, unsigned a0, 
             h1[r1 * ld + col + 1] = bf16_hi(u1);
         }
     }
-    // layers 2 and 3: each pair of layer-2 n-tiles is one layer-3 k-step
+    // layer 2, its eight accumulators side by side (each k-step of one waits
+    // for its previous k-step)
+    float c2[8][4];
+#pragma unroll
+    for (int nt = 0; nt < 8; nt++) {
+        c2[nt][0] = c2[nt][2] = s.b2[8 * nt + 2 * tig];
+        c2[nt][1] = c2[nt][3] = s.b2[8 * nt + 2 * tig + 1];
+    }
+#pragma unroll
+    for (int j = 0; j < 4; j++)
+#pragma unroll
+        for (int nt = 0; nt < 8; nt++) {
+            const uint2 b = s.w2[nt][j][lane];
+            mma_bf16(c2[nt], A2[j][0], A2[j][1], A2[j][2], A2[j][3], b.x, b.y);
+        }
+    // layer 3: each pair of layer-2 n-tiles is one k-step
     yc[0] = yc[2] = s.b3[2 * tig];
     yc[1] = yc[3] = s.b3[2 * tig + 1];
 #pragma unroll
@@ -153,14 +168,7 @@ __device__ __forceinline__ void mlp_tile_forward(const MlpSmem& s, unsigned a0, 
 #pragma unroll
         for (int hh = 0; hh < 2; hh++) {
             const int nt = 2 * jp + hh;
-            const float bl = s.b2[8 * nt + 2 * tig], bh = s.b2[8 * nt + 2 * tig + 1];
-            float c[4] = {bl, bh, bl, bh};
-#pragma unroll
-            for (int j = 0; j < 4; j++) {
-                const uint2 b = s.w2[nt][j][lane];
-                mma_bf16(c, A2[j][0], A2[j][1], A2[j][2], A2[j][3], b.x, b.y);
-            }
-            const unsigned u0 = bf16_pack_relu(c[0], c[1]), u1 = bf16_pack_relu(c[2], c[3]);
+            const unsigned u0 = bf16_pack_relu(c2[nt][0], c2[nt][1]), u1 = bf16_pack_relu(c2[nt][2], c2[nt][3]);
             A3[2 * hh] = u0;
             A3[2 * hh + 1] = u1;
             if constexpr (CAP) {
