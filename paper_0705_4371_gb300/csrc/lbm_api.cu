@@ -52,13 +52,12 @@ constexpr int kDefaultLog = 65536;
 // dominated by latency): register-fed tiles for polynomial-f* FP32 (shape 1;
 // alone 600 x 500 takes 13.4 us, 12.7 - 14.3 staged), 6-row staged tiles for
 // the others (shape 5; FP16 500 x 256: 7.1 against 8.6 on shape 4).  Above,
-// the 8-row tiles' warps win wherever arithmetic is what bounds a step (shape
-// 4; 4096 x 2048: entropic FP32 115 against 131; 2048 x 1024 ELBM 91 against
-// 125) and, less, where memory does (polynomial FP32: 94 against 97 at
-// 4096 x 2048, 13.1 against 14.3 at 1280 x 640; between 600 000 and 800 000
-// sites it keeps shape 5).  FP16 gains from 1e6 sites on (1024 x 600: 10.7
-// against 9.4; 2048 x 1024: 20 against 24; 4096 x 2048: 68 against 84).
-// FP64 storage: 8-row tiles.  The energy forms: FP64 storage's
+// polynomial-f* FP32, bound by memory, keeps the 6-row tiles' three copies in
+// flight (97 at 4096 x 2048, 94 on shape 4); where arithmetic is what bounds
+// a step the 8-row tiles' warps win (shape 4; 4096 x 2048: entropic FP32 115
+// against 131; 2048 x 1024 ELBM 91 against 125), for FP16 from 1e6 sites on
+// (1024 x 600: 10.7 against 9.4; 2048 x 1024: 20 against 24; 4096 x 2048: 68
+// against 84).  FP64 storage: 8-row tiles.  The energy forms: FP64 storage's
 // solve wants the most resident warps (register-fed shape 1); the
 // float-float solve of FP32 / FP16 storage and the network's warm start run
 // best in the staged shape 4 (measured at 2048 x 1024: Newton start 89 us
@@ -69,8 +68,8 @@ int default_tile_shape(int lattice, int eq, int precision, long long sites, bool
     if (eq < LB_EQ_ENTROPIC_ENERGY) {
         if (precision == LB_F64 || elbm) return 4;
         if (precision == LB_F16_DEV) return sites <= 1000000 ? 5 : 4;
-        if (eq == LB_EQ_POLY && sites <= 600000) return 1;
-        return sites <= (eq == LB_EQ_POLY ? 800000 : 600000) ? 5 : 4;
+        if (eq == LB_EQ_POLY) return sites <= 600000 ? 1 : 5;
+        return sites <= 600000 ? 5 : 4;
     }
     if (precision == LB_F64) return 1;
     return 4;

@@ -549,26 +549,29 @@ template <> __device__ __forceinline__ float phi_fn<float>(float x) {
     return fmaf(1.0f + x, log1pf(x), -x);
 }
 
+// (FP64 takes 64 cycles per warp instruction and SM quarter, whatever the
+// lanes or the dependences: what counts is the number of operations, over
+// both branches when a warp's lanes take both.  log1p alone takes about as many
+// as both sums here.)
 template <> __device__ __forceinline__ double phi_fn<double>(double x) {
-    if (fabs(x) <= 0.015625) {
-        // terms n = 2..9; truncation < 1e-16 relative at |x| = 1/64
-        double p = 0.0;
-#pragma unroll
-        for (int n = 9; n >= 2; n--) {
-            const double c = ((n & 1) ? -1.0 : 1.0) / (double(n) * double(n - 1));
-            p = fma(p, x, c);
-        }
-        return x * x * p;
-    }
     if (fabs(x) <= 0.0625) {
         // terms n = 2..17; truncation < 1e-18 relative at |x| = 1/16
         double p = 0.0;
 #pragma unroll
         for (int n = 17; n >= 2; n--) {
             const double c = ((n & 1) ? -1.0 : 1.0) / (double(n) * double(n - 1));
-            p = fma(p, x, c);
+            p = n == 17 ? c : fma(p, x, c);
         }
         return x * x * p;
+    }
+    if (x >= -0.5 && x <= 1.0) {
+        // ln(1 + x) = 2 artanh(t), t = x / (2 + x): |t| <= 1/3, artanh(t) =
+        // t sum t^{2k} / (2k + 1), k <= 16 (truncation < 2e-18)
+        const double t = x * recip<double>(2.0 + x), z = t * t;
+        double q = 1.0 / 33.0;
+#pragma unroll
+        for (int k = 15; k >= 0; k--) q = fma(q, z, 1.0 / double(2 * k + 1));
+        return fma((1.0 + x) * (t + t), q, -x);
     }
     if (x <= -1.0) return 1.0;
     return fma(1.0 + x, log1p(x), -x);

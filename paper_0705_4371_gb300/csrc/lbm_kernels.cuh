@@ -1995,12 +1995,13 @@ __global__ void __launch_bounds__(kSiteBlock) k_collide_site(const __grid_consta
 // clock), the exact dS of the sites near the front, the selection -- so the
 // state stays in the shared memory of a cluster of 16 blocks (16 SMs' FP64
 // pipes), neighbours read each other's edge sites there, every block lists its
-// candidates, and the hardware's cluster barrier separates the collision from
-// the selection and, when a step has candidates, the Ehrenfests' step from
-// the next free flight.  The exact dS of a warp's pending sites takes a lane
-// per population (its series and logarithms are the longest FP64 chain of a
-// step), and a candidate's f* is evaluated while the barrier completes.
-// 800 sites, FP64: 23.5 us per step in one launch each (4 blocks), 5.9 us so
+// candidates and gives them their f* at once, and the hardware's cluster
+// barrier separates the collision from the selection; only a step with more
+// than k candidates, where some take their post-collision populations back,
+// needs a second one before the next free flight.  The exact dS of a warp's
+// pending sites takes a lane per population (its series are the longest FP64
+// chain of a step).
+// 800 sites, FP64: 23.5 us per step in one launch each (4 blocks), 5.7 us so
 // (2.5 us without the selection).
 // Every population passes through the storage type, so results are those of
 // one launch per step.
@@ -2180,14 +2181,18 @@ __global__ void __launch_bounds__(kTubeThreads) k_tube(const __grid_constant__ P
         // previous step's barrier
         const int cn = c == 2 ? 0 : c + 1;
         if (tid == 0) sh.count[cn] = 0u;
-        cluster_arrive();
-        T h[L::Q];
         if (cand) {
-            // f* from the stored post-collision populations, in case
+            // the Ehrenfests' step from the stored post-collision populations,
+            // as if every candidate were selected; with more than k of them
+            // the others take theirs (g) back
+            T h[L::Q];
 #pragma unroll
             for (int i = 0; i < L::Q; i++) h[i] = Store<S>::load(nxt + i * per + tid, 0);
             ehrenfest_value<L, S, EQ>(P, h);
+#pragma unroll
+            for (int i = 0; i < L::Q; i++) Store<S>::store(nxt + i * per + tid, 0, store_round<L, S>(i, h[i]));
         }
+        cluster_arrive();
         cluster_wait();
         // every block's count, in lanes 0 .. 15; m: the step's candidates
         // (the same for every thread)
@@ -2244,13 +2249,15 @@ __global__ void __launch_bounds__(kTubeThreads) k_tube(const __grid_constant__ P
                     for (int e = 0; e < m; e++) slot += idx0[e] < (unsigned)x && th.selected(key0[e], idx0[e]);
                 }
             }
-            if (take) {
+            if (take && s == steps - 1) P.sel_idx[slot] = x;   // (order unspecified)
+            if (m > P.k) {
+                if (cand && !take)
 #pragma unroll
-                for (int i = 0; i < L::Q; i++) Store<S>::store(nxt + i * per + tid, 0, store_round<L, S>(i, h[i]));
-                if (s == steps - 1) P.sel_idx[slot] = x;   // (order unspecified)
+                    for (int i = 0; i < L::Q; i++)
+                        Store<S>::store(nxt + i * per + tid, 0, store_round<L, S>(i, g[i]));
+                cluster_arrive();
+                cluster_wait();
             }
-            cluster_arrive();
-            cluster_wait();
         }
         if (rank == 0 && tid == 0) {
             P.count_ring[ring] = min(m, P.k);
