@@ -124,8 +124,8 @@ __device__ __forceinline__ T energy_moment(const T* g, T rho0) {
     T e2 = T(L::sum_w_c2) * rho0;
 #pragma unroll
     for (int i = 0; i < L::Q; i++)
-        if (L::cx(i) * L::cx(i) + L::cy(i) * L::cy(i) == 1) e2 += g[i];
-        else if (L::cx(i) * L::cx(i) + L::cy(i) * L::cy(i) == 2) e2 += T(2) * g[i];
+        if (L::cx(i) * L::cx(i) + L::cy(i) * L::cy(i) == 1) e2 = e2 + g[i];
+        else if (L::cx(i) * L::cx(i) + L::cy(i) * L::cy(i) == 2) e2 = e2 + T(2) * g[i];
     return e2;
 }
 
@@ -444,9 +444,9 @@ __device__ __forceinline__ bool update_site(const Params& P, T* g, int x, int y,
     return pending;
 }
 
-// update_site of two adjacent sites at once in packed FP32 arithmetic
-// (polynomial and entropic f* of FP32 and FP16 storage; every operation the
-// scalar one's, half by half).  g: pre-collision deviations in,
+// update_site of two adjacent sites at once in packed FP32 arithmetic (FP32
+// and FP16 storage; every operation the scalar one's, half by half).  nc, mu3:
+// the sites' Newton counts and start points (energy forms).  g: pre-collision deviations in,
 // post-collision deviations out, before the storage's rounding.  Returns bit 0
 // / bit 1: the bound does not clear the first / second site.
 // The scalar update issues about 240 instructions per site, 145 of them FP32
@@ -454,13 +454,15 @@ __device__ __forceinline__ bool update_site(const Params& P, T* g, int x, int y,
 // the export: FP16 4911 -> 4602 us, polynomial FP32 (bound by memory) 6314 ->
 // 6165 us; 1531 x 765 entropic FP32 1208 -> 1143 us.
 template <typename S, int EQ>
-__device__ __forceinline__ unsigned update_pair(const Params& P, f2* g, bool& nonfinite) {
+__device__ __forceinline__ unsigned update_pair(const Params& P, f2* g, bool& nonfinite, NewtonCount* nc = nullptr,
+                                                f2 mu3 = f2(0.0f)) {
     using L = D2Q9;
-    static_assert(EQ < EQ_ENERGY && sizeof(typename Store<S>::T) == 4, "FP32 arithmetic, no energy solve");
+    static_assert(sizeof(typename Store<S>::T) == 4, "FP32 arithmetic");
     f2 gs[L::Q], drho, rho, jx, jy, ux, uy;
     moments<L, f2>(g, f2(P.rho0f), drho, rho, jx, jy);
     velocity<f2>(jx, jy, rho, ux, uy);
-    equilibrium<L, f2, EQ>(P, drho, rho, ux, uy, gs);
+    if constexpr (EQ >= EQ_ENERGY) energy_solve_pair(rho, jx, jy, energy_moment<L, f2>(g, f2(P.rho0f)), mu3, gs, nc);
+    else equilibrium<L, f2, EQ>(P, drho, rho, ux, uy, gs);
     const f2 s = (rho + ux) + uy;
     nonfinite |= !isfinite(s.x) | !isfinite(s.y);
     f2 d[L::Q];
@@ -1737,24 +1739,29 @@ __device__ __forceinline__ void tma_tile(const Params& P, S* box, int x0, int y0
                 gb[i] = eb ? T(L::w(i)) * r1 : gb[i];
             }
         }
-        if constexpr (EQ < EQ_ENERGY && !kF64<T>) {
+        // (the sites that are not the row's do not count as solved)
+        float ma = 0.0f, mb = 0.0f;
+        if constexpr (EQ == EQ_ENERGY_MLP) {
+            ma = mlp_site_start<T>(P, mslot.s, true, ga);
+            mb = mlp_site_start<T>(P, mslot.s, true, gb);
+        }
+        if constexpr (!kF64<T>) {
             f2 g[L::Q];
 #pragma unroll
             for (int i = 0; i < L::Q; i++) g[i] = f2(ga[i], gb[i]);
-            pend = update_pair<S, EQ>(P, g, state.nonfinite);
+            NewtonCount n2[2] = {};
+            pend = update_pair<S, EQ>(P, g, state.nonfinite, n2, f2(ma, mb));
+            if constexpr (EQ >= EQ_ENERGY) {
+                if (!ea) state.nc.add(n2[0]);
+                if (!eb) state.nc.add(n2[1]);
+            }
 #pragma unroll
             for (int i = 0; i < L::Q; i++) {
                 ga[i] = g[i].x;
                 gb[i] = g[i].y;
             }
         } else {
-            // (the sites that are not the row's do not count as solved)
             NewtonCount na = state.nc;
-            float ma = 0.0f, mb = 0.0f;
-            if constexpr (EQ == EQ_ENERGY_MLP) {
-                ma = mlp_site_start<T>(P, mslot.s, true, ga);
-                mb = mlp_site_start<T>(P, mslot.s, true, gb);
-            }
             if (update_site<L, T, EQ, Store<S>::kProject, false>(P, ga, x0 + c, y, t, state.nonfinite, na, ma)) pend = 1u;
             if (EQ >= EQ_ENERGY && !ea) state.nc = na;
             na = state.nc;
@@ -1793,13 +1800,14 @@ __device__ __forceinline__ void tma_tile(const Params& P, S* box, int x0, int y0
 // (128 registers per thread with 8-row tiles, 170 with 6-row tiles); three
 // (85 registers per thread) where the tiles take half the shared memory:
 // FP16 storage, or FP32 tiles 64 sites wide.
-template <typename S, int R, int TX>
+template <typename S, int EQ, int R, int TX>
 constexpr int tma_min_blocks() {
+    if (EQ >= EQ_ENERGY) return 2;   // (the packed solve spills at 85)
     return (sizeof(S) == 2 && R == 8) || (sizeof(S) == 4 && TX == 64 && R == 8) ? 3 : 2;
 }
 
 template <typename S, int EQ, int R, int STAGES, int TX = kTmaTX>
-__global__ void __launch_bounds__(32 * R, tma_min_blocks<S, R, TX>())
+__global__ void __launch_bounds__(32 * R, tma_min_blocks<S, EQ, R, TX>())
     k_collide_d2q9_tma(const __grid_constant__ Params P, const __grid_constant__ CUtensorMap tm) {
     using L = D2Q9;
     using T = typename Store<S>::T;
