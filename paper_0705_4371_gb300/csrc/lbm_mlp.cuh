@@ -144,43 +144,49 @@ __device__ __forceinline__ void mlp_tile_forward(const MlpSmem& s, unsigned a0, 
             h1[r1 * ld + col + 1] = bf16_hi(u1);
         }
     }
-    // layer 2, its eight accumulators side by side (each k-step of one waits
-    // for its previous k-step)
-    float c2[8][4];
-#pragma unroll
-    for (int nt = 0; nt < 8; nt++) {
-        c2[nt][0] = c2[nt][2] = s.b2[8 * nt + 2 * tig];
-        c2[nt][1] = c2[nt][3] = s.b2[8 * nt + 2 * tig + 1];
-    }
-#pragma unroll
-    for (int j = 0; j < 4; j++)
-#pragma unroll
-        for (int nt = 0; nt < 8; nt++) {
-            const uint2 b = s.w2[nt][j][lane];
-            mma_bf16(c2[nt], A2[j][0], A2[j][1], A2[j][2], A2[j][3], b.x, b.y);
-        }
-    // layer 3: each pair of layer-2 n-tiles is one k-step
+    // layers 2 and 3: W of layer 2's accumulators at a time take their k-steps
+    // side by side (each k-step of one waits for its previous one; all eight
+    // where a block's two warps are alone with the chain, CAP), and each pair
+    // of layer-2 n-tiles is one layer-3 k-step
+    constexpr int W = CAP ? 8 : 2;
     yc[0] = yc[2] = s.b3[2 * tig];
     yc[1] = yc[3] = s.b3[2 * tig + 1];
 #pragma unroll
-    for (int jp = 0; jp < 4; jp++) {
-        unsigned A3[4];
+    for (int n0 = 0; n0 < 8; n0 += W) {
+        float c[W][4];
 #pragma unroll
-        for (int hh = 0; hh < 2; hh++) {
-            const int nt = 2 * jp + hh;
-            const unsigned u0 = bf16_pack_relu(c2[nt][0], c2[nt][1]), u1 = bf16_pack_relu(c2[nt][2], c2[nt][3]);
-            A3[2 * hh] = u0;
-            A3[2 * hh + 1] = u1;
-            if constexpr (CAP) {
-                const int col = 8 * nt + 2 * tig;
-                h2[r0 * ld + col] = bf16_lo(u0);
-                h2[r0 * ld + col + 1] = bf16_hi(u0);
-                h2[r1 * ld + col] = bf16_lo(u1);
-                h2[r1 * ld + col + 1] = bf16_hi(u1);
-            }
+        for (int q = 0; q < W; q++) {
+            const int col = 8 * (n0 + q) + 2 * tig;
+            c[q][0] = c[q][2] = s.b2[col];
+            c[q][1] = c[q][3] = s.b2[col + 1];
         }
-        const uint2 b = s.w3[jp][lane];
-        mma_bf16(yc, A3[0], A3[1], A3[2], A3[3], b.x, b.y);
+#pragma unroll
+        for (int j = 0; j < 4; j++)
+#pragma unroll
+            for (int q = 0; q < W; q++) {
+                const uint2 b = s.w2[n0 + q][j][lane];
+                mma_bf16(c[q], A2[j][0], A2[j][1], A2[j][2], A2[j][3], b.x, b.y);
+            }
+#pragma unroll
+        for (int q = 0; q < W; q += 2) {
+            unsigned A3[4];
+#pragma unroll
+            for (int hh = 0; hh < 2; hh++) {
+                const unsigned u0 = bf16_pack_relu(c[q + hh][0], c[q + hh][1]);
+                const unsigned u1 = bf16_pack_relu(c[q + hh][2], c[q + hh][3]);
+                A3[2 * hh] = u0;
+                A3[2 * hh + 1] = u1;
+                if constexpr (CAP) {
+                    const int col = 8 * (n0 + q + hh) + 2 * tig;
+                    h2[r0 * ld + col] = bf16_lo(u0);
+                    h2[r0 * ld + col + 1] = bf16_hi(u0);
+                    h2[r1 * ld + col] = bf16_lo(u1);
+                    h2[r1 * ld + col + 1] = bf16_hi(u1);
+                }
+            }
+            const uint2 b = s.w3[(n0 + q) / 2][lane];
+            mma_bf16(yc, A3[0], A3[1], A3[2], A3[3], b.x, b.y);
+        }
     }
 }
 
