@@ -304,14 +304,17 @@ template <> struct Par<double> {
 // every FP32 / FP16 form.
 // ---------------------------------------------------------------------------
 
-// FP32 to FP64 by integer operations (the conversion instruction runs on the
-// FP64 pipe, two per SM and clock); subnormal, infinite and NaN values take
-// the instruction.
+// FP32 to FP64 by integer operations: the conversion instruction runs on the
+// FP64 pipe (two per SM and clock), and does so even where a predicate turns
+// it off.  Subnormal values are scaled by 2^64 first; exponent 255 (infinity,
+// NaN) becomes 2047.
 __device__ __forceinline__ double widen(float x) {
-    const unsigned b = __float_as_uint(x), m = b & 0x7fffffffu;
-    if (m - 0x00800000u >= 0x7f000000u && m != 0u) return (double)x;
-    const unsigned hi = m ? (m >> 3) + (896u << 20) : 0u;
-    return __hiloint2double((int)(hi | (b & 0x80000000u)), (int)(b << 29));
+    const bool small = (__float_as_uint(x) & 0x7fffffffu) < 0x00800000u;
+    const unsigned b = __float_as_uint(small ? x * 0x1p64f : x), m = b & 0x7fffffffu;
+    unsigned e = small ? (896u - 64u) << 20 : 896u << 20;
+    if (m >= 0x7f800000u) e = 1792u << 20;
+    if (m == 0u) e = 0u;
+    return __hiloint2double((int)(((m >> 3) + e) | (b & 0x80000000u)), (int)(b << 29));
 }
 
 // FP64 value of population i whose stored deviation is g (FP64 storage holds

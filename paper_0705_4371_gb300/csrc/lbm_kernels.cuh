@@ -2400,9 +2400,11 @@ struct Sum2 {
 // [s0, s1), exported as mode 0: populations f [Q][ny][nx]; 1: rho, ux, uy,
 // 2E; 2: exact dS (outputs indexed by the site's index y nx + x).
 // The moments of FP32 / FP16 storage were bound by the FP64 pipe (27
-// operations per site, conversions included); six are left, and the
-// sums share their parts: 4096 x 2048, FP32: 355 -> 222 us, FP64 2048 x 1024
-// (divisions and products with lattice velocities before): 302 -> 100 us.
+// operations per site, conversions included); six are left, the sums share
+// their parts, and the conversions run on the integer pipe (a predicated
+// conversion instruction still took its FP64 slots): 4096 x 2048, FP32:
+// 355 -> 222 -> 144 us, FP64 2048 x 1024 (divisions and products with lattice
+// velocities before): 302 -> 100 us.
 template <typename L, typename S, int EQ>
 __global__ void k_export(const __grid_constant__ Params P, int mode, double* o0, double* o1, double* o2,
                          double* o3, long long s0, long long s1) {
