@@ -53,10 +53,12 @@ enum lb_lattice { LB_D1Q3 = 0, LB_D2Q9 = 1 };
  *                   Sec. 4.2 product formula);
  *   LB_EQ_ENTROPIC_ENERGY      entropic with the energy constraint as well,
  *                   M = (rho, rho u1, rho u2, 2E) ((argmax), Lagrange form of
- *                   Sec. 3.3), solved per site by Newton from the polynomial
- *                   start point (FP32 iterations, then finishing steps to a
- *                   residual of 1e-12 with the residual in float-float for
- *                   FP32 / FP16 storage, in FP64 for FP64 storage);
+ *                   Sec. 3.3), solved per site by Newton on the scalar
+ *                   equation left when the other multipliers are eliminated,
+ *                   from the polynomial start point (FP32 iterations, then
+ *                   finishing steps to a residual of 1e-12 with the residual
+ *                   in float-float for FP32 / FP16 storage, in FP64 for FP64
+ *                   storage);
  *   LB_EQ_ENTROPIC_ENERGY_MLP  as above, Newton warm-started by the 4-64-64-4
  *                   network loaded with lb_set_mlp (BF16 tensor cores). */
 enum lb_equilibrium {
@@ -352,12 +354,13 @@ int lb_kernel_times(lb_handle* h, double* collide_ms, long long* collide_launche
  * Shared-memory-staged shapes (tensor-memory-accelerator copies, for every
  * population plane, of the R rows of the R x C-site block tile's sources in
  * that plane plus 16 bytes of halo columns; R rows, C columns, STAGES tiles
- * in flight per block): 4 = 8 x 128, STAGES 2 (default of FP64 storage);
- * 5 = 6 x 128, STAGES 3 (default of FP16 storage and of FP32 storage, plain
- * and deviation, above 600 000 sites; FP32 storage with the polynomial
- * quasiequilibrium up to 600 000 sites defaults to the register-fed shape
- * 1);  6 = 8 x 64, STAGES 2 (three blocks
- * per SM).  The
+ * in flight per block): 4 = 8 x 128, STAGES 2 (FP16 storage 3);
+ * 5 = 6 x 128, STAGES 3;  6 = 8 x 64, STAGES 2.  Defaults: 4 for FP64
+ * storage and the ELBM collision; for FP32 storage with the polynomial
+ * quasiequilibrium 1 up to 600 000 sites, then 5 up to 1e6, 4 up to 5e6 and
+ * 5 above; with the entropic one 5 up to 600 000 sites and 4 above; for FP16
+ * storage 5 up to 1e6 sites and 4 above (lb_set_collision chooses anew
+ * unless a shape was set here).  The
  * energy-constrained forms are built for shapes 0 (1, 8, 2: 128 registers
  * per thread), 1 (2 and 3 run 1), 4 and 5, and refuse 6 (LB_ERR_ARG); their
  * defaults: 1 for FP64 storage, 4 for FP32 / FP16 storage (Newton start and

@@ -49,15 +49,16 @@ constexpr int kXferEvents = 16;      // events of one chunked transfer (>= Q pla
 constexpr int kDefaultLog = 65536;
 // Default tile shapes by measurement on GB300 (us per step of two runs side by
 // side).  Up to 600 000 sites (one or two tiles per resident block, a step
-// dominated by latency): register-fed tiles for polynomial-f* FP32 (shape 1;
-// alone 600 x 500 takes 13.4 us, 12.7 - 14.3 staged), 6-row staged tiles for
-// the others (shape 5; FP16 500 x 256: 7.1 against 8.6 on shape 4).  Above,
-// polynomial-f* FP32, bound by memory, keeps the 6-row tiles' three copies in
-// flight (97 at 4096 x 2048, 94 on shape 4); where arithmetic is what bounds
-// a step the 8-row tiles' warps win (shape 4; 4096 x 2048: entropic FP32 115
-// against 131; 2048 x 1024 ELBM 91 against 125), for FP16 from 1e6 sites on
-// (1024 x 600: 10.7 against 9.4; 2048 x 1024: 20 against 24; 4096 x 2048: 68
-// against 84).  FP64 storage: 8-row tiles.  The energy forms: FP64 storage's
+// dominated by latency): register-fed tiles for polynomial-f* FP32 (shape 1),
+// 6-row staged tiles for the others (shape 5; entropic FP16 600 x 500: 7.9
+// against 8.5 on shape 4).  Above, the 8-row tiles' warps win (shape 4) from
+// 1e6 sites on (FP16 and polynomial-f* FP32) or at once: polynomial FP32
+// 1280 x 800: 14.8 against 16.8 on shape 5, 2560 x 1280: 37.1 against 41.3;
+// entropic FP32 4096 x 2048: 94 against 100; entropic FP16 2048 x 1024: 24.7
+// against 26.7; 2048 x 1024 ELBM: 52 against 57.  The largest polynomial-f*
+// FP32 grids, bound by memory, take the 6-row tiles again, whose three copies
+// in flight are as fast within 2 % (3500 x 1750: 69.1 against 68.1).  FP64
+// storage: 8-row tiles.  The energy forms: FP64 storage's
 // solve wants the most resident warps (register-fed shape 1); the
 // float-float solve of FP32 / FP16 storage and the network's warm start run
 // best in the staged shape 4 (measured at 2048 x 1024: Newton start 89 us
@@ -68,7 +69,7 @@ int default_tile_shape(int lattice, int eq, int precision, long long sites, bool
     if (eq < LB_EQ_ENTROPIC_ENERGY) {
         if (precision == LB_F64 || elbm) return 4;
         if (precision == LB_F16_DEV) return sites <= 1000000 ? 5 : 4;
-        if (eq == LB_EQ_POLY) return sites <= 600000 ? 1 : 5;
+        if (eq == LB_EQ_POLY) return sites <= 600000 ? 1 : (sites <= 1000000 || sites > 5000000 ? 5 : 4);
         return sites <= 600000 ? 5 : 4;
     }
     if (precision == LB_F64) return 1;
@@ -173,7 +174,7 @@ struct lb_handle {
     // tensor maps of the two population buffers (shared-memory-staged shapes)
     CUtensorMap tmap[2];
     unsigned* tile_counter;
-    // claim order of the staged shapes' tiles: boundary tiles first; two
+    // claim order of the staged shapes' tiles: those with rows to patch first; two
     // orders of tile_order_n claims, by the parity of the buffer read
     int* tile_order;
     int tile_order_n;

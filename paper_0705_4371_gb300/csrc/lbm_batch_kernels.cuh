@@ -24,7 +24,8 @@ constexpr int kBatchSmemRuns = 256;   // tile bases kept in shared memory (more 
 
 struct BatchShared {
     int abort;
-    int tile[4];   // per stage: item of its run (-1: none left; -2 - e: edge item e)
+    StageRing<4> ring;   // work: items of their runs
+    int next_run[4];     // the run of each stage's next work
     int base[kBatchSmemRuns + 1];   // first item of each run (batches of up to kBatchSmemRuns runs)
     int dims[kBatchSmemRuns][2];    // nx, ny of each run
 };
@@ -63,7 +64,10 @@ __global__ void __launch_bounds__(32 * R, 16 / R) k_collide_batch(const __grid_c
     Params* sp = reinterpret_cast<Params*>(smem + batch_params_offset<S, R, STAGES>());
     MlpSlot<EQ> mslot;   // empty: the batch runs the polynomial and entropic forms
     if (threadIdx.x == 0) {
-        for (int st = 0; st < STAGES; st++) mbar_init(&full[st], 1);
+        for (int st = 0; st < STAGES; st++) {
+            mbar_init(&full[st], 1);
+            sh.ring.done[st] = 0;
+        }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         sh.abort = 0;
     }
@@ -78,89 +82,99 @@ __global__ void __launch_bounds__(32 * R, 16 / R) k_collide_batch(const __grid_c
         }
     __syncthreads();
     const int* tile_base = base_in_smem ? sh.base : A.tile_base;
-    int run_hint = 0;   // tiles are claimed in increasing order: runs only move forward
 
-    // Thread 0 takes the item it claimed at the previous refill and claims
-    // the next (the atomic's latency then overlaps an item's computation),
-    // issues a bulk copy of the item's run parameters into the stage's slot
-    // and the tile's copies, all completing on the stage's mbarrier (-1: no
-    // item left; the phase then completes by a plain arrive).  The run's nx
-    // and ny, which place the tile, come from a table in shared memory.
-    int next_item = 0;   // claimed at the previous refill (the atomic's latency overlaps an item)
-    auto fill = [&](int st) {
-        unsigned long long* bar = &full[st];
-        const int tile = next_item;
-        if (tile >= A.total_tiles) {
-            sh.tile[st] = -1;
-            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+    // Thread 0 claims items one refill ahead (the atomic's latency then
+    // overlaps an item's computation) and publishes the item, as its run's
+    // work, before it leaves the stage that the item will refill.
+    int run_hint = 0;    // thread 0: items are claimed in increasing order, runs only move forward
+    int next_item = 0;
+    auto publish = [&](int st) {
+        const int item = next_item;
+        next_item = (int)atomicAdd(A.tile_counter, 1u);
+        if (item >= A.total_tiles) {
+            sh.ring.next[st] = -1;
             return;
         }
-        next_item = (int)atomicAdd(A.tile_counter, 1u);
-        int lo = run_hint;   // the last run whose first tile is <= tile
-        while (tile_base[lo + 1] <= tile) lo++;
+        int lo = run_hint;   // the last run whose first item is <= item
+        while (tile_base[lo + 1] <= item) lo++;
         run_hint = lo;
         // a run's work: its edge items (the x = 0 and x = nx - 1 columns,
         // 32 R sites each), then its tiles
         const int nx = base_in_smem ? sh.dims[lo][0] : A.P[lo].nx;
         const int ny = base_in_smem ? sh.dims[lo][1] : A.P[lo].ny;
         const int edge_items = ((nx > 1 ? 2 : 1) * ny + 32 * R - 1) / (32 * R);
-        int lt = tile - tile_base[lo];
-        if (lt < edge_items) {
-            sh.tile[st] = -2 - lt;
-            mbar_expect_tx(bar, (unsigned)sizeof(Params));
-            bulk_copy_g2s(sp + st, A.P + lo, (unsigned)sizeof(Params), bar);
+        const int lt = item - tile_base[lo];
+        sh.ring.next[st] = lt < edge_items ? -2 - lt : lt - edge_items;
+        sh.next_run[st] = lo;
+    };
+    // One thread: put the published work into a stage, a bulk copy of its
+    // run's parameters and the tile's copies, all completing on the stage's
+    // mbarrier (no work left: a plain arrive).
+    auto fill = [&](int st) {
+        unsigned long long* bar = &full[st];
+        const int lt = sh.ring.next[st];
+        sh.ring.tile[st] = lt;
+        if (lt == -1) {
+            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
             return;
         }
-        lt -= edge_items;
-        sh.tile[st] = lt;
+        const int run = sh.next_run[st];
+        const int nx = base_in_smem ? sh.dims[run][0] : A.P[run].nx;
         const int tiles_x = (nx + TX - 1) / TX;
         const int ty = lt / tiles_x, tx = lt - ty * tiles_x;
-        mbar_expect_tx(bar, (unsigned)(LY::TX_BYTES + sizeof(Params)));
-        bulk_copy_g2s(sp + st, A.P + lo, (unsigned)sizeof(Params), bar);
+        sh.ring.x0[st] = tx * TX;
+        sh.ring.y0[st] = ty * R;
+        mbar_expect_tx(bar, (unsigned)((lt < 0 ? 0 : LY::TX_BYTES) + sizeof(Params)));
+        bulk_copy_g2s(sp + st, A.P + run, (unsigned)sizeof(Params), bar);
+        if (lt < 0) return;
         S* base = stages + (size_t)st * (LY::STAGE_BYTES / sizeof(S));
 #pragma unroll
         for (int i = 0; i < L::Q; i++)
-            tma_load_3d(base + i * LY::PLANE, A.tm + lo, tx * TX - LY::H, ty * R - L::cy(i), i, bar);
+            tma_load_3d(base + i * LY::PLANE, A.tm + run, tx * TX - LY::H, ty * R - L::cy(i), i, bar);
     };
     if (threadIdx.x == 0) {
         next_item = (int)atomicAdd(A.tile_counter, 1u);
-        for (int st = 0; st < STAGES - 1; st++) fill(st);
+        for (int st = 0; st < STAGES; st++) {
+            publish(st);
+            fill(st);
+        }
     }
-    int jj = 0;
-    for (;; jj++) {
-        const int st = jj % STAGES;
-        const unsigned parity = (unsigned)((jj / STAGES) & 1);
-        // the barrier also ends every warp's reads of the stage and the
-        // parameter slot that thread 0 refills next
-        if (__syncthreads_or(!mbar_wait(&full[st], parity))) {
-            if (threadIdx.x == 0) {
-                for (int q = 0; q < A.nruns; q++) atomicOr(A.P[q].err, ERR_TIMEOUT);
-                sh.abort = 1;
-            }
+    int st = 0;
+    unsigned parity = 0u;
+    for (;;) {
+        // a wait that gives up leaves its stage held, so that every other
+        // warp's wait gives up in turn
+        if (!mbar_wait(&full[st], parity)) {
+            sh.abort = 1;
             break;
         }
-        const int lt = sh.tile[st];
+        const int lt = sh.ring.tile[st];
         if (lt == -1) break;
-        if (threadIdx.x == 0) {
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            fill((jj + STAGES - 1) % STAGES);
-        }
+        if (threadIdx.x == 0) publish(st);
         const Params& P = sp[st];
-        const int tiles_x = (P.nx + TX - 1) / TX;
-        const int ty = lt / tiles_x, tx = lt - ty * tiles_x;
         const long long t = __ldcg(P.step);
         S* box = stages + (size_t)st * (LY::STAGE_BYTES / sizeof(S));
         TileState<GlobalCandSink> state{{}, {0, 0, 0, 0}, false};
         if (lt <= -2) state = edge_item<S, EQ, R>(P, -2 - lt, t, state, mslot);
-        else tma_tile<S, EQ, R, kTmaTX>(P, box, tx * TX, ty * R, t, state, mslot, P);
+        else tma_tile<S, EQ, R, kTmaTX>(P, box, sh.ring.x0[st], sh.ring.y0[st], t, state, mslot, P);
         if (state.nonfinite) atomicOr(P.err, ERR_NONFINITE);
+        __syncwarp();
+        if ((threadIdx.x & 31) == 0 && stage_leave(&sh.ring.done[st], R)) fill(st);
+        if (++st == STAGES) {
+            st = 0;
+            parity ^= 1u;
+        }
     }
     __syncthreads();
     if (sh.abort && threadIdx.x == 0) {
+        for (int q = 0; q < A.nruns; q++) atomicOr(A.P[q].err, ERR_TIMEOUT);
         // wait (bounded) for copies still in flight into every stage
         for (int k2 = 0; k2 < STAGES; k2++) {
-            const int j2 = jj + k2;
-            mbar_wait(&full[j2 % STAGES], (unsigned)((j2 / STAGES) & 1));
+            mbar_wait(&full[st], parity);
+            if (++st == STAGES) {
+                st = 0;
+                parity ^= 1u;
+            }
         }
     }
 }

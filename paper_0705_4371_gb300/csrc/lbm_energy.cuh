@@ -33,7 +33,8 @@
 // a 3 x 3 covariance and its Cholesky factors per iteration, residual sums
 // of nine float-float terms): bound by FP32 issue at about 2000 instructions
 // per site.  2048 x 1024, FP32: 64 us per step against 166 us
-// (three such runs side by side; one alone 89 us against 205 us).
+// (three such runs side by side; one alone 89 us against 205 us), 49 us with
+// two sites per lane in packed arithmetic.
 #pragma once
 
 #include "lbm_device.cuh"

@@ -3,13 +3,15 @@
 //
 //   k_collide_d2q9   the whole time step in one persistent launch: every
 //                    warp walks row tiles of 32 x VEC sites (pull-stream +
-//                    moments + f* + dS + LBGK), appends the sites with
-//                    dS > delta to a global candidate list (warp ballot, one
-//                    atomic per tile that has any), and the block that
-//                    finishes last runs the global radix select of the k
-//                    largest dS and the Ehrenfests' step f <- f* at those
-//                    sites (Sec. 3.2; (ESLB)).  No block waits for another.
+//                    moments + f* + dS + LBGK), the block keeps the k best
+//                    of its sites with dS > delta, and the block that
+//                    finishes last selects the k largest dS of all blocks'
+//                    and makes the Ehrenfests' step f <- f* at those sites
+//                    (Sec. 3.2; (ESLB)).  No block waits for another.
+//   k_collide_d2q9_tma   the same step with the sources of block tiles
+//                    staged in shared memory by bulk tensor copies
 //   k_collide_site   the same step, one site per thread (D1Q3)
+//   k_tube           many steps of a short D1Q3 run in one launch (one cluster)
 //   k_select         the selection as a stand-alone kernel (test hook)
 #pragma once
 
@@ -594,7 +596,7 @@ __device__ __forceinline__ unsigned block_push(const Params& P, BlockCandT<CAP>&
             bc.key[slot] = key;
             bc.idx[slot] = site;
         } else {
-            // no room (the callers cut or flush before it can happen)
+            // no room (the global list has room for every site)
             const unsigned g = atomicAdd(P.cand_count, 1u);
             P.cand_key[g] = key;
             P.cand_idx[g] = site;
@@ -1291,11 +1293,42 @@ constexpr int tma_cand_cap() {
     return TX * R + kBlockCand;
 }
 
+// The stages of a staged block, handed on without a barrier of the block: a
+// warp that has finished with a stage's tile says so (done), and the one that
+// finishes last refills the stage at once with the work thread 0 has claimed
+// for it (next).  A warp therefore never waits for the others, only for its
+// next tile's copies, and every stage but those being computed is in flight.
+// With one barrier per tile instead (every warp waiting for the slowest, one
+// stage idle), barriers were the largest stall (FP16: 2.6 of 11 cycles per
+// issue, now 0.5).  us per step, exports shared out, before and now: 4096 x
+// 2048 polynomial FP32 96.9, 94.1; FP16 71.2, 70.3; 2048 x 1024 FP64 300,
+// 289; ELBM 56.2, 55.1; energy 49.9, 48.7; 64 runs in one launch 431, 421.
+template <int N>
+struct StageRing {
+    int tile[N];   // work a stage holds (-1: none left; -2 - e: edge item e)
+    int x0[N], y0[N];   // the tile's origin
+    int next[N];   // work for the stage's next refill
+    int done[N];   // warps that have finished with the stage's work
+};
+
+// The calling warp has finished with a stage (lane 0 calls, after a
+// __syncwarp): true for the last of n warps, which sees the others' accesses
+// as done and refills the stage.
+__device__ __forceinline__ bool stage_leave(int* done, int n) {
+    int before;
+    asm volatile("atom.acq_rel.cta.shared::cta.add.u32 %0, [%1], 1;" : "=r"(before) : "r"(smem_u32(done)) : "memory");
+    if (before != n - 1) return false;
+    *done = 0;
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    return true;
+}
+
 // Shared state of a staged block besides its tiles.  p: the launch's
 // parameters, for the out-of-line paths (a reference to the kernel's
 // __grid_constant__ parameter passed to a function that is not inlined
 // reads it through generic loads of the parameter space; the shared copy
 // answers at shared-memory latency).
+constexpr unsigned kCutAsked = 0x80000000u;
 template <int CAP>
 struct TmaShared {
     Params p;
@@ -1303,12 +1336,13 @@ struct TmaShared {
     BlockCandT<CAP> bc;
     int is_last;
     int abort;
-    int tile[8];   // tile held by each stage (-1: none left)
+    unsigned begun;   // the last work any warp has begun (its ordinal); kCutAsked: cut before the next
+    StageRing<8> ring;
 };
 
 template <typename S, int R, int STAGES, int EQ, int TX = kTmaTX>
 constexpr size_t tma_smem_bytes() {
-    return 128 + (size_t)STAGES * TmaLayout<S, R, TX>::STAGE_BYTES + 8 * STAGES +
+    return 128 + (size_t)STAGES * TmaLayout<S, R, TX>::STAGE_BYTES + 8 * (STAGES + 1) +
            sizeof(TmaShared<tma_cand_cap<R, TX>()>) + 16 +
            (EQ == EQ_ENERGY_MLP ? sizeof(MlpSlot<EQ>) + 16 : 0);
 }
@@ -1323,10 +1357,9 @@ constexpr size_t tma_smem_bytes() {
 template <int CAP>
 struct CandSink {
     BlockCandT<CAP>* bc;
-    unsigned count;
     template <typename T>
     __device__ __forceinline__ void put(const Params& P, T ds, unsigned site) {
-        count += block_push<T>(P, *bc, ds > Par<T>::delta(P), ds, site);
+        block_push<T>(P, *bc, ds > Par<T>::delta(P), ds, site);
     }
 };
 struct GlobalCandSink {
@@ -1798,13 +1831,20 @@ __device__ __forceinline__ void tma_tile(const Params& P, S* box, int x0, int y0
 }
 // Resident blocks per SM the staged kernel is compiled for: two in general
 // (128 registers per thread with 8-row tiles, 170 with 6-row tiles); three
-// (85 registers per thread) where the tiles take half the shared memory:
-// FP16 storage, or FP32 tiles 64 sites wide.
+// (85 registers per thread) for FP32 tiles 64 sites wide, which take half the
+// shared memory.
 template <typename S, int EQ, int R, int TX>
 constexpr int tma_min_blocks() {
     if (EQ >= EQ_ENERGY) return 2;   // (the packed solve spills at 85)
-    return (sizeof(S) == 2 && R == 8) || (sizeof(S) == 4 && TX == 64 && R == 8) ? 3 : 2;
+    return sizeof(S) == 4 && TX == 64 && R == 8 ? 3 : 2;
 }
+
+// Stages of the 8-row tiles: two fill the shared memory two blocks share; FP16
+// storage has room for a third (us per step of two runs side by side, 4096 x
+// 2048, polynomial f*: 65.6; two stages and three blocks, 85 registers: 69.0;
+// four stages: 67.1; entropic f*: 86.0; 130.6; 91.3).
+template <typename S>
+constexpr int kStages8 = sizeof(S) == 2 ? 3 : 2;
 
 template <typename S, int EQ, int R, int STAGES, int TX = kTmaTX>
 __global__ void __launch_bounds__(32 * R, tma_min_blocks<S, EQ, R, TX>())
@@ -1816,48 +1856,52 @@ __global__ void __launch_bounds__(32 * R, tma_min_blocks<S, EQ, R, TX>())
     unsigned char* smem = smem_raw + ((128 - (smem_u32(smem_raw) & 127)) & 127);
     S* stages = reinterpret_cast<S*>(smem);
     unsigned long long* full = reinterpret_cast<unsigned long long*>(smem + STAGES * LY::STAGE_BYTES);
+    unsigned long long* gather = full + STAGES;   // the warps' rendezvous before a cut
     constexpr int kCap = tma_cand_cap<R, TX>();
-    constexpr int kRoom = kCap - TX * R;   // what the buffer holds at the top of a tile
+    constexpr int kRoom = kCap - TX * R;
     using Shared = TmaShared<kCap>;
-    Shared& sh = *reinterpret_cast<Shared*>(smem + STAGES * LY::STAGE_BYTES + 8 * STAGES);
-    constexpr size_t kMlpOff = (STAGES * LY::STAGE_BYTES + 8 * STAGES + sizeof(Shared) + 15) / 16 * 16;
+    Shared& sh = *reinterpret_cast<Shared*>(smem + STAGES * LY::STAGE_BYTES + 8 * (STAGES + 1));
+    constexpr size_t kMlpOff = (STAGES * LY::STAGE_BYTES + 8 * (STAGES + 1) + sizeof(Shared) + 15) / 16 * 16;
     MlpSlot<EQ>& mslot = *reinterpret_cast<MlpSlot<EQ>*>(smem + kMlpOff);
     if (threadIdx.x == 0) {
-        for (int st = 0; st < STAGES; st++) mbar_init(&full[st], 1);
+        for (int st = 0; st < STAGES; st++) {
+            mbar_init(&full[st], 1);
+            sh.ring.done[st] = 0;
+        }
+        mbar_init(gather, R);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         sh.p = P;
         sh.abort = 0;
+        sh.begun = 0u;
         sh.bc.n = 0;
     }
     const int tiles_x = (P.nx + TX - 1) / TX;
     const int tiles = tiles_x * ((P.ny + R - 1) / R);
     // the x = 0 and x = nx - 1 columns go first, as edge items of 32 R sites
     const int edge_items = ((P.nx > 1 ? 2 : 1) * P.ny + 32 * R - 1) / (32 * R);
-    const int claims = edge_items + tiles;
 
     // Work is handed out by claims: claim c < edge_items is edge item c, the
-    // others tile tile_order[c - edge_items] (boundary tiles spread over the
-    // first claims) or c - edge_items.  Thread 0 refills a
-    // stage with the work it claimed at the previous refill and claims the
-    // next (the latencies of the atomic and of the order entry then overlap
-    // a tile's computation), and publishes it with the stage's mbarrier:
-    // the tile's index, -2 - e for edge item e, -1 when none is left (the
-    // phase is then completed by a plain arrive, without a copy, as for an
-    // edge item).
-    // A block's first STAGES claims are fixed (b, b + G, b + 2 G, ... for
-    // block b of G): the pipeline fills without waiting for the atomic; the
-    // counter hands out the claims from STAGES G on.
-    int next_claim = 0, next_tile = 0, fixed = 0;
-    auto claim = [&]() {
-        if (fixed < STAGES) next_claim = (int)blockIdx.x + fixed++ * (int)gridDim.x;
-        else next_claim = (int)atomicAdd(P.tile_counter, 1u) + STAGES * (int)gridDim.x;
-        const int c = next_claim - edge_items;
-        next_tile = c < 0 ? -2 - next_claim : c;
-        if (P.tile_order && c >= 0 && c < tiles) next_tile = __ldg(P.tile_order + c);
+    // others tile tile_order[c - edge_items] (the tiles with rows to patch
+    // first) or c - edge_items.  A block's first STAGES claims are fixed
+    // (b, b + G, b + 2 G, ... for block b of G): the pipeline fills without
+    // waiting for the atomic; the counter hands out the claims from STAGES G
+    // on.  Thread 0 claims two refills ahead and reads the claim's order
+    // entry one ahead (both latencies then overlap a tile's computation), and
+    // publishes it before it leaves the stage it will refill.
+    int claimed = 0;   // thread 0: a claim
+    int next = 0;      // thread 0: the claim before it, as work: a tile, -2 - e for edge item e, -1 for none
+    auto resolve = [&]() {
+        const int c = claimed - edge_items;
+        next = c < 0 ? -2 - claimed : c < tiles ? c : -1;
+        if (P.tile_order && c >= 0 && c < tiles) next = __ldg(P.tile_order + c);
     };
     if (threadIdx.x == 0) {
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<unsigned long long>(&tm)) : "memory");
-        claim();
+        for (int st = 0; st < STAGES; st++) {
+            claimed = (int)blockIdx.x + st * (int)gridDim.x;
+            resolve();
+            sh.ring.next[st] = next;
+        }
     }
     // Launched as a programmatic dependent of the previous kernel in the
     // stream: the block may start while that kernel finishes, and the code
@@ -1872,77 +1916,102 @@ __global__ void __launch_bounds__(32 * R, tma_min_blocks<S, EQ, R, TX>())
     __syncthreads();
     const long long t = *P.step;
 
+    auto claim = [&]() { claimed = (int)atomicAdd(P.tile_counter, 1u) + STAGES * (int)gridDim.x; };
+    // One thread: put the claimed work into a stage (the phase of an edge
+    // item, or of no work, is completed by a plain arrive, without a copy).
     auto fill = [&](int st) {
         unsigned long long* bar = &full[st];
-        if (next_claim >= claims || next_tile < 0) {
-            sh.tile[st] = next_claim >= claims ? -1 : next_tile;
-            if (next_claim < claims) claim();
+        const int tile = sh.ring.next[st];
+        sh.ring.tile[st] = tile;
+        if (tile < 0) {
             asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
             return;
         }
-        const int tile = next_tile;
-        claim();
-        sh.tile[st] = tile;
         const int ty = tile / tiles_x, tx = tile - ty * tiles_x;
+        sh.ring.x0[st] = tx * TX;
+        sh.ring.y0[st] = ty * R;
         mbar_expect_tx(bar, (unsigned)LY::TX_BYTES);
         S* base = stages + (size_t)st * (LY::STAGE_BYTES / sizeof(S));
 #pragma unroll
         for (int i = 0; i < L::Q; i++)
             tma_load_3d(base + i * LY::PLANE, &tm, tx * TX - LY::H, ty * R - L::cy(i), i, bar);
     };
-    if (threadIdx.x == 0)
-        for (int st = 0; st < STAGES - 1; st++) fill(st);
+    if (threadIdx.x == 0) {
+        for (int st = 0; st < STAGES; st++) fill(st);
+        claim();
+        resolve();
+        claim();
+    }
     // The sites the dS bound does not clear are resolved as they are
-    // updated; the candidates go to the block's buffer, which the block cuts
-    // to its k best between tiles.  A cut happens once some warp appended
-    // more than its share (1 / R) of the room above what a cut keeps: the
-    // buffer then never holds more than kRoom entries at the top of a tile,
-    // and one tile adds at most TX * R.
+    // updated; the candidates go to the block's buffer.  A warp that finds it
+    // filling up asks for a cut: before the first work that no warp has begun
+    // by then, the warps meet and cut the buffer to its k best (or flush it,
+    // where k does not fit).  The warps are at most STAGES tiles apart; what
+    // a tile begun before the cut finds no room for goes to the global list.
     const int kept = P.k > 0 && P.k < kRoom ? P.k : 0;
-    const unsigned share = (unsigned)((kRoom - kept) / R);
-    TileState<CandSink<kCap>> state{{&sh.bc, 0u}, {0, 0, 0, 0}, false};
-    int jj = 0;
-    for (;; jj++) {
-        const int st = jj % STAGES;
-        const unsigned parity = (unsigned)((jj / STAGES) & 1);
-        // every thread waits.  One vote decides, for every warp at once, to
-        // stop (a wait that gave up anywhere: abort is written before the
-        // barrier only) or to cut the candidates (a warp's count is its own),
-        // so that the barriers stay matched
-        const bool ok = mbar_wait(&full[st], parity);
-        if (!ok) sh.abort = 1;
-        if (__syncthreads_or(!ok || state.sink.count > share)) {
-            if (sh.abort) {
-                if (threadIdx.x == 0) atomicOr(P.err, ERR_TIMEOUT);
+    const unsigned cut_above = (unsigned)(kept + (kRoom - kept) / 2);
+    TileState<CandSink<kCap>> state{{&sh.bc}, {0, 0, 0, 0}, false};
+    int st = 0;
+    unsigned parity = 0u, cuts = 0u;
+    for (unsigned jj = 1u;; jj++) {
+        // one atomic both announces the work as begun and finds a cut asked
+        // for before it (the asking bit outranks every ordinal, and freezes
+        // the one it found), so every warp cuts before the same work; its
+        // latency passes with the wait
+        unsigned begun = 0u;
+        if ((threadIdx.x & 31) == 0) begun = atomicMax(&sh.begun, jj);
+        // a wait that gives up (here or below) leaves its stage held, so that
+        // every other warp's wait gives up in turn
+        if (!mbar_wait(&full[st], parity)) {
+            sh.abort = 1;
+            break;
+        }
+        const int tile = sh.ring.tile[st];
+        if (tile == -1) break;
+        if (threadIdx.x == 0) {
+            sh.ring.next[st] = next;
+            resolve();
+            claim();
+        }
+        begun = __shfl_sync(0xffffffffu, begun, 0);
+        if (begun >= kCutAsked && jj > (begun & ~kCutAsked)) {
+            if ((threadIdx.x & 31) == 0)
+                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(gather)) : "memory");
+            if (!mbar_wait(gather, cuts++ & 1u)) {
+                sh.abort = 1;
                 break;
             }
             if (P.k < kRoom) block_cut(sh.bc, sh.ss.sc, P.k);
             else block_flush(sh.p, sh.bc);
-            state.sink.count = 0;
-        }
-        const int tile = sh.tile[st];
-        if (tile == -1) break;
-        if (threadIdx.x == 0) {
-            // the stage being refilled was last read in iteration jj - 1,
-            // whose reads the barrier at the top of this iteration ordered
-            // before this point
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            fill((jj + STAGES - 1) % STAGES);
+            if (threadIdx.x == 0) sh.begun = jj;
+            __syncthreads();
         }
         if (tile <= -2) {
             state = edge_item<S, EQ, R>(sh.p, -2 - tile, t, state, mslot);
-            continue;
+        } else {
+            S* box = stages + (size_t)st * (LY::STAGE_BYTES / sizeof(S));
+            tma_tile<S, EQ, R, TX>(P, box, sh.ring.x0[st], sh.ring.y0[st], t, state, mslot, sh.p);
         }
-        const int ty = tile / tiles_x, tx = tile - ty * tiles_x;
-        S* box = stages + (size_t)st * (LY::STAGE_BYTES / sizeof(S));
-        tma_tile<S, EQ, R, TX>(P, box, tx * TX, ty * R, t, state, mslot, sh.p);
+        __syncwarp();
+        if ((threadIdx.x & 31) == 0) {
+            if (sh.bc.n > cut_above) atomicOr(&sh.begun, kCutAsked);
+            if (stage_leave(&sh.ring.done[st], R)) fill(st);
+        }
+        if (++st == STAGES) {
+            st = 0;
+            parity ^= 1u;
+        }
     }
     __syncthreads();
     if (sh.abort && threadIdx.x == 0) {
+        atomicOr(P.err, ERR_TIMEOUT);
         // wait (bounded) for copies still in flight into every stage
         for (int k2 = 0; k2 < STAGES; k2++) {
-            const int j2 = jj + k2;
-            mbar_wait(&full[j2 % STAGES], (unsigned)((j2 / STAGES) & 1));
+            mbar_wait(&full[st], parity);
+            if (++st == STAGES) {
+                st = 0;
+                parity ^= 1u;
+            }
         }
     }
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -2517,7 +2586,7 @@ __global__ void k_ghost(const __grid_constant__ Params P, S* field, int col, int
 // thread in x, warps per block, minimum resident blocks per SM):
 //   0: 1, 8, 3     1: 1, 8, 4     2: 2, 8, 2     3: 4, 8, 1
 // and of the staged kernel (rows x columns per block tile, tiles in flight):
-//   4: 8 x 128, 2     5: 6 x 128, 3     6: 8 x 64, 2
+//   4: 8 x 128, 2 (FP16: 3)     5: 6 x 128, 3     6: 8 x 64, 2
 // The persistent grid is (resident blocks per SM) x (SM count), from the
 // occupancy calculator, capped by the number of tiles (small grids then
 // spread over as many SMs as they have tiles: their step is latency-bound).
@@ -2584,7 +2653,7 @@ struct LaunchImpl {
             // two staged shapes (5: 6-row tiles, 168 registers; 4: 8-row
             // tiles, 128); shape 6 is refused for them by the host
             if (shape == 5) return launch_d2q9_tma<S, EQ, 6, 3>(P, tmap, st);
-            if (shape == 4) return launch_d2q9_tma<S, EQ, 8, 2>(P, tmap, st);
+            if (shape == 4) return launch_d2q9_tma<S, EQ, 8, kStages8<S>>(P, tmap, st);
             if (shape == 0) return launch_d2q9<S, EQ, 1, 8, 2>(P, st);
             return launch_d2q9<S, EQ, 1, 8, 4>(P, st);
         } else if constexpr (L::Q == 9) {
@@ -2592,7 +2661,7 @@ struct LaunchImpl {
                 case 1: return launch_d2q9<S, EQ, 1, 8, 4>(P, st);
                 case 2: return launch_d2q9<S, EQ, 2, 8, 2>(P, st);
                 case 3: return launch_d2q9<S, EQ, 4, 8, 1>(P, st);
-                case 4: return launch_d2q9_tma<S, EQ, 8, 2>(P, tmap, st);
+                case 4: return launch_d2q9_tma<S, EQ, 8, kStages8<S>>(P, tmap, st);
                 case 5: return launch_d2q9_tma<S, EQ, 6, 3>(P, tmap, st);
                 case 6: return launch_d2q9_tma<S, EQ, 8, 2, 64>(P, tmap, st);
                 default: return launch_d2q9<S, EQ, 1, 8, 3>(P, st);
@@ -2663,7 +2732,7 @@ struct LaunchImpl {
         *per_sm = 1;
         if constexpr (L::Q == 9 && EQ >= EQ_ENERGY) {
             if (shape == 5) return setup_d2q9_tma<S, EQ, 6, 3>(per_sm);
-            if (shape == 4) return setup_d2q9_tma<S, EQ, 8, 2>(per_sm);
+            if (shape == 4) return setup_d2q9_tma<S, EQ, 8, kStages8<S>>(per_sm);
             if (shape == 0) return occupancy_d2q9<S, EQ, 1, 8, 2>(per_sm);
             return occupancy_d2q9<S, EQ, 1, 8, 4>(per_sm);
         } else if constexpr (L::Q == 9) {
@@ -2671,7 +2740,7 @@ struct LaunchImpl {
                 case 1: return occupancy_d2q9<S, EQ, 1, 8, 4>(per_sm);
                 case 2: return occupancy_d2q9<S, EQ, 2, 8, 2>(per_sm);
                 case 3: return occupancy_d2q9<S, EQ, 4, 8, 1>(per_sm);
-                case 4: return setup_d2q9_tma<S, EQ, 8, 2>(per_sm);
+                case 4: return setup_d2q9_tma<S, EQ, 8, kStages8<S>>(per_sm);
                 case 5: return setup_d2q9_tma<S, EQ, 6, 3>(per_sm);
                 case 6: return setup_d2q9_tma<S, EQ, 8, 2, 64>(per_sm);
                 default: return occupancy_d2q9<S, EQ, 1, 8, 3>(per_sm);
