@@ -9,7 +9,8 @@
 // idle tails per run.  A tile's sites go through the same per-site update
 // as a single run (tma_tile); the sites the dS bound does not clear are
 // resolved in place, and the candidates go straight to their run's global
-// list.  One block barrier per item.  A second launch (k_batch_select, one
+// list.  The stages are handed on by the warps that finish with them, without
+// a barrier of the block (StageRing).  A second launch (k_batch_select, one
 // block per run) then runs every run's selection and Ehrenfests' step
 // (Sec. 3.2) and resets the step's item counter.
 #pragma once

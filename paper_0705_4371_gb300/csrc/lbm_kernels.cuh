@@ -1227,9 +1227,8 @@ __global__ void __launch_bounds__(32 * WARPS, MINB) k_collide_d2q9(const __grid_
 // flight per block, so the bytes in flight do not depend on registers.
 // Warp w computes row w of the tile, lane l the site pairs x0 + 2 l + 64 s,
 // + 1: shared-memory reads and global stores are both consecutive across the
-// warp.  In tiles that touch the y sides or the obstacle the sites use the
-// rule-by-rule gather, from shared memory where the source lies in its
-// plane's window and from the source field otherwise; the x = 0 and
+// warp.  In rows at the y sides or the obstacle, patch_row first writes what
+// the boundary rules replace into the staged planes; the x = 0 and
 // x = nx - 1 columns are edge items of their own.  Every wait on an
 // mbarrier is bounded: on expiry the block flags ERR_TIMEOUT, stops issuing
 // copies, waits (bounded) for the copies it issued, and ends.
@@ -1287,7 +1286,8 @@ struct TmaLayout {
 };
 
 // Candidate buffer of a staged block: room for one tile's sites above what
-// a cut keeps (the block cuts between tiles).
+// a cut keeps (the block cuts between tiles; the global list, which has a
+// slot per site, takes what a tile begun before a cut finds no room for).
 template <int R, int TX>
 constexpr int tma_cand_cap() {
     return TX * R + kBlockCand;
@@ -1675,7 +1675,7 @@ __device__ __noinline__ void patch_row(const Params& P, S* box, int x0, int y) {
             }
         }
     }
-    // the stage is refilled by the async proxy after the block's next barrier
+    // the stage is refilled by the async proxy after every warp has left it
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncwarp();
 }
@@ -1821,8 +1821,8 @@ __device__ __forceinline__ void tma_tile(const Params& P, S* box, int x0, int y0
         }
         pmask |= (pend & ((ea ? 0u : 1u) | (eb ? 0u : 2u))) << (2 * s);
     }
-    // the row's pending sites, from the staged planes (valid until the
-    // next tile's barrier), out of line: the update keeps its registers
+    // the row's pending sites, from the staged planes (valid until the warp
+    // leaves the stage), out of line: the update keeps its registers
     if (__any_sync(0xffffffffu, pmask != 0u))
         state.sink = resolve_staged_row<S, EQ, R, TX>(Pc, box, x0, y, pmask, state.sink);
     if (P.probe_ring && y == P.probe_y && lane == 0 && P.probe_x >= x0 && P.probe_x < x0 + TX &&
