@@ -605,14 +605,22 @@ __device__ __forceinline__ unsigned block_push(const Params& P, BlockCandT<CAP>&
     return (unsigned)__popc(m);
 }
 
-// Keep the k best of the buffer (all threads call; blockDim >= 128).
+// Keep the k best of the buffer (all threads call; blockDim >= 128, or at most
+// kPer entries per thread).  This and block_flush below return past a barrier
+// that follows every thread's read of the count, so that a caller may go on to
+// append at once: otherwise a warp that returned early could raise the count
+// before a slower one has read it, and the two would take different branches,
+// and barriers, from there on.
 template <int CAP>
 __device__ __noinline__ void block_cut(BlockCandT<CAP>& bc, TopkScratch& sc, int k) {
     constexpr int kPer = (CAP + 127) / 128;
     const int tid = threadIdx.x, nt = blockDim.x;
     __syncthreads();
     const int n = (int)min(bc.n, (unsigned)CAP);
-    if (n <= k) return;   // uniform: n was read after the barrier
+    if (n <= k) {   // uniform: n was read after the barrier
+        __syncthreads();
+        return;
+    }
     const Thresh th = block_topk(sc, n, k, [&](int e) { return bc.key[e]; }, [&](int e) { return bc.idx[e]; });
     unsigned long long kk[kPer];
     unsigned ii[kPer];
@@ -643,7 +651,10 @@ template <int CAP>
 __device__ __noinline__ void block_flush(const Params& P, BlockCandT<CAP>& bc) {
     __syncthreads();
     const int n = (int)min(bc.n, (unsigned)CAP);
-    if (n == 0) return;   // uniform
+    if (n == 0) {   // uniform
+        __syncthreads();
+        return;
+    }
     if (threadIdx.x == 0) bc.base = atomicAdd(P.cand_count, (unsigned)n);
     __syncthreads();
     const unsigned base = bc.base;
@@ -659,9 +670,11 @@ __device__ __noinline__ void block_flush(const Params& P, BlockCandT<CAP>& bc) {
 // Make room for another blockDim candidates (all threads call).
 template <int CAP>
 __device__ __forceinline__ void block_room(const Params& P, BlockCandT<CAP>& bc, TopkScratch& sc) {
-    __syncthreads();
     const int room = CAP - (int)blockDim.x;
-    if ((int)bc.n > room) {   // uniform
+    __syncthreads();
+    const bool full = (int)bc.n > room;
+    __syncthreads();   // every thread has read the count before any appends
+    if (full) {   // uniform
         if (P.k <= room) block_cut(bc, sc, P.k);
         else block_flush(P, bc);
     }
