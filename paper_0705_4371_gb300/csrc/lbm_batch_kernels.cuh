@@ -143,9 +143,9 @@ __global__ void __launch_bounds__(32 * R, 16 / R) k_collide_batch(const __grid_c
     int st = 0;
     unsigned parity = 0u;
     for (;;) {
-        // a wait that gives up leaves its stage held, so that every other
+        // a warp whose wait gives up leaves its stage held, so that every other
         // warp's wait gives up in turn
-        if (!mbar_wait(&full[st], parity)) {
+        if (!warp_wait(&full[st], parity)) {
             sh.abort = 1;
             break;
         }

@@ -21,6 +21,7 @@
 #include <cuda.h>
 
 #include "lbm_device.cuh"
+#include "lbm_rendezvous.h"
 #include "lbm_energy.cuh"
 #include "lbm_mlp.cuh"
 #include "lbm_internal.h"
@@ -1277,6 +1278,11 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long* bar, unsigned pari
         if (mbar_try_wait(bar, parity)) return true;
     return false;
 }
+// The same for a whole warp (every lane calls): false on every lane when any
+// lane's wait gave up, so that the warp leaves, or goes on, as one.
+__device__ __forceinline__ bool warp_wait(unsigned long long* bar, unsigned parity) {
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity));
+}
 __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* tm, int c0, int c1, int c2,
                                             unsigned long long* bar) {
     asm volatile(
@@ -1350,6 +1356,7 @@ struct TmaShared {
     int is_last;
     int abort;
     unsigned begun;   // the last work any warp has begun (its ordinal); kCutAsked: cut before the next
+    unsigned met;     // outcome of the warps' rendezvous before a cut (rendezvous_met)
     StageRing<8> ring;
 };
 
@@ -1886,6 +1893,7 @@ __global__ void __launch_bounds__(32 * R, tma_min_blocks<S, EQ, R, TX>())
         sh.p = P;
         sh.abort = 0;
         sh.begun = 0u;
+        sh.met = 0u;
         sh.bc.n = 0;
     }
     const int tiles_x = (P.nx + TX - 1) / TX;
@@ -1973,9 +1981,9 @@ __global__ void __launch_bounds__(32 * R, tma_min_blocks<S, EQ, R, TX>())
         // latency passes with the wait
         unsigned begun = 0u;
         if ((threadIdx.x & 31) == 0) begun = atomicMax(&sh.begun, jj);
-        // a wait that gives up (here or below) leaves its stage held, so that
-        // every other warp's wait gives up in turn
-        if (!mbar_wait(&full[st], parity)) {
+        // a warp whose wait gives up (here or below) leaves its stage held, so
+        // that every other warp's wait gives up in turn
+        if (!warp_wait(&full[st], parity)) {
             sh.abort = 1;
             break;
         }
@@ -1990,10 +1998,17 @@ __global__ void __launch_bounds__(32 * R, tma_min_blocks<S, EQ, R, TX>())
         if (begun >= kCutAsked && jj > (begun & ~kCutAsked)) {
             if ((threadIdx.x & 31) == 0)
                 asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(gather)) : "memory");
-            if (!mbar_wait(gather, cuts++ & 1u)) {
+            // one outcome for the block, also where some warps' waits gave up
+            // and the others' did not: the cut's barriers need every warp
+            const bool met = warp_wait(gather, cuts & 1u);
+            bool cut = false;
+            if ((threadIdx.x & 31) == 0)
+                cut = rendezvous_met(met, cuts, [&](unsigned e, unsigned d) { return atomicCAS(&sh.met, e, d); });
+            if (!__shfl_sync(0xffffffffu, (int)cut, 0)) {
                 sh.abort = 1;
                 break;
             }
+            cuts++;
             if (P.k < kRoom) block_cut(sh.bc, sh.ss.sc, P.k);
             else block_flush(sh.p, sh.bc);
             if (threadIdx.x == 0) sh.begun = jj;
