@@ -1347,7 +1347,7 @@ __device__ __forceinline__ bool stage_leave(int* done, int n) {
 // __grid_constant__ parameter passed to a function that is not inlined
 // reads it through generic loads of the parameter space; the shared copy
 // answers at shared-memory latency).
-constexpr unsigned kCutAsked = 0x80000000u;
+constexpr unsigned kCutAsked = 0x80000000u, kGaveUp = 0xffffffffu;
 template <int CAP>
 struct TmaShared {
     Params p;
@@ -1982,8 +1982,12 @@ __global__ void __launch_bounds__(32 * R, tma_min_blocks<S, EQ, R, TX>())
         unsigned begun = 0u;
         if ((threadIdx.x & 31) == 0) begun = atomicMax(&sh.begun, jj);
         // a warp whose wait gives up (here or below) leaves its stage held, so
-        // that every other warp's wait gives up in turn
-        if (!warp_wait(&full[st], parity)) {
+        // that every other warp's wait gives up in turn; the one reduction
+        // hands lane 0's finding to the warp and makes a lane's expired wait
+        // the warp's (kGaveUp outranks every finding)
+        if (!mbar_wait(&full[st], parity)) begun = kGaveUp;
+        begun = __reduce_max_sync(0xffffffffu, begun);
+        if (begun == kGaveUp) {
             sh.abort = 1;
             break;
         }
@@ -1994,7 +1998,6 @@ __global__ void __launch_bounds__(32 * R, tma_min_blocks<S, EQ, R, TX>())
             resolve();
             claim();
         }
-        begun = __shfl_sync(0xffffffffu, begun, 0);
         if (begun >= kCutAsked && jj > (begun & ~kCutAsked)) {
             if ((threadIdx.x & 31) == 0)
                 asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(gather)) : "memory");
