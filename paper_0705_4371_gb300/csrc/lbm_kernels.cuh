@@ -916,7 +916,11 @@ __device__ __noinline__ PopArr<L::Q, typename Store<S>::T> gather_ruled(const Pa
 }
 
 // ---------------------------------------------------------------------------
-// Vector loads and stores of VEC consecutive populations (aligned).
+// Vector loads and stores of VEC consecutive populations (aligned).  Ordinary
+// loads throughout, and no __restrict__ on the source field: a kernel launched
+// as a programmatic dependent is alive while its predecessor still writes the
+// field it will read, so the read-only data path (__ldg) is not for it, and a
+// read-only promise would let a load move above griddepcontrol.wait.
 // ---------------------------------------------------------------------------
 template <typename S, int VEC> struct VecIO;
 template <typename S> struct VecIO<S, 1> {
@@ -929,7 +933,7 @@ template <typename S> struct VecIO<S, 1> {
 };
 template <> struct VecIO<float, 4> {
     __device__ static void load(const void* p, long long i, float* v) {
-        const float4 a = __ldg(reinterpret_cast<const float4*>(static_cast<const float*>(p) + i));
+        const float4 a = *reinterpret_cast<const float4*>(static_cast<const float*>(p) + i);
         v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
     }
     __device__ static void store(void* p, long long i, const float* v) {
@@ -938,7 +942,7 @@ template <> struct VecIO<float, 4> {
 };
 template <> struct VecIO<float, 2> {
     __device__ static void load(const void* p, long long i, float* v) {
-        const float2 a = __ldg(reinterpret_cast<const float2*>(static_cast<const float*>(p) + i));
+        const float2 a = *reinterpret_cast<const float2*>(static_cast<const float*>(p) + i);
         v[0] = a.x; v[1] = a.y;
     }
     __device__ static void store(void* p, long long i, const float* v) {
@@ -948,7 +952,7 @@ template <> struct VecIO<float, 2> {
 template <> struct VecIO<double, 4> {
     __device__ static void load(const void* p, long long i, double* v) {
         const double2* q = reinterpret_cast<const double2*>(static_cast<const double*>(p) + i);
-        const double2 a = __ldg(q), b = __ldg(q + 1);
+        const double2 a = q[0], b = q[1];
         v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
     }
     __device__ static void store(void* p, long long i, const double* v) {
@@ -959,7 +963,7 @@ template <> struct VecIO<double, 4> {
 };
 template <> struct VecIO<double, 2> {
     __device__ static void load(const void* p, long long i, double* v) {
-        const double2 a = __ldg(reinterpret_cast<const double2*>(static_cast<const double*>(p) + i));
+        const double2 a = *reinterpret_cast<const double2*>(static_cast<const double*>(p) + i);
         v[0] = a.x; v[1] = a.y;
     }
     __device__ static void store(void* p, long long i, const double* v) {
@@ -968,7 +972,7 @@ template <> struct VecIO<double, 2> {
 };
 template <> struct VecIO<__half, 4> {
     __device__ static void load(const void* p, long long i, float* v) {
-        const uint2 a = __ldg(reinterpret_cast<const uint2*>(static_cast<const __half*>(p) + i));
+        const uint2 a = *reinterpret_cast<const uint2*>(static_cast<const __half*>(p) + i);
         const float2 lo = __half22float2(*reinterpret_cast<const __half2*>(&a.x));
         const float2 hi = __half22float2(*reinterpret_cast<const __half2*>(&a.y));
         v[0] = lo.x; v[1] = lo.y; v[2] = hi.x; v[3] = hi.y;
@@ -984,7 +988,7 @@ template <> struct VecIO<__half, 4> {
 };
 template <> struct VecIO<__half, 2> {
     __device__ static void load(const void* p, long long i, float* v) {
-        const unsigned a = __ldg(reinterpret_cast<const unsigned*>(static_cast<const __half*>(p) + i));
+        const unsigned a = *reinterpret_cast<const unsigned*>(static_cast<const __half*>(p) + i);
         const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&a));
         v[0] = f.x; v[1] = f.y;
     }
@@ -1047,7 +1051,7 @@ template <> struct PairIO<double> {
 // Interior-path accessors with 32-bit element indices (every population
 // array holds fewer than 2^31 elements; checked at creation).
 template <typename S, int VEC>
-__device__ __forceinline__ void load_vec(const S* __restrict__ p, int i, typename Store<S>::T* v) {
+__device__ __forceinline__ void load_vec(const S* p, int i, typename Store<S>::T* v) {
     VecIO<S, VEC>::load(p + i, 0, v);
 }
 template <typename S, int VEC>
@@ -1113,7 +1117,7 @@ __global__ void __launch_bounds__(32 * WARPS, MINB) k_collide_d2q9(const __grid_
     mslot.fill(P);
     __syncthreads();
     const long long t = P.probe_ring ? __ldcg(P.step) : 0;   // (the probe's log only)
-    const S* __restrict__ src = static_cast<const S*>(P.src);
+    const S* src = static_cast<const S*>(P.src);
     S* __restrict__ dst = static_cast<S*>(P.dst);
     const int nxp = P.nxp, plane = (int)P.plane;
     bool nonfinite = false;
@@ -1629,7 +1633,7 @@ __device__ __noinline__ void patch_row(const Params& P, S* box, int x0, int y) {
     constexpr int C = TX / 32;   // sites per lane
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     S* sb = box + warp * LY::W + LY::H;
-    const S* __restrict__ src = static_cast<const S*>(P.src);
+    const S* src = static_cast<const S*>(P.src);
     const long long row = (long long)y * P.nxp;
     if (P.prestream) {
 #pragma unroll 1
