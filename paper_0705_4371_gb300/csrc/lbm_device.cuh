@@ -619,47 +619,60 @@ __device__ __noinline__ T delta_s_slow(PopArr<L::Q, T> g, PopArr<L::Q, T> gs, T 
 // operations) and a relative margin of 2^-16 on each side, far above the
 // roundings: a site is cleared only if the FP64 bound clears it too, and one
 // near the limit gets its exact dS as any other site that is not cleared.
+// The populations, f* and delta enter divided by the power of two of the
+// site's density (dS is linear in it), so that the bound holds at every
+// density FP64 represents.  Squares that FP32 loses (|d| below 2^-60 of the
+// density) are covered by a floor of Q, 2^-99 unless every d is zero; m is
+// kept above 2^-40, where m^2 and the floor are far from FP32's limits.
 
-// |x| as FP32, truncated to 20 significant bits (0 below 2^-126, infinity
-// from 2^128 on and for NaN), without an FP64 operation.
-__device__ __forceinline__ float abs_float(double x) {
+// |x| / 2^s as FP32, truncated to 20 significant bits (0 below 2^-126, infinity
+// from 2^128 on and for NaN), without an FP64 operation.  scale: (s + 896) << 20.
+constexpr int kNoScale = 896 << 20;
+__device__ __forceinline__ float abs_float(double x, int scale) {
     const int h = __double2hiint(x) & 0x7fffffff;
-    return __int_as_float(min(max(h - (896 << 20), 0), 0x0ff00000) << 3);
+    return __int_as_float(min(max(h - scale, 0), 0x0ff00000) << 3);
 }
 
 template <typename L, typename T, int EQ>
-__device__ __forceinline__ bool ds_cleared(const T* d, const T* gs, T rho, T ux, T uy, T rho0,
-                                           T delta, float deltaf) {
+__device__ __forceinline__ bool ds_cleared(const T* d, const T* gs, T rho, T ux, T uy, T rho0, T delta) {
     // the bound's arithmetic type
     constexpr bool narrow = kF64<T>;
     using B = float;
+    int scale = kNoScale;   // of the density (not below 2^-896: the difference in abs_float stays in range)
+    if constexpr (narrow) scale = max((__double2hiint(rho) & 0x7ff00000) - (127 << 20), 0);
     B q0 = B(0), q1 = B(0), q2 = B(0);
+    int any = 0;   // bits of the d
 #pragma unroll
     for (int i = 0; i < L::Q; i++) {
         B di;
-        if constexpr (narrow) di = abs_float(d[i]);
-        else di = d[i];
+        if constexpr (narrow) {
+            di = abs_float(d[i], scale);
+            any |= (__double2hiint(d[i]) & 0x7fffffff) | __double2loint(d[i]);
+        } else {
+            di = d[i];
+        }
         if (L::w(i) == L::w(0)) q0 = fmaf(di, di, q0);
         else if (L::w(i) == L::w(1)) q1 = fmaf(di, di, q1);
         else q2 = fmaf(di, di, q2);
     }
     constexpr double wmin = L::Q == 9 ? 1.0 / 36.0 : 1.0 / 6.0;
     B Q = fmaf(q0, B(1.0 / L::w(0)), fmaf(q1, B(1.0 / L::w(1)), L::Q == 9 ? q2 * B(1.0 / L::w(5)) : B(0)));
-    B m, dl;
+    B m;
     if constexpr (narrow) {
-        const B r = abs_float(rho), vx = abs_float(ux) * B(1.0 + 0x1p-18), vy = abs_float(uy) * B(1.0 + 0x1p-18);
         if constexpr (EQ == 0) {
-            m = r * fmaf(B(-1.5), fmaf(vx, vx, vy * vy), fmaf(B(-3), vx + vy, B(1)));
+            const B vx = abs_float(ux, kNoScale) * B(1.0 + 0x1p-18), vy = abs_float(uy, kNoScale) * B(1.0 + 0x1p-18);
+            m = abs_float(rho, scale) * fmaf(B(-1.5), fmaf(vx, vx, vy * vy), fmaf(B(-3), vx + vy, B(1)));
         } else {
             m = B(INFINITY);
 #pragma unroll
             for (int i = 0; i < L::Q; i++)
-                m = fminf(m, gs[i] > T(0) ? abs_float(gs[i]) * B(1.0 / L::w(i)) : B(-1));
+                m = fminf(m, gs[i] > T(0) ? abs_float(gs[i], scale) * B(1.0 / L::w(i)) : B(-1));
         }
-        Q *= B(1.0 + 0x1p-16);
+        Q = any ? fmaxf(Q * B(1.0 + 0x1p-16), B(0x1p-99)) : B(0);
         m *= B(1.0 - 0x1p-16);
-        dl = deltaf * (deltaf > B(0) ? B(1.0 - 0x1p-16) : B(1.0 + 0x1p-16));
-        return (rho > T(0)) & (m > B(0)) & (B(16.0 / wmin) * Q <= m * m) & (B(0.55) * Q <= dl * m);
+        const B ad = abs_float(delta, scale);
+        const B dl = delta > T(0) ? ad * B(1.0 - 0x1p-16) : ad * B(-1.0 - 0x1p-16);
+        return (rho > T(0)) & (m > B(0x1p-40)) & (B(16.0 / wmin) * Q <= m * m) & (B(0.55) * Q <= dl * m);
     } else {
         if constexpr (EQ == 0) {
             const B usq = fmaf(ux, ux, uy * uy);

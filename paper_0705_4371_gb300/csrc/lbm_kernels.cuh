@@ -423,7 +423,7 @@ __device__ __forceinline__ bool update_site(const Params& P, T* g, int x, int y,
     if constexpr (PROJ) conserve_neq<L, EQ>(d);
     // (no short-circuit: the site's update stays one branch-free block)
     const bool pending =
-        (P.k > 0) & !ds_cleared<L, T, EQ>(d, gs, rho, ux, uy, Par<T>::rho0(P), Par<T>::delta(P), P.deltaf);
+        (P.k > 0) & !ds_cleared<L, T, EQ>(d, gs, rho, ux, uy, Par<T>::rho0(P), Par<T>::delta(P));
     if constexpr (RESOLVE) {
         T ds = T(-1);
         if (pending && !ghost_column(P, x)) ds = site_ds<L, T, EQ>(P, g, gs);
