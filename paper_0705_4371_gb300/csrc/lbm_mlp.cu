@@ -209,6 +209,11 @@ __global__ void __launch_bounds__(128) k_mlp_forward(const float* __restrict__ p
 // batch of 4096 on 128 SMs, and the register tiles (2 x 4 of dz1, 4 x 4 of
 // dW2) take one shared-memory access per four multiply-adds.
 // ---------------------------------------------------------------------------
+// Groups of a batch of n > 0 samples (no sum that exceeds an int).
+__host__ __device__ constexpr int grad_groups(int n) { return (n - 1) / kGradRows + 1; }
+static_assert(grad_groups(1) == 1 && grad_groups(kGradRows) == 1 && grad_groups(kGradRows + 1) == 2 &&
+              grad_groups(0x7fffffff) == 1 << 26, "groups of the smallest and largest batches");
+
 struct __align__(16) GradSmem {
     float w2[kMlpHid][kMlpHid];        // BF16-rounded W2, W3 as floats
     float w3[kMlpOut][kMlpHid];
@@ -447,7 +452,7 @@ __global__ void __launch_bounds__(kGradThreads) k_mlp_grad(const float* __restri
     __syncthreads();
     GradAcc acc;
     grad_zero(acc);
-    for (int g = blockIdx.x; g < (n + kGradRows - 1) / kGradRows; g += gridDim.x)
+    for (int g = blockIdx.x; g < grad_groups(n); g += gridDim.x)
         grad_group(s, grad_load(feat, dmu, 0, n, g), n - g * kGradRows, inv_count, acc);
     grad_store(acc, partial + (size_t)blockIdx.x * kPartialLd);
 }
@@ -551,7 +556,7 @@ __global__ void __launch_bounds__(kGradThreads) k_mlp_train(const TrainArgs A) {
             __syncthreads();
             GradAcc acc;
             grad_zero(acc);
-            for (int g = blockIdx.x; g < (n + kGradRows - 1) / kGradRows; g += B) {
+            for (int g = blockIdx.x; g < grad_groups(n); g += B) {
                 const GradIn cur = in;
                 in = grad_load(A.feat, A.dmu, i0, n, g + B);   // the next group's (zeros beyond the batch)
                 grad_group(s, cur, n - g * kGradRows, inv, acc);
