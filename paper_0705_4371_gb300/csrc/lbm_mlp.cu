@@ -644,7 +644,8 @@ int grad_grid(long long n, int most) {
     return (int)std::max(1ll, std::min<long long>((n + kGradRows - 1) / kGradRows, most));
 }
 
-// Shared memory of the training kernel with G blocks, B of them with samples.
+// Shared memory of the training kernel with G blocks, B of them with samples
+// (at its largest where every block has some).
 size_t train_smem(int G, int B) {
     const int per = (kPartial + G - 1) / G;
     return sizeof(GradSmem) + (size_t)(3 + train_segs(B)) * per * sizeof(float);
@@ -783,7 +784,9 @@ int lb_mlp_train(float* params, const float* feat, const float* dmu, long long n
     // reduction (152 blocks: 32 entries each, one per lane)
     const int A_blocks = grad_grid(std::min<long long>(n, batch), sms), G = sms;
     const size_t smem = train_smem(G, A_blocks);
-    CK(cudaFuncSetAttribute(k_mlp_train, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    // the limit belongs to the kernel, which other threads launch too: always
+    // the largest size, so that no call lowers it under another's launch
+    CK(cudaFuncSetAttribute(k_mlp_train, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)train_smem(G, G)));
     CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_mlp_train, kGradThreads, smem));
     if (per_sm < 1) return fail(LB_ERR_CUDA, "the training kernel does not fit on this device");
     // working memory: block partials, Adam's moments, the chunk's step scales, the barrier

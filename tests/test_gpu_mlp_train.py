@@ -82,3 +82,44 @@ def test_normalise_matches_fp64_sums(env, n):
         assert np.allclose(got, want, rtol=1.5e-7)
     else:
         assert np.allclose(got[[0, 1, 2, 3, 8, 9, 10, 11]], want[[0, 1, 2, 3, 8, 9, 10, 11]], rtol=1.5e-7)
+
+
+def test_two_threads_train_at_once(env):
+    # batches of one and of many sample groups need different amounts of shared
+    # memory of one kernel; neither thread may disturb the other's launches
+    import threading
+    torch, lbm = env
+    n, calls = 256, 400
+    feat, dmu = _data(torch, 77, n)
+    p0 = torch.from_numpy(mlp_random_params(91).astype(np.float32)).cuda()
+
+    def train(batch):
+        p = p0.clone()
+        lbm.mlp_train(p.data_ptr(), feat.data_ptr(), dmu.data_ptr(), n, batch, 1, 1e-3, 1e-3, None, st[batch].cuda_stream)
+        return p
+
+    st = {b: torch.cuda.Stream() for b in (32, 256)}
+    torch.cuda.synchronize()
+    want = {}
+    for b in st:
+        with torch.cuda.stream(st[b]):
+            want[b] = train(b)
+    torch.cuda.synchronize()
+    failed = []
+
+    def work(batch):
+        try:
+            with torch.cuda.stream(st[batch]):
+                for _ in range(calls):
+                    p = train(batch)
+                st[batch].synchronize()
+                assert torch.equal(p, want[batch])
+        except Exception as e:
+            failed.append((batch, e))
+
+    threads = [threading.Thread(target=work, args=(b,)) for b in st]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failed, failed
