@@ -326,9 +326,23 @@ int lb_mlp_adam(float* params, const float* grad, float* m, float* v, long long 
  * one shorter), `epochs` passes; the learning rate decays geometrically
  * from lr0 at the first step to lr1 at the last.  params (device) in and
  * out; loss_log (device, optional): mean batch loss of each epoch.
- * Asynchronous; allocates its working memory on the stream. */
+ * Asynchronous; allocates its working memory on the stream.  The steps run
+ * in one kernel whose blocks wait for one another between them; a wait that
+ * gives up (seconds; not expected, as every block is resident) ends the
+ * training, and the parameters, its normalisation entries included, are then
+ * NaN: lb_mlp_train_status reports it. */
 int lb_mlp_train(float* params, const float* feat, const float* dmu, long long n, int batch, int epochs,
                  double lr0, double lr1, float* loss_log, void* cuda_stream);
+
+/* Whether the trainings into params (device) queued on the stream so far ran
+ * to their end: LB_OK, or LB_ERR_TIMEOUT where a wait gave up.  Synchronises
+ * the stream. */
+int lb_mlp_train_status(const float* params, void* cuda_stream);
+
+/* lb_mlp_train with the bound of its waits given, in polls (lb_mlp_train:
+ * 2^24); 0 gives up at the first one.  For tests of that path. */
+int lb_mlp_train_bounded(float* params, const float* feat, const float* dmu, long long n, int batch, int epochs,
+                         double lr0, double lr1, float* loss_log, int polls, void* cuda_stream);
 
 /* Newton statistics of the energy forms since the last reset: total
  * FP32 iterations, finishing iterations (float-float for FP32 / FP16

@@ -502,19 +502,26 @@ struct TrainArgs {
     float *partial, *m, *v;     // [sum_blocks][kPartialLd], Adam moments [kMlpParams]
     int sum_blocks;             // blocks with samples (every block reduces)
     float* loss_log;            // mean batch loss of each epoch (may be null)
-    unsigned long long* barrier;   // arrivals (zero at launch)
+    // arrivals (zero at launch), and a word that is not zero once a barrier
+    // gave up, in this launch or an earlier one of the call
+    unsigned long long* barrier;
+    int polls;                  // most polls of a barrier
 };
 
 // Grid barrier of a cooperative launch (every block is resident): arrival
 // count target reached, or false when the bounded wait gave up.
-constexpr long long kBarrierPolls = 1ll << 24;
-__device__ __forceinline__ bool train_barrier(unsigned long long* count, unsigned long long target, int& ok) {
+constexpr int kBarrierPolls = 1 << 24;
+// What a call whose barrier gave up leaves in the normalisation entries, which
+// training never writes otherwise (a NaN of this one payload).
+constexpr unsigned kGaveUpBits = 0x7fc7e57au;
+__device__ __forceinline__ bool train_barrier(unsigned long long* count, unsigned long long target, int polls,
+                                              int& ok) {
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
         atomicAdd(count, 1ull);
         int done = 0;
-        for (long long it = 0; it < kBarrierPolls && !done; it++) {
+        for (int it = polls; it > 0 && !done; it--) {
             unsigned long long c;
             asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(c) : "l"(count) : "memory");
             done = c >= target;
@@ -528,6 +535,17 @@ __device__ __forceinline__ bool train_barrier(unsigned long long* count, unsigne
 // Partial sums per entry in the reduction over G blocks: one per warp.
 __host__ __device__ constexpr int train_segs(int G) { return G < kGradThreads / 32 ? G : kGradThreads / 32; }
 
+// A barrier gave up (never expected of a cooperative launch): the block's
+// entries e0 .. e0 + ne - 1 are not a result, and the parameters say so
+// (lb_mlp_train_status).
+__device__ __forceinline__ void train_give_up(const TrainArgs& A, int e0, int ne) {
+    const int tid = threadIdx.x;
+    if (tid == 0) atomicExch(A.barrier + 1, 1ull);
+    for (int e = tid; e < ne; e += kGradThreads)
+        if (e0 + e < kMlpTrainable) A.p[e0 + e] = nanf("");
+    if (tid < kMlpParams - kMlpMean) A.p[kMlpMean + tid] = __uint_as_float(kGaveUpBits);
+}
+
 __global__ void __launch_bounds__(kGradThreads) k_mlp_train(const TrainArgs A) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     GradSmem& s = *reinterpret_cast<GradSmem*>(smem_raw);
@@ -538,6 +556,13 @@ __global__ void __launch_bounds__(kGradThreads) k_mlp_train(const TrainArgs A) {
     float *own_p = own, *own_m = own + per, *own_v = own + 2 * per, *red = own + 3 * per;   // red[segs][per]
     const int segs = train_segs(B);
     __shared__ int ok;
+    // an earlier launch of the call gave up: nothing to go on from (a block that
+    // finds the word set during this launch takes no part; the others' waits are
+    // bounded)
+    if (__ldcg(A.barrier + 1) != 0ull) {
+        train_give_up(A, e0, ne);
+        return;
+    }
     for (int e = tid; e < ne; e += kGradThreads) {
         const bool w = e0 + e < kMlpTrainable;
         own_p[e] = w ? A.p[e0 + e] : 0.0f;
@@ -566,7 +591,7 @@ __global__ void __launch_bounds__(kGradThreads) k_mlp_train(const TrainArgs A) {
         const long long bn = b + 1 == A.nb ? 0 : b + 1;
         const StepScale sc = A.scale[t];
         in = grad_load(A.feat, A.dmu, bn * A.batch, (int)min((long long)A.batch, A.n - bn * A.batch), blockIdx.x);
-        if (!train_barrier(A.barrier, arrived += G, ok)) break;
+        if (!train_barrier(A.barrier, arrived += G, A.polls, ok)) break;
         // warp w adds the partials of blocks w, w + segs, ...
         const int seg = tid >> 5;
         if (seg < segs)
@@ -594,13 +619,10 @@ __global__ void __launch_bounds__(kGradThreads) k_mlp_train(const TrainArgs A) {
         }
         ep += bn == 0;
         b = bn;
-        if (!train_barrier(A.barrier, arrived += G, ok)) break;
+        if (!train_barrier(A.barrier, arrived += G, A.polls, ok)) break;
     }
     if (!ok) {
-        // a barrier gave up (never expected of a cooperative launch): the
-        // parameters are not a result
-        for (int e = tid; e < ne; e += kGradThreads)
-            if (e0 + e < kMlpTrainable) A.p[e0 + e] = nanf("");
+        train_give_up(A, e0, ne);
         return;
     }
     for (int e = tid; e < ne; e += kGradThreads)
@@ -768,6 +790,22 @@ int lb_mlp_adam(float* params, const float* grad, float* m, float* v, long long 
 
 int lb_mlp_train(float* params, const float* feat, const float* dmu, long long n, int batch, int epochs,
                  double lr0, double lr1, float* loss_log, void* cuda_stream) {
+    return lb_mlp_train_bounded(params, feat, dmu, n, batch, epochs, lr0, lr1, loss_log, kBarrierPolls, cuda_stream);
+}
+
+int lb_mlp_train_status(const float* params, void* cuda_stream) {
+    if (!params) return fail(LB_ERR_ARG, "params is NULL");
+    cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+    unsigned bits = 0;
+    CK(cudaMemcpyAsync(&bits, params + kMlpMean, sizeof(bits), cudaMemcpyDeviceToHost, st));
+    CK(cudaStreamSynchronize(st));
+    if (bits == kGaveUpBits) return fail(LB_ERR_TIMEOUT, "a grid barrier of the training kernel gave up");
+    return LB_OK;
+}
+
+int lb_mlp_train_bounded(float* params, const float* feat, const float* dmu, long long n, int batch, int epochs,
+                         double lr0, double lr1, float* loss_log, int polls, void* cuda_stream) {
+    if (polls < 0) return fail(LB_ERR_ARG, "polls must be >= 0");
     if (!params || !feat || !dmu) return fail(LB_ERR_ARG, "NULL argument");
     if (n <= 0 || batch <= 0 || epochs < 0) return fail(LB_ERR_ARG, "n, batch must be > 0, epochs >= 0");
     if (batch > (1 << 24)) return fail(LB_ERR_ARG, "batch too large");
@@ -790,6 +828,7 @@ int lb_mlp_train(float* params, const float* feat, const float* dmu, long long n
     CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_mlp_train, kGradThreads, smem));
     if (per_sm < 1) return fail(LB_ERR_CUDA, "the training kernel does not fit on this device");
     // working memory: block partials, Adam's moments, the chunk's step scales, the barrier
+    // and the word that says that one gave up
     constexpr long long kChunk = 1 << 16;   // steps per launch
     const size_t scale_b = (size_t)std::min(std::max(total, 1ll), kChunk) * sizeof(StepScale);
     const size_t mv_b = 2 * (size_t)kMlpParams * sizeof(float);
@@ -801,7 +840,7 @@ int lb_mlp_train(float* params, const float* feat, const float* dmu, long long n
     if (e == cudaSuccess && loss_log) e = cudaMemsetAsync(loss_log, 0, (size_t)epochs * sizeof(float), st);
     TrainArgs A = {params, feat, dmu, n, nb, batch, 0, 0, reinterpret_cast<StepScale*>(mem),
                    reinterpret_cast<float*>(mem + scale_b + mv_b + 16), m, m + kMlpParams, A_blocks, loss_log,
-                   reinterpret_cast<unsigned long long*>(mem + scale_b + mv_b)};
+                   reinterpret_cast<unsigned long long*>(mem + scale_b + mv_b), polls};
     for (long long t = 0; t < total && e == cudaSuccess; t += kChunk) {
         A.t0 = t;
         A.steps = (int)std::min(kChunk, total - t);

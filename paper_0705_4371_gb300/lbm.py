@@ -105,6 +105,8 @@ def load(path=None):
         "lb_mlp_grad": ([vp, vp, vp, ip, vp, vp, vp], ip),
         "lb_mlp_adam": ([vp, vp, vp, vp, C.c_longlong, dp, vp], ip),
         "lb_mlp_train": ([vp, vp, vp, C.c_longlong, ip, ip, dp, dp, vp, vp], ip),
+        "lb_mlp_train_status": ([vp, vp], ip),
+        "lb_mlp_train_bounded": ([vp, vp, vp, C.c_longlong, ip, ip, dp, dp, vp, ip, vp], ip),
         "lb_set_slab": ([H, ip, ip, ip, ip], ip),
         "lb_slab_collide": ([H], ip),
         "lb_slab_candidates": ([H, vp, vp, ip, C.POINTER(ip)], ip),
@@ -228,6 +230,17 @@ def mlp_train(params, feat, dmu, n, batch, epochs, lr0, lr1, loss_log=None, stre
     """lb_mlp_train: epochs of mini-batch Adam with a geometric learning-rate decay."""
     _check(load().lb_mlp_train(_vp(params), _vp(feat), _vp(dmu), int(n), int(batch), int(epochs),
                                float(lr0), float(lr1), _vp(loss_log), _vp(stream)))
+
+
+def mlp_train_status(params, stream=None):
+    """lb_mlp_train_status: raises where a training into params (on the stream) gave up; synchronises."""
+    _check(load().lb_mlp_train_status(_vp(params), _vp(stream)))
+
+
+def mlp_train_bounded(params, feat, dmu, n, batch, epochs, lr0, lr1, polls, loss_log=None, stream=None):
+    """lb_mlp_train_bounded: lb_mlp_train with the bound of its waits given (tests)."""
+    _check(load().lb_mlp_train_bounded(_vp(params), _vp(feat), _vp(dmu), int(n), int(batch), int(epochs),
+                                       float(lr0), float(lr1), _vp(loss_log), int(polls), _vp(stream)))
 
 
 class Lattice:

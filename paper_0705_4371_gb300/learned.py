@@ -60,6 +60,7 @@ def train_energy_mlp(n=1_000_000, seed=inputs.SEED_ENERGY_SAMPLES, init_seed=1, 
     losses = torch.zeros(max(1, epochs), dtype=torch.float32, device=dev)
     lbm.mlp_train(p.data_ptr(), data["feat"].data_ptr(), data["dmu"].data_ptr(), n, batch, epochs,
                   lr0, lr1, losses.data_ptr(), st)
+    lbm.mlp_train_status(p.data_ptr(), st)
     torch.cuda.synchronize(dev)
     t2 = time.perf_counter()
     info = dict(losses=losses.cpu().numpy()[:epochs].tolist(), dataset_stats=data["stats"],

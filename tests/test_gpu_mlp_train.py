@@ -123,3 +123,28 @@ def test_two_threads_train_at_once(env):
     for t in threads:
         t.join()
     assert not failed, failed
+
+
+def test_a_wait_that_gives_up_is_reported(env):
+    # no polls: the first grid barrier gives up in every block, without a wait;
+    # the later launches of the call (more than 65 536 steps) end at once
+    torch, lbm = env
+    feat, dmu = _data(torch, 31, 96)
+    p0 = torch.from_numpy(mlp_random_params(91).astype(np.float32)).cuda()
+    st = torch.cuda.current_stream().cuda_stream
+    for epochs in (1, 30_000):
+        p = p0.clone()
+        lbm.mlp_train_bounded(p.data_ptr(), feat.data_ptr(), dmu.data_ptr(), 96, 32, epochs, 1e-3, 1e-3, 0, stream=st)
+        with pytest.raises(lbm.LBError) as e:
+            lbm.mlp_train_status(p.data_ptr(), st)
+        assert e.value.code == lbm.LB_ERR_TIMEOUT
+        assert torch.isnan(p[-12:]).all()
+    # the context, the kernel and the same buffer go on as before
+    a, b = p0.clone(), p
+    b.copy_(p0)
+    for q in (a, b):
+        lbm.mlp_train(q.data_ptr(), feat.data_ptr(), dmu.data_ptr(), 96, 32, 2, 1e-3, 1e-3, None, st)
+        lbm.mlp_train_status(q.data_ptr(), st)
+    assert torch.isfinite(a).all() and torch.equal(a, b)
+    with pytest.raises(lbm.LBError):
+        lbm.mlp_train_bounded(a.data_ptr(), feat.data_ptr(), dmu.data_ptr(), 96, 32, 1, 1e-3, 1e-3, -1)
