@@ -148,3 +148,37 @@ def test_a_wait_that_gives_up_is_reported(env):
     assert torch.isfinite(a).all() and torch.equal(a, b)
     with pytest.raises(lbm.LBError):
         lbm.mlp_train_bounded(a.data_ptr(), feat.data_ptr(), dmu.data_ptr(), 96, 32, 1, 1e-3, 1e-3, -1)
+
+
+def test_more_steps_than_a_launch(env):
+    # launches of 65 536 steps: the next one goes on from the moments, the step
+    # count and the epoch of the one before.  The tolerance of the test above
+    # (1e-3 lr a step in the root mean square) and its losses
+    torch, lbm = env
+    n, batch, epochs, lr = 64, 32, 33_500, 1e-6
+    feat, dmu = _data(torch, 41, n)
+    p0 = torch.from_numpy(mlp_random_params(91).astype(np.float32)).cuda()
+    a = p0.clone()
+    losses = torch.zeros(epochs, dtype=torch.float32, device="cuda")
+    lbm.mlp_train(a.data_ptr(), feat.data_ptr(), dmu.data_ptr(), n, batch, epochs, lr, lr, losses.data_ptr())
+    b, g = p0.clone(), torch.zeros_like(p0)
+    m, v = torch.zeros_like(p0), torch.zeros_like(p0)
+    loss = torch.zeros(2, dtype=torch.float32, device="cuda")
+    last = []
+    for t in range(2 * epochs):
+        i0 = batch * (t % 2)
+        lbm.mlp_grad(b.data_ptr(), feat[i0:].data_ptr(), dmu[i0:].data_ptr(), batch, g.data_ptr(),
+                     loss[t % 2:].data_ptr())
+        lbm.mlp_adam(b.data_ptr(), g.data_ptr(), m.data_ptr(), v.data_ptr(), t + 1, lr)
+        if t % 2 and t > 2 * epochs - 20:
+            last.append(float(loss.mean()))
+    torch.cuda.synchronize()
+    moved = (b - p0).double().square().mean().sqrt()
+    assert float((a - b).double().square().mean().sqrt()) <= 1e-3 * lr * 2 * epochs
+    assert float(moved) > 1e-2 * lr * 2 * epochs       # (the bound is well below what the steps do)
+    assert np.allclose(losses.cpu().numpy()[-len(last):], last, rtol=1e-4)
+    # what the first launch alone gives is another result
+    c = p0.clone()
+    lbm.mlp_train(c.data_ptr(), feat.data_ptr(), dmu.data_ptr(), n, batch, 32_768, lr, lr, None)
+    lbm.mlp_train_status(c.data_ptr())
+    assert torch.isfinite(c).all() and not torch.equal(a, c)

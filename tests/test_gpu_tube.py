@@ -67,3 +67,29 @@ def test_elbm_tube_equals_single_steps(lbm):
     b = _run(lbm, w, "f64", f0, (40,), True, lbm.LB_COLLISION_ELBM)
     for u, v in zip(a, b):
         assert np.array_equal(u, v)
+
+
+def test_more_steps_than_a_launch_and_than_the_logs_hold(lbm):
+    # launches of 4096 steps, and logs that wrap after 65 536: the tail of the
+    # run in single steps gives the same state, counts and probe series
+    w = inputs.shock_tube(100, 1.0 / 30.0, 1e-9, 3, 10)
+    cfg = oracle_cfg(w)
+    f0 = ora.init_field(cfg, *inputs.shock_tube_fields(w)) * (1 + 1e-3 * inputs.uniform(5, (3, 1, 100)))
+    total, single, log = 66_001, 700, 65_536
+
+    def run(parts):
+        with lbm.Lattice.from_workload(w, precision=lbm.LB_F64) as g:
+            g.set_probe(17, 0)
+            g.set_state(f0)
+            for n, timed in parts:
+                g.set_timing(timed)
+                g.step(n)
+            g.sync()
+            return g.get_state(), g.counts(log), g.probe(log), g.selected()
+
+    want = run([(total - single, False), (single, True)])
+    for parts in ([(total, False)], [(5000, False), (1, False), (total - 5001, False)]):
+        for u, v in zip(run(parts), want):
+            assert np.array_equal(u, v)
+    for u, v in zip(_run(lbm, w, "f64", f0, (4097,), False), _run(lbm, w, "f64", f0, (4097,), True)):
+        assert np.array_equal(u, v)
