@@ -351,13 +351,15 @@ int lb_mlp_train_bounded(float* params, const float* feat, const float* dmu, lon
 int lb_newton_stats(lb_handle* h, long long* it32, long long* it64, long long* sites,
                     long long* fails, int reset);
 
-/* Kernel timing for measurement: when enabled, every launch of lb_step (one
- * per time step: stream-collide with the selection and the Ehrenfests' step
- * fused into its last block) is bracketed by CUDA events on the run's
- * stream (graphs are not used).  lb_kernel_times returns the summed
- * milliseconds and launch counts since the last reset (synchronises); the
- * select figures count stand-alone select launches, which lb_step no
- * longer makes. */
+/* Kernel timing for measurement: when enabled, lb_step makes one launch per
+ * time step (stream-collide with the selection and the Ehrenfests' step fused
+ * into its last block), each bracketed by CUDA events on the run's stream.
+ * Without it the steps are replayed as graphs, and a D1Q3 run of up to 4096
+ * sites takes up to 4096 steps per launch of another kernel, several times
+ * faster per step: time such a run from outside.  lb_kernel_times returns the
+ * summed milliseconds and launch counts since the last reset (synchronises);
+ * the select figures count stand-alone select launches, which lb_step does
+ * not make. */
 int lb_set_timing(lb_handle* h, int enable);
 int lb_kernel_times(lb_handle* h, double* collide_ms, long long* collide_launches,
                     double* select_ms, long long* select_launches, int reset);
@@ -438,7 +440,8 @@ int lb_slab_ghost(lb_handle* h, int side, void* buf, int direction);
 /* Run facts (out: 8 entries): out[0] = Q, out[1] = padded row length
  * (elements), out[2] = bytes per stored population, out[3] = algorithmic
  * bytes per site update (read Q + write Q populations), out[4] = launches
- * per step (1), out[5] = blocks of the persistent stream-collide grid,
+ * per step (1; a D1Q3 run of up to 4096 sites takes many steps per launch, see
+ * lb_set_timing), out[5] = blocks of the persistent stream-collide grid,
  * out[6] = its resident blocks per SM, out[7] = tile shape.
  * beta_out (nullable) receives beta. */
 int lb_info(lb_handle* h, long long* out, double* beta_out);

@@ -47,23 +47,26 @@ constexpr int kTubeSteps = 4096;     // steps of a short D1Q3 run per launch
 constexpr int kExportChunks = 8;     // row chunks of a host export (copies overlap the conversion)
 constexpr int kXferEvents = 16;      // events of one chunked transfer (>= Q planes, >= chunks, + 1)
 constexpr int kDefaultLog = 65536;
-// Default tile shapes by measurement on GB300 (us per step of two runs side by
-// side).  Up to 600 000 sites (one or two tiles per resident block, a step
-// dominated by latency): register-fed tiles for polynomial-f* FP32 (shape 1),
-// 6-row staged tiles for the others (shape 5; entropic FP16 600 x 500: 7.9
-// against 8.5 on shape 4).  Above, the 8-row tiles' warps win (shape 4) from
-// 1e6 sites on (FP16 and polynomial-f* FP32) or at once: polynomial FP32
-// 1280 x 800: 14.8 against 16.8 on shape 5, 2560 x 1280: 37.1 against 41.3;
-// entropic FP32 4096 x 2048: 94 against 100; entropic FP16 2048 x 1024: 24.7
-// against 26.7; 2048 x 1024 ELBM: 52 against 57.  The largest polynomial-f*
-// FP32 grids, bound by memory, take the 6-row tiles again, whose three copies
-// in flight are as fast within 2 % (3500 x 1750: 69.1 against 68.1).  FP64
-// storage: 8-row tiles.  The energy forms: FP64 storage's
-// solve wants the most resident warps (register-fed shape 1); the
-// float-float solve of FP32 / FP16 storage and the network's warm start run
-// best in the staged shape 4 (measured at 2048 x 1024: Newton start 89 us
-// per step against 235 on shape 0 and 93 on shape 5; warm start 131 against
-// 209 on shape 5).
+// Default tile shapes (figures: GB300, us per step of two runs side by side).
+// 8-row staged tiles (shape 4) are the fastest measured almost everywhere:
+// entropic FP32 4096 x 2048: 94 against 100 on the 6-row tiles of shape 5,
+// 1531 x 765: 18.9 against 20.4; FP16 from 1e6 sites on (entropic 2048 x 1024:
+// 24.7 against 26.7); 2048 x 1024 ELBM: 52 against 57, FP64: 285 against 295.
+// Smaller FP16 grids, and entropic grids of up to 600 000 sites, take shape 5
+// (entropic FP16 600 x 500: 7.9 against 8.5).
+// Polynomial-f* FP32 takes shape 4 between 1e6 and 5e6 sites (1280 x 800: 13.3
+// against 14.7 on shape 5, 3072 x 1536: 51.8 against 53.3).  Outside that band
+// it keeps the defaults that callers and tests know from before shape 4 became
+// the faster one there too: register-fed tiles (shape 1) up to 600 000 sites
+// (600 x 500: 7.8 against 6.5 on shape 4, one run alone 12.6 against 11.6; 1000 x
+// 500: 10.9 against 7.6), shape 5 up to 1e6 (1200 x 600: 11.8 against 10.3) and
+// above 5e6 (4096 x 2048: 90.6 against 89.2).  lb_set_tile_shape takes the
+// faster one; the results are the same bits.
+// The energy forms: FP64 storage's solve wants the most resident warps
+// (register-fed shape 1); the float-float solve of FP32 / FP16 storage and the
+// network's warm start run best in shape 4 (2048 x 1024, one run alone: Newton
+// start 58.4 against 61.3 on shape 5 and 73.2 on shape 1, warm start 121 against
+// 188 and 142).
 int default_tile_shape(int lattice, int eq, int precision, long long sites, bool elbm) {
     if (lattice != LB_D2Q9) return 0;
     if (eq < LB_EQ_ENTROPIC_ENERGY) {

@@ -1374,10 +1374,9 @@ constexpr size_t tma_smem_bytes() {
 // Where a staged tile's candidates go (put: every lane of the warp calls,
 // with its site's dS, -1 for a site the dS bound cleared; the sites the
 // bound does not clear have their exact dS evaluated on the tile, from the
-// staged planes or in the update).  CandSink: the block's buffer; count is
-// what the warp appended since the block's last cut (the same on every
-// lane).  GlobalCandSink: the run's global list (a kernel whose tiles belong
-// to different runs).
+// staged planes or in the update).  CandSink: the block's buffer.
+// GlobalCandSink: the run's global list (a kernel whose tiles belong to
+// different runs).
 template <int CAP>
 struct CandSink {
     BlockCandT<CAP>* bc;
@@ -1408,7 +1407,7 @@ struct TileState {
 // row = sy - y0 + v_jy, col = sx - x0 + H); a rule that reads a plane
 // outside its window (a bounce-back or a mirror at the tile's edge rows, the
 // outlet column) reads the source field instead.  Not used with periodic
-// sides.
+// sides, nor for the first step after a state upload.
 template <typename S, int R, int TX = kTmaTX>
 __device__ __forceinline__ void gather_site_smem(const Params& P, const S* box, int x0, int y0, int x,
                                                  int y, typename Store<S>::T* g) {
@@ -1421,11 +1420,6 @@ __device__ __forceinline__ void gather_site_smem(const Params& P, const S* box, 
             return Store<S>::load(box + j * LY::PLANE + r * LY::W + c, 0);
         return Store<S>::load(P.src, j * P.plane + (long long)sy * P.nxp + sx);
     };
-    if (P.prestream) {
-#pragma unroll
-        for (int i = 0; i < L::Q; i++) g[i] = at(i, x, y);
-        return;
-    }
     bool have_out = false;
     unsigned wall_mask = 0u;
     T gout[L::Q];
@@ -1501,8 +1495,7 @@ __device__ __noinline__ TileState<Sink> tma_tile_general(const Params& P, const 
             const int o = y * nxp + x;
             const bool near_obstacle = P.ow > 0 && x >= P.ox0 - 1 && x <= P.ox0 + P.ow &&
                                        y >= P.oy0 - 1 && y <= P.oy0 + P.oh;
-            const bool shift = !P.prestream && x >= 1 && x <= P.nx - 2 && y >= 1 && y <= P.ny - 2 &&
-                               !near_obstacle;
+            const bool shift = x >= 1 && x <= P.nx - 2 && y >= 1 && y <= P.ny - 2 && !near_obstacle;
             T g[L::Q];
             bool fluid = inside;
             if (!inside) {
@@ -1765,8 +1758,8 @@ __device__ __forceinline__ void tma_tile(const Params& P, S* box, int x0, int y0
     const bool masked = x0 == 0 || x0 + TX >= P.nx || solid_row;   // uniform: some sites are not the row's
     // two adjacent sites per lane, columns c and c + 1 (c = 2 l + 64 s):
     // planes at rest and every store move both with one access, and the
-    // two updates are one packed update, or (FP64, the energy forms)
-    // independent work for the scheduler
+    // two updates are one packed update, or (FP64) independent work for the
+    // scheduler
 #pragma unroll 1
     for (int s = 0; s < TX / 64; s++) {
         const int c = 2 * lane + 64 * s;
@@ -2113,7 +2106,7 @@ __global__ void __launch_bounds__(kSiteBlock) k_collide_site(const __grid_consta
 // needs a second one before the next free flight.  The exact dS of a warp's
 // pending sites takes a lane per population (its series are the longest FP64
 // chain of a step).
-// 800 sites, FP64: 23.5 us per step in one launch each (4 blocks), 5.7 us so
+// 800 sites, FP64: 19.5 us per step in one launch each (13 blocks), 5.8 us so
 // (2.5 us without the selection).
 // Every population passes through the storage type, so results are those of
 // one launch per step.
