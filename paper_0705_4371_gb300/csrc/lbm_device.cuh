@@ -430,17 +430,20 @@ template <> __host__ __device__ __forceinline__ f2 recip<f2>(f2 x) {
 }
 
 // sqrt(x), x > 0: FP32 correctly rounded; FP64 from the hardware's
-// approximation r of 1 / sqrt(x): s = x r, with e = 1 - s r:
-// s + s e (1/2 + 3/8 e), whose error ~ 5/16 e^3 is below 2^-57 -- five FP64
-// operations.
+// approximation r of 1 / sqrt(x): with s = x r and the residual d = x - s^2,
+// sqrt(x) = s sqrt(1 + d / s^2) = s + d r (1/2 + 3/8 e) up to e^3, e = 1 - s r
+// (below 2^-57) -- six FP64 operations.  The residual takes in the rounding of
+// s: the result is within 0.52 ulp (s + s e (1/2 + 3/8 e), one operation less,
+// is off by 0.76, more than a square root's 0.5, and the f* of it were further
+// from extended precision than the printed formula's).
 template <typename T> __host__ __device__ __forceinline__ T dsqrt(T x);
 template <> __host__ __device__ __forceinline__ float dsqrt<float>(float x) { return sqrtf(x); }
 template <> __host__ __device__ __forceinline__ double dsqrt<double>(double x) {
 #ifdef __CUDA_ARCH__
     double r;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-    const double s = x * r, e = fma(-s, r, 1.0);
-    return fma(s * e, fma(0.375, e, 0.5), s);
+    const double s = x * r, e = fma(-s, r, 1.0), d = fma(-s, s, x);
+    return fma(d * r, fma(0.375, e, 0.5), s);
 #else
     return sqrt(x);
 #endif
