@@ -429,27 +429,33 @@ template <> __host__ __device__ __forceinline__ f2 recip<f2>(f2 x) {
     return f2(recip<float>(x.x), recip<float>(x.y));
 }
 
-// sqrt(x), x > 0: FP32 correctly rounded; FP64 from the hardware's
-// approximation r of 1 / sqrt(x): with s = x r and the residual d = x - s^2,
-// sqrt(x) = s sqrt(1 + d / s^2) = s + d r (1/2 + 3/8 e) up to e^3, e = 1 - s r
-// (below 2^-57) -- six FP64 operations.  The residual takes in the rounding of
-// s: the result is within 0.52 ulp (s + s e (1/2 + 3/8 e), one operation less,
-// is off by 0.76, more than a square root's 0.5, and the f* of it were further
-// from extended precision than the printed formula's).
-template <typename T> __host__ __device__ __forceinline__ T dsqrt(T x);
-template <> __host__ __device__ __forceinline__ float dsqrt<float>(float x) { return sqrtf(x); }
-template <> __host__ __device__ __forceinline__ double dsqrt<double>(double x) {
+// sigma = sqrt(1 + q) - 1, q >= 0, to the rounding of sigma itself (a square
+// root rounded near 1 leaves an error that is the same at every site of a quiet
+// region, and it adds up).  FP32: q / (1 + sqrt(1 + q)).  FP64: from the
+// hardware's approximation r of 1 / sqrt(x), x = 1 + q: with s = x r,
+// e = 1 - s r and the residual d = q - (s - 1) (s + 1),
+// sigma = s - 1 + d r (1/2 + 3/8 e) up to e^3 (below 2^-57) -- nine FP64
+// operations.  Against extended precision the f* of it are 42 % (D1Q3) and 33 %
+// (D2Q9) closer than the printed formula in correctly rounded FP64.
+template <typename T> __host__ __device__ __forceinline__ T root_excess(T q);
+template <> __host__ __device__ __forceinline__ float root_excess<float>(float q) {
+    return q * recip<float>(1.0f + sqrtf(1.0f + q));
+}
+template <> __host__ __device__ __forceinline__ double root_excess<double>(double q) {
 #ifdef __CUDA_ARCH__
+    const double x = 1.0 + q;
     double r;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-    const double s = x * r, e = fma(-s, r, 1.0), d = fma(-s, s, x);
-    return fma(d * r, fma(0.375, e, 0.5), s);
+    const double s = x * r, e = fma(-s, r, 1.0), s0 = s - 1.0, d = fma(-s0, s + 1.0, q);
+    return fma(d * r, fma(0.375, e, 0.5), s0);
 #else
-    return sqrt(x);
+    return q / (1.0 + sqrt(1.0 + q));
 #endif
 }
-
-template <> __host__ __device__ __forceinline__ f2 dsqrt<f2>(f2 x) { return f2(sqrtf(x.x), sqrtf(x.y)); }
+template <> __host__ __device__ __forceinline__ f2 root_excess<f2>(f2 q) {
+    const f2 x = f2(1.0f) + q;
+    return q * recip<f2>(f2(1.0f) + f2(sqrtf(x.x), sqrtf(x.y)));
+}
 
 // Entropic for mass and momentum, by axis.  Sec. 4.1's closed form (with the
 // left/right labels read so that the momentum is +rho u) is rho times
@@ -464,11 +470,7 @@ template <> __host__ __device__ __forceinline__ f2 dsqrt<f2>(f2 x) { return f2(s
 template <typename T>
 __host__ __device__ __forceinline__ void entropic_axis(T u, T* A) {
     const T u3 = T(3) * u;
-    const T q = u3 * u;
-    const T s = dsqrt<T>(T(1) + q);
-    T sigma;
-    if constexpr (kF64<T>) sigma = s - T(1);
-    else sigma = q * recip<T>(T(1) + s);
+    const T sigma = root_excess<T>(u3 * u);
     A[0] = -sigma;
     const T two = sigma + sigma;
     A[1] = two + u3;
@@ -482,9 +484,9 @@ __host__ __device__ __forceinline__ void feq_entropic(T drho, T rho, T ux, T uy,
         // correction): a rounded weight's error would be the same at every
         // site and step, a drift of the mass (5e-14 after 500 steps)
         const T c = T(1.0 / 6.0), q = rho * c, r6 = dfma<T>(dfma<T>(T(-6), q, rho), c, q);
-        const T s = dsqrt<T>(dfma<T>(T(3) * ux, ux, T(1)));
-        const T a = dfma<T>(T(2), s, T(-1)), u3 = T(3) * ux;
-        gs[0] = T(4) * r6 * (T(2) - s);
+        const T u3 = T(3) * ux, sigma = root_excess<T>(u3 * ux);
+        const T a = dfma<T>(T(2), sigma, T(1));   // 2 s - 1
+        gs[0] = T(4) * r6 * (T(1) - sigma);
         gs[1] = r6 * (a - u3);
         gs[2] = r6 * (a + u3);
         if constexpr (!ZERO0)
