@@ -2106,7 +2106,7 @@ __global__ void __launch_bounds__(kSiteBlock) k_collide_site(const __grid_consta
 // needs a second one before the next free flight.  The exact dS of a warp's
 // pending sites takes a lane per population (its series are the longest FP64
 // chain of a step).
-// 800 sites, FP64: 19.5 us per step in one launch each (13 blocks), 5.8 us so
+// 800 sites, FP64: 19.5 us per step in one launch each (13 blocks), 6.1 us so
 // (2.5 us without the selection).
 // Every population passes through the storage type, so results are those of
 // one launch per step.
